@@ -425,31 +425,34 @@ static int coop_capacity(int which = 0) {
     if (which == 0)
       LMA_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, f64::k_f64_coop, f64::NTH, 0));
     else
-      LMA_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, f64::k_f64_flow, f64::NTH, 0));
+      LMA_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, f64::k_f64_flow, f64::FTH, 0));
     LMA_CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     cap[dev][which] = std::max(1, nb * sms);
   }
   return cap[dev][which];
 }
 
-// Tiles of the dataflow form, column by column (see k_f64_flow).
+// Tiles of the dataflow form's bulk, column by column (see k_f64_flow): the matrix
+// tiles within two of the diagonal are the chain's and the band's.
 static std::vector<int2> flow_tiles(int npan, int nrt, int nid) {
   std::vector<int2> t;
   for (int j = 0; j < npan; ++j)
     for (int i = j; i < nrt; ++i) {
       const int e = i - npan;
       if (e > j && (e + 1) * f64::TS <= nid) continue;  // identity-row tile that stays zero
+      if (i < npan && i <= j + 2) continue;
       t.push_back(make_int2(i, j));
     }
   return t;
 }
+static size_t flow_counters(int npan, int nrt) { return (size_t)(nrt + 1) * f64::CSTR + 2 * (size_t)npan; }
 
 // Launch variants: 0 one launch per panel (k_f64_panel), 1 two launches per
 // panel (k_f64_solve2 + k_f64_update2), 2-4 one cooperative launch
 // (k_f64_coop) with 1, 2 or 4 CTAs per SM, 5 the dataflow form (k_f64_flow,
-// as many CTAs as fit).  `bar` (a zeroed counter for k_f64_coop; npan x nrt
-// zeroed tile flags for k_f64_flow, whose tile list goes to `tl`) and `err`
-// (set on a wait timeout) serve the cooperative forms.
+// at most one CTA per SM).  `bar` (a zeroed counter for k_f64_coop;
+// flow_counters() zeroed words for k_f64_flow, whose tile list goes to `tl`)
+// and `err` (set on a wait timeout) serve the cooperative forms.
 static void right_looking_fp64(cudaStream_t st, const Win& w, Win* wd, double* buf, double* dv, int* info,
                                int nid = 0, int variant = 0, unsigned* bar = nullptr, int* err = nullptr,
                                int2* tl = nullptr) {
@@ -458,12 +461,19 @@ static void right_looking_fp64(cudaStream_t st, const Win& w, Win* wd, double* b
   const int npan = w.npad / TS, nrt = (w.rows + TS - 1) / TS;
   const int64_t ld = w.npad;
   if (variant == 5) {
-    const std::vector<int2> tiles = flow_tiles(npan, nrt, nid);
-    const int G = std::max(1, std::min(coop_capacity(1), (int)tiles.size()));
+    // padding panels are left out (L = I there already); appended rows follow row ld
+    const int np = (w.n + TS - 1) / TS, nt = np + (w.rows - w.npad + TS - 1) / TS;
+    const std::vector<int2> tiles = flow_tiles(np, nt, nid);
+    int sms = 0, dev = 0;
+    LMA_CK(cudaGetDevice(&dev));
+    LMA_CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    const int cap = std::min(sms, coop_capacity(1));
+    const int band = std::max(np > 2 ? 1 : 0, std::min({kBand, np - 2, cap - 2}));
+    const int G = 1 + band + std::max(1, std::min(cap - 1 - band, (int)tiles.size()));
     stage_copy(tl, tiles.data(), sizeof(int2) * tiles.size(), st);
-    LMA_CK(cudaMemsetAsync(bar, 0, sizeof(unsigned) * (size_t)npan * nrt, st));
-    launch_coop("k_f64_flow", k_f64_flow, (unsigned)G, NTH, 0, st, buf, ld, w.rows, npan, nid, dv, info,
-                (const int2*)tl, (int)tiles.size(), bar, err);
+    LMA_CK(cudaMemsetAsync(bar, 0, sizeof(unsigned) * flow_counters(np, nt), st));
+    launch_coop("k_f64_flow", k_f64_flow, (unsigned)G, FTH, 0, st, buf, ld, w.rows, np, nt, nid, dv, info,
+                (const int2*)tl, (int)tiles.size(), band, bar, err);
     return;
   }
   if (variant >= 2) {
@@ -513,9 +523,9 @@ static void factor_fp64_single(cudaStream_t st, Arena& tmp, double* buf, int n, 
   w.npad = npad;
   w.rows = npad + extra;
   double* dv = tmp.alloc<double>((size_t)npad * TB);
-  const size_t nflag = (size_t)(npad / f64::TS) * ((w.rows + f64::TS - 1) / f64::TS);
-  unsigned* bar = tmp.alloc<unsigned>(nflag);
-  int2* tl = tmp.alloc<int2>(nflag);
+  const int npt = npad / f64::TS, nrt = (w.rows + f64::TS - 1) / f64::TS;
+  unsigned* bar = tmp.alloc<unsigned>(flow_counters(npt, nrt));
+  int2* tl = tmp.alloc<int2>((size_t)npt * nrt);
   const size_t bytes = (size_t)w.rows * npad * sizeof(double);
   double* scratch = nullptr;
   int* sinfo = nullptr;

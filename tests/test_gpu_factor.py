@@ -1,0 +1,51 @@
+"""The FP64 dataflow factorisation of Sigma_SS and I + A and the FP32 diagonal
+block factorisation at the edges of their tiles, against the oracle.
+
+The bounds are the repository's: 1e-9 for the FP64 form; for the mixed form
+1e-4 on the mean and, as FP32 windows allow, 6e-4 on the variance and 1.5e-4 on
+the log-likelihood."""
+import numpy as np
+import pytest
+
+from oracle import lma_oracle as O2
+from workloads import make_random_problem
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def L():
+    import paper_1411_4510_gb300 as L
+    yield L
+    L.lma_autotune_pin(None)
+
+
+def _rel(a, b):
+    return float(np.linalg.norm(np.asarray(a) - np.asarray(b)) / np.linalg.norm(np.asarray(b)))
+
+
+def _errors(L, p, precision):
+    f = O2.fit(p)
+    m_ref, v_ref = O2.predict(f)
+    model = L.lma_fit(precision=precision, **L.problem_args(p))
+    assert L.lma_model_precision(model) == precision
+    mean, var = L.lma_predict(model, p.XU, p.test_block_ptr)
+    return _rel(mean, m_ref), _rel(var, v_ref), abs(L.lma_model_loglik(model) - f.loglik) / abs(f.loglik)
+
+
+@pytest.mark.parametrize("s", [1, 15, 16, 17, 32, 33, 47, 49, 64, 65, 161])
+def test_dataflow_factor_at_tile_edges(L, s):
+    """One to eleven 16-column panels, the last one full or not, with the appended identity rows and the y row."""
+    p = make_random_problem(40 + s, (60, 55, 70), d=3, s=s, B=1, test_sizes=(5, 0, 7))
+    L.lma_autotune_pin(None)
+    L.lma_autotune_pin("fp64 factor", 5)
+    em, ev, el = _errors(L, p, L.FP64)
+    assert em <= 1e-9 and ev <= 1e-9 and el <= 1e-9, (em, ev, el)
+
+
+@pytest.mark.parametrize("sizes", [(1, 1, 1), (63, 1, 64), (64, 64, 64), (65, 63, 66), (129, 128, 1)])
+def test_diagonal_blocks_at_tile_edges(L, sizes):
+    """Windows of one to five 64-column panels, full and padded ones, first and second panels of a group."""
+    p = make_random_problem(7, sizes, d=2, s=min(20, sum(sizes)), B=1, test_sizes=(3, 4, 5))
+    em, ev, el = _errors(L, p, L.MIXED)
+    assert em <= 1e-4 and ev <= 6e-4 and el <= 1.5e-4, (em, ev, el)

@@ -5,6 +5,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <type_traits>
+
 #include "lma_types.cuh"
 
 namespace lma {
@@ -490,6 +492,211 @@ struct CholSmem {
   T D[TB][TB + 1];
   T X[TB][TB + 1];
 };
+
+// Shared memory of diag_factor64 besides the tile itself.
+constexpr int DP = 68;  // row pitch of the 64-wide tiles: 8 rows x 4 columns without bank conflicts, 16-byte aligned
+template <typename T>
+struct alignas(16) Diag64Smem {
+  T X[64][DP];
+  alignas(16) T A[3][64][8];   // a_rj = L_rj / sqrt(pivot j) of the last panels, one 8-column panel each
+  alignas(16) T C[8][65][8];   // the panels' unscaled columns (a replaced pivot is 1 here)
+  alignas(16) T Xu[2][64][8];  // the panels' unscaled inverse rows, by column
+  alignas(16) T rj[64];
+};
+
+// 8 values between (16-byte aligned) shared memory and registers, 16 bytes at a time.
+__device__ __forceinline__ void load8(float (&v)[8], const float* p) {
+#pragma unroll
+  for (int q = 0; q < 8; q += 4) {
+    const float4 f = *reinterpret_cast<const float4*>(p + q);
+    v[q] = f.x;
+    v[q + 1] = f.y;
+    v[q + 2] = f.z;
+    v[q + 3] = f.w;
+  }
+}
+__device__ __forceinline__ void load8(double (&v)[8], const double* p) {
+#pragma unroll
+  for (int q = 0; q < 8; q += 2) {
+    const double2 f = *reinterpret_cast<const double2*>(p + q);
+    v[q] = f.x;
+    v[q + 1] = f.y;
+  }
+}
+__device__ __forceinline__ void store8(float* p, const float (&v)[8]) {
+#pragma unroll
+  for (int q = 0; q < 8; q += 4) *reinterpret_cast<float4*>(p + q) = make_float4(v[q], v[q + 1], v[q + 2], v[q + 3]);
+}
+__device__ __forceinline__ void store8(double* p, const double (&v)[8]) {
+#pragma unroll
+  for (int q = 0; q < 8; q += 2) *reinterpret_cast<double2*>(p + q) = make_double2(v[q], v[q + 1]);
+}
+
+// Cholesky of the 64 x 64 diagonal tile held in D (shared memory, lower part
+// significant) together with the inverse of the factor; L (zeros above the
+// diagonal) goes to Lout (leading dim ld), inv(L) to Dv (row-major).  Called by
+// the 256 threads of the CTA; the caller's stores to D need no barrier.
+//
+// The tile is one serial chain of 64 pivots, so the chain runs in one warp:
+// 8-column panels are factorised by warp 0 in registers (a lane holds rows lane
+// and lane + 32; pivot and column broadcast by shuffles, no barrier), while warps
+// 1 and 2 turn the previous panel's 8 rows of the inverse into final ones and warps
+// 3-7 apply the previous panels to the rest of D and of the inverse, 8 columns at
+// a time; one barrier per panel.  Per element the updates are the right-looking
+//   D_rc -= a_rj D_cj,  X_rc -= a_rj X_jc   (a_rj = (D_rj r) r, r = rsqrt(pivot_j))
+// in the order j = 0, 1, ... of a plain column loop, rows of X scaled by r at the end.
+// A non-positive or NaN pivot is recorded in *info (first failing column + 1,
+// offset k0) and replaced by 1 so the sweep stays finite.
+//
+// A barrier and an update of the whole tile per column (the form before) made
+// k_chol_step_tc 35 us for 64 windows; this one 14 (first panel of a 128-column
+// group) and 18 (second panel, with its product).
+template <typename T>
+__device__ void diag_factor64(T (*D)[DP], Diag64Smem<T>& sm, T* Lout, int64_t ld, T* Dv, int* info, int k0) {
+  const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
+  T aa[8], ab[8];  // warp 0: the last panel's a values of rows lane, lane + 32
+  int first = 0;   // first failing column + 1
+  // warp 0: columns [j0, j0 + 8): the panel before applied, then factorised; up: the pivot rows are the lanes'
+  // second rows
+  auto panel = [&](int pp, auto up) {
+    const int j0 = 8 * pp, jl = j0 & 31;
+    T da[8], db[8];
+    load8(da, &D[lane][j0]);
+    load8(db, &D[lane + 32][j0]);
+    if (pp > 0) {
+#pragma unroll
+      for (int c = 0; c < 8; ++c) {
+        T cv[8];
+        load8(cv, sm.C[pp - 1][j0 + c]);
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+          da[c] = fma(-aa[q], cv[q], da[c]);
+          db[c] = fma(-ab[q], cv[q], db[c]);
+        }
+      }
+    }
+    T ca[8], cb[8];
+    T rv = T(0);
+#pragma unroll
+    for (int jj = 0; jj < 8; ++jj) {
+      const T src = up ? db[jj] : da[jj];
+      T piv = __shfl_sync(0xffffffffu, src, jl + jj);
+      T cv[8];
+#pragma unroll
+      for (int c = jj + 1; c < 8; ++c) cv[c] = __shfl_sync(0xffffffffu, src, jl + c);
+      const bool good = piv > T(0);
+      piv = good ? piv : T(1);
+      if (!good && first == 0) first = j0 + jj + 1;
+      const T r = rsqrt(piv);
+      ca[jj] = (!up && lane == jl + jj) ? piv : da[jj];
+      cb[jj] = (up && lane == jl + jj) ? piv : db[jj];
+      aa[jj] = (da[jj] * r) * r;
+      ab[jj] = (db[jj] * r) * r;
+#pragma unroll
+      for (int c = jj + 1; c < 8; ++c) {
+        da[c] = fma(-aa[jj], cv[c], da[c]);
+        db[c] = fma(-ab[jj], cv[c], db[c]);
+      }
+      if (lane == jj) rv = r;
+    }
+    store8(sm.A[pp % 3][lane], aa);
+    store8(sm.A[pp % 3][lane + 32], ab);
+    store8(sm.C[pp][lane], ca);
+    store8(sm.C[pp][lane + 32], cb);
+    if (lane < 8) sm.rj[j0 + lane] = rv;
+  };
+  using Lower = std::integral_constant<bool, false>;
+  using Upper = std::integral_constant<bool, true>;
+  __syncthreads();
+  if (warp == 0) panel(0, Lower{});
+#pragma unroll 1
+  for (int pp = 0; pp < 8; ++pp) {
+    const int j0 = 8 * pp;
+    __syncthreads();  // panel pp, the inverse rows of panel pp - 1 and the updates of panel pp - 1 are done
+    if (warp == 0) {
+      if (pp < 3) panel(pp + 1, Lower{});
+      else if (pp < 7) panel(pp + 1, Upper{});
+    } else if (warp <= 2) {
+      // inverse rows j0 .. j0 + 7, column c of this lane: panel pp - 1, then the panel's own triangle
+      const int c = t - 32;
+      if (c < j0 + 8) {
+        T x[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) x[i] = c < j0 - 8 ? sm.X[j0 + i][c] : (j0 + i == c ? T(1) : T(0));
+        if (c < j0) {
+          T xu[8];
+          load8(xu, sm.Xu[(pp - 1) & 1][c]);
+#pragma unroll
+          for (int i = 0; i < 8; ++i) {
+            T a[8];
+            load8(a, sm.A[(pp + 2) % 3][j0 + i]);
+#pragma unroll
+            for (int q = 0; q < 8; ++q) x[i] = fma(-a[q], xu[q], x[i]);
+          }
+        }
+#pragma unroll
+        for (int i = 1; i < 8; ++i) {
+          T a[8];
+          load8(a, sm.A[pp % 3][j0 + i]);
+#pragma unroll
+          for (int q = 0; q < i; ++q) x[i] = fma(-a[q], x[q], x[i]);
+        }
+        T rj[8];
+        load8(rj, sm.rj + j0);
+        store8(sm.Xu[pp & 1][c], x);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) sm.X[j0 + i][c] = x[i] * rj[i];
+      }
+    } else if (pp < 7) {
+      // rows of D below the next panel's columns take panel pp, rows of X panel pp - 1 (a column's first one
+      // starts from zero): four threads a row, four columns of it in flight per thread
+      const int u = t - 96, p = u & 3;
+      for (int rd = j0 + 16 + (u >> 2); rd < 64; rd += 40) {
+        T a[8];
+        load8(a, sm.A[pp % 3][rd]);
+#pragma unroll 4
+        for (int c = j0 + 16 + p; c <= rd; c += 4) {
+          T cv[8];
+          load8(cv, sm.C[pp][c]);
+          T d = D[rd][c];
+#pragma unroll
+          for (int q = 0; q < 8; ++q) d = fma(-a[q], cv[q], d);
+          D[rd][c] = d;
+        }
+      }
+      if (pp > 0)
+        for (int rx = j0 + 8 + 39 - (u >> 2); rx < 64; rx += 40) {  // (the threads whose rows of D are the longest first)
+          T a[8];
+          load8(a, sm.A[(pp + 2) % 3][rx]);
+#pragma unroll 4
+          for (int c = p; c < j0; c += 4) {
+            T xu[8];
+            load8(xu, sm.Xu[(pp - 1) & 1][c]);
+            T x = c < j0 - 8 ? sm.X[rx][c] : T(0);
+#pragma unroll
+            for (int q = 0; q < 8; ++q) x = fma(-a[q], xu[q], x);
+            sm.X[rx][c] = x;
+          }
+        }
+    }
+  }
+  if (t == 0 && first && *info == 0) *info = k0 + first;
+  __syncthreads();
+#pragma unroll
+  for (int e = t; e < 64 * 8; e += 256) {
+    const int r = e >> 3, c = (e & 7) * 8;
+    T l[8], rj[8], x[8];
+    load8(l, sm.C[e & 7][r]);
+    load8(rj, sm.rj + c);
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      l[q] = c + q <= r ? l[q] * rj[q] : T(0);  // L_rc = D_rc r_c
+      x[q] = c + q <= r ? sm.X[r][c + q] : T(0);
+    }
+    store8(Lout + (int64_t)r * ld + c, l);
+    store8(Dv + r * 64 + c, x);
+  }
+}
 
 // Cholesky of the N x N diagonal tile held in D (shared memory, lower part
 // significant) together with the inverse of the factor; L (zeros above the

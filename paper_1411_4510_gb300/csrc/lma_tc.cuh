@@ -553,74 +553,73 @@ __global__ void __launch_bounds__(256, 2) k_chol_step_tc(const Win* __restrict__
   const Win w = wins[blockIdx.x];
   const int k0 = kp * TB;
   if (k0 >= w.npad) return;
-  const int r0 = k0 + blockIdx.y * 128;
-  if (r0 >= w.rows) return;
   extern __shared__ __align__(16) unsigned char smraw[];
   TcSmem<64>& sm = tc_smem<64>(smraw);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   float* A = buf + w.base;
   const int64_t ld = w.npad;
-  if (tid == 0) {
-    mbar_init(&sm.bar[0], 1);
-    mbar_init(&sm.bar[1], 1);
-    mbar_fence_init();
+  // the block itself, loaded ahead of the product (coalesced, four float4 a thread)
+  float4 own[4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const int i = tid + 256 * j;
+    own[j] = *reinterpret_cast<const float4*>(A + (int64_t)(k0 + (i >> 4)) * ld + k0 + 4 * (i & 15));
   }
-  if (warp == 0) tmem_alloc(&sm.tmem, 64);
-  fence_before_sync();
-  __syncthreads();
-  fence_after_sync();
-  const uint32_t tmem = sm.tmem;
-  TcPipe pipe;
-  bool ok = true;
   const int K = k0 - kb;
+  bool ok = true;
+  uint32_t tmem = 0;
   if (K > 0) {
-    auto rowA = [&](int r) -> const float* {
-      const int row = r0 + r;
-      return (r < TB && row < w.rows) ? A + (int64_t)row * ld + kb : nullptr;
-    };
+    if (tid == 0) {
+      mbar_init(&sm.bar[0], 1);
+      mbar_init(&sm.bar[1], 1);
+      mbar_fence_init();
+    }
+    if (warp == 0) tmem_alloc(&sm.tmem, 64);
+    fence_before_sync();
+    __syncthreads();
+    fence_after_sync();
+    tmem = sm.tmem;
+    TcPipe pipe;
+    auto rowA = [&](int r) -> const float* { return r < TB ? A + (int64_t)(k0 + r) * ld + kb : nullptr; };
     auto rowB = [&](int c) -> const float* { return A + (int64_t)(k0 + c) * ld + kb; };
     ok = tile_product<64>(sm, pipe, tmem, K, rowA, rowB);
-  }
-  if (!ok && tid == 0) atomicExch(err, 1);
-  const int q = warp & 3, half = warp >> 2;
-  const int rl = q * 32 + lane;
-  const int row = r0 + rl;
-  float v[32];
-  if (K > 0 && ok) {
-    float t[16];
-    tmem_ld16(tmem + ((uint32_t)(q * 32) << 16) + half * 32, t);
-#pragma unroll
-    for (int j = 0; j < 16; ++j) v[j] = t[j];
-    tmem_ld16(tmem + ((uint32_t)(q * 32) << 16) + half * 32 + 16, t);
-#pragma unroll
-    for (int j = 0; j < 16; ++j) v[16 + j] = t[j];
-  } else {
-#pragma unroll
-    for (int j = 0; j < 32; ++j) v[j] = 0.f;
+    if (!ok && tid == 0) atomicExch(err, 1);
   }
   // all MMAs have completed (tile_product drained both stages): stage memory is free
   float* scratch = reinterpret_cast<float*>(&sm.st[0]);
-  float(*Dm)[TB + 1] = reinterpret_cast<float(*)[TB + 1]>(scratch);
-  if (row < w.rows && rl < TB) {  // the diagonal block's rows only; the rows below are left to the panel kernels
-    const float* src = A + (int64_t)row * ld + k0 + half * 32;
-    float4 av[8];
+  float(*Dm)[DP] = reinterpret_cast<float(*)[DP]>(scratch);
 #pragma unroll
-    for (int j4 = 0; j4 < 8; ++j4) av[j4] = *reinterpret_cast<const float4*>(src + 4 * j4);
-#pragma unroll
-    for (int j4 = 0; j4 < 8; ++j4) {
-      float* d = &Dm[rl][half * 32 + 4 * j4];
-      d[0] = av[j4].x - v[4 * j4 + 0];
-      d[1] = av[j4].y - v[4 * j4 + 1];
-      d[2] = av[j4].z - v[4 * j4 + 2];
-      d[3] = av[j4].w - v[4 * j4 + 3];
-    }
+  for (int j = 0; j < 4; ++j) {
+    const int i = tid + 256 * j;
+    *reinterpret_cast<float4*>(&Dm[i >> 4][4 * (i & 15)]) = own[j];
   }
-  fence_before_sync();
-  __syncthreads();
-  if (warp == 0) tmem_dealloc(tmem, 64);
-  if (blockIdx.y == 0)
-    diag_factor<float>(Dm, A + (int64_t)k0 * ld + k0, ld, dinv + w.dinv + (int64_t)kp * TB * TB, info + blockIdx.x,
-                       k0);
+  if (K > 0) {
+    __syncthreads();
+    const int q = warp & 3, half = warp >> 2;  // rows 32 q + lane (the first 64 of the tile's 128), columns 32 half ..
+    if (ok && q < 2) {
+      float* d = &Dm[q * 32 + lane][half * 32];
+#pragma unroll
+      for (int g = 0; g < 2; ++g) {
+        float t[16];
+        tmem_ld16(tmem + ((uint32_t)(q * 32) << 16) + half * 32 + 16 * g, t);
+#pragma unroll
+        for (int j = 0; j < 16; j += 4) {
+          float4* p = reinterpret_cast<float4*>(d + 16 * g + j);
+          float4 v = *p;
+          v.x -= t[j];
+          v.y -= t[j + 1];
+          v.z -= t[j + 2];
+          v.w -= t[j + 3];
+          *p = v;
+        }
+      }
+    }
+    fence_before_sync();
+    __syncthreads();
+    if (warp == 0) tmem_dealloc(tmem, 64);
+  }
+  diag_factor64<float>(Dm, *reinterpret_cast<Diag64Smem<float>*>(scratch + TB * DP), A + (int64_t)k0 * ld + k0,
+                       ld, dinv + w.dinv + (int64_t)kp * TB * TB, info + blockIdx.x, k0);
 }
 
 }  // namespace lma

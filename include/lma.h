@@ -44,7 +44,7 @@ typedef enum {
 } lma_status;
 
 typedef enum {
-  LMA_FP64 = 0,   /* plain FP64 GPU form: every step in double, one window per launch   */
+  LMA_FP64 = 0,   /* plain FP64 GPU form: every step in double on the CUDA cores         */
   LMA_MIXED = 1   /* FP32 covariance tiles / factorisations / solves, batched over all
                      windows; FP64 for Sigma_SS, the global summary and all reductions   */
 } lma_precision;

@@ -806,10 +806,19 @@ __device__ void flow_band(FlowBand& w, double* buf, int64_t ld, int npan, const 
   }
 }
 
-// A group's tiles t = first, first + step, ... of the list.
-__device__ void flow_bulk(FlowBulk& w, int bar, double* buf, int64_t ld, int rows, int npan, int nid,
-                          const double* dinv, const int2* tiles, int ntiles, int first, int step, unsigned* prog,
-                          const unsigned* xprog, int* err) {
+// One matrix of a factorisation, as the bulk sees it.
+struct FlowMat {
+  double* buf;
+  const double* dinv;
+  unsigned* cnt;  // zeroed counters: prog (nrt x CSTR), xprog (CSTR), hsub (npan), hdiag (npan)
+  int64_t ld;
+  int rows, npan, nrt, nid;
+};
+
+// A group's tiles t = first, first + step, ... < ntiles; tile(t, m, i, j) gives the matrix and the tile.  HAND: the
+// list holds tiles (j + 1, j) and (j, j) too; they get the panels below j and j - 1 and are handed to the chain.
+template <bool HAND, class Tile>
+__device__ void flow_bulk(FlowBulk& w, int bar, int ntiles, int first, int step, Tile tile, int* err) {
   const int lane = threadIdx.x & 31, gw = (threadIdx.x >> 5) & 3, gt = threadIdx.x & 127;
   const int r = lane & 15, h = lane >> 4;
   const int c0 = 2 * gw + h, c1 = 2 * (7 - gw) + h;  // this thread's elements: row r, columns c0 and c1
@@ -817,13 +826,19 @@ __device__ void flow_bulk(FlowBulk& w, int bar, double* buf, int64_t ld, int row
   volatile unsigned* shared_have = &w.have;
   auto sync = [&] { bar_sync(bar, 128); };
   for (int t = first; t < ntiles; t += step) {
-    const int i = tiles[t].x, j = tiles[t].y;
-    const bool app = i >= npan;
-    const int ri = flow_row0(i, npan, ld), rj = j * TS;
-    const int k0 = (app && (i - npan + 1) * TS <= nid) ? i - npan : 0;  // identity rows: zero before column i - npan
-    const bool li = ri + lrow < rows;
-    double* pi = buf + (int64_t)(ri + lrow) * ld + lc;
-    const double* pj = buf + (int64_t)(rj + lrow) * ld + lc;
+    FlowMat m;
+    int i, j;
+    tile(t, m, i, j);
+    unsigned* prog = m.cnt;
+    unsigned* xprog = m.cnt + (int64_t)m.nrt * CSTR;
+    const bool app = i >= m.npan;
+    const int ri = flow_row0(i, m.npan, m.ld), rj = j * TS;
+    const int k0 = (app && (i - m.npan + 1) * TS <= m.nid) ? i - m.npan : 0;  // identity rows: zero before column i - npan
+    const bool handed = HAND && !app && i <= j + 1;
+    const int kend = HAND && i == j ? j - 1 : j;
+    const bool li = ri + lrow < m.rows;
+    double* pi = m.buf + (int64_t)(ri + lrow) * m.ld + lc;
+    const double* pj = m.buf + (int64_t)(rj + lrow) * m.ld + lc;
     const double2 zero = make_double2(0.0, 0.0);
     double2 ga = zero, gb = zero;
     auto load = [&](int k) {
@@ -839,12 +854,12 @@ __device__ void flow_bulk(FlowBulk& w, int bar, double* buf, int64_t ld, int row
     const unsigned *fi = prog + (int64_t)i * CSTR, *fj = prog + (int64_t)j * CSTR;
     unsigned have = 0;
     bool ahead = false;  // ga / gb hold panel k already
-    for (int k = k0; k < j; ++k) {
+    for (int k = k0; k < kend; ++k) {
       if (!ahead) {
         if (have < (unsigned)(k + 1)) {
           if (gw == 0) {
-            const unsigned m = wait_rows(fi, fj, (unsigned)(k + 1), err);
-            if (lane == 0) *shared_have = m;
+            const unsigned v = wait_rows(fi, fj, (unsigned)(k + 1), err);
+            if (lane == 0) *shared_have = v;
           }
           sync();
           have = *shared_have;
@@ -856,7 +871,7 @@ __device__ void flow_bulk(FlowBulk& w, int bar, double* buf, int64_t ld, int row
       stash(w.a, ga);
       stash(w.b, gb);
       sync();
-      ahead = k + 1 < j && have >= (unsigned)(k + 2);
+      ahead = k + 1 < kend && have >= (unsigned)(k + 2);
       if (ahead) load(k + 1);
 #pragma unroll
       for (int kk = 0; kk < TS; kk += 2) {
@@ -869,30 +884,35 @@ __device__ void flow_bulk(FlowBulk& w, int bar, double* buf, int64_t ld, int row
         a1 = fma(-a.y, b1.y, a1);
       }
     }
-    if (gt == 0) *shared_have = wait_count(xprog, (unsigned)(j + 1), err) ? 1u : 0u;
+    if (!handed && gt == 0) *shared_have = wait_count(xprog, (unsigned)(j + 1), err) ? 1u : 0u;
     sync();
     w.a[r][c0] = a0;
     w.a[r][c1] = a1;
-    if (!*shared_have) return;
-    stash(w.b, __ldcg(reinterpret_cast<const double2*>(dinv + (int64_t)j * TS * TS + lrow * TS + lc)));
-    sync();
-    // out = T inv(L_jj)^T; inv(L_jj) is lower, so columns c <= 2 p + 1 end at k = 2 p + 1
-    double o0 = 0.0, o1 = 0.0;
+    if (!handed) {
+      if (!*shared_have) return;
+      stash(w.b, __ldcg(reinterpret_cast<const double2*>(m.dinv + (int64_t)j * TS * TS + lrow * TS + lc)));
+      sync();
+      // out = T inv(L_jj)^T; inv(L_jj) is lower, so columns c <= 2 p + 1 end at k = 2 p + 1
+      double o0 = 0.0, o1 = 0.0;
 #pragma unroll
-    for (int kk = 0; kk < TS; ++kk) {
-      const double u = w.a[r][kk];
-      if (kk < 2 * gw + 2) o0 = fma(u, w.b[c0][kk], o0);
-      if (kk < 16 - 2 * gw) o1 = fma(u, w.b[c1][kk], o1);
+      for (int kk = 0; kk < TS; ++kk) {
+        const double u = w.a[r][kk];
+        if (kk < 2 * gw + 2) o0 = fma(u, w.b[c0][kk], o0);
+        if (kk < 16 - 2 * gw) o1 = fma(u, w.b[c1][kk], o1);
+      }
+      sync();
+      w.a[r][c0] = o0;
+      w.a[r][c1] = o1;
     }
-    sync();
-    w.a[r][c0] = o0;
-    w.a[r][c1] = o1;
     sync();
     if (li) *reinterpret_cast<double2*>(pi + j * TS) = *reinterpret_cast<const double2*>(&w.a[lrow][lc]);
     sync();
     if (gt == 0) {
       __threadfence();
-      st_rel(prog + (int64_t)i * CSTR, (unsigned)(j + 1));
+      if (!handed)
+        st_rel(prog + (int64_t)i * CSTR, (unsigned)(j + 1));
+      else
+        st_rel(xprog + CSTR + (i == j ? m.npan : 0) + j, 1u);
     }
   }
 }
@@ -913,7 +933,172 @@ __global__ void __launch_bounds__(FTH, 1) k_f64_flow(double* buf, int64_t ld, in
   else if (b < 0)
     flow_band(sm.b, buf, ld, npan, dinv, 1 + (int)blockIdx.x, nband, prog, xprog, hsub, hdiag, err);
   else
-    flow_bulk(sm.g[g], 1 + g, buf, ld, rows, npan, nid, dinv, tiles, ntiles, g * nb + b, nb * FG, prog, xprog, err);
+    flow_bulk<false>(
+        sm.g[g], 1 + g, ntiles, g * nb + b, nb * FG,
+        [&](int t, FlowMat& m, int& i, int& j) {
+          i = tiles[t].x;
+          j = tiles[t].y;
+          m = FlowMat{buf, dinv, cnt, ld, rows, npan, nrt, nid};
+        },
+        err);
+}
+
+// The same for many matrices at once (the FP64 form's windows): one launch
+// factorises `nwin` windows and solves their extra rows.  Block c < nchain is the
+// chain of windows c, c + nchain, ...; the other CTAs' groups take the tiles of all
+// windows (list: window, i, j; round by round of nchain windows, then column by
+// column), among them, ahead of column j's others, (j + 1, j) and (j + 1, j + 1) up
+// to the panel that the chain applies itself.  The FP64 pipe bounds it once there are enough windows: a group's warp
+// keeps two of its four 64-clock slots a 16-column step busy.  dv16: 16 x 16
+// inverse diagonal tiles (npan per window from its dv on), cnt: FlowMat counters.
+//
+// 16 windows of 250 points with 65 extra rows: 0.21 ms against 17.2 of 64-wide panel
+// launches, a window at a time, before; 20 windows of 500 with 201: 1.9 against 63.7.
+struct FlowWin {
+  int64_t base, dv, cnt;
+  int ld, rows, npan, nrt;
+};
+__global__ void __launch_bounds__(FTH, 1) k_f64_windows(const FlowWin* __restrict__ wins, int nwin, int nchain,
+                                                        double* buf, double* dv16, int* info,
+                                                        const int4* __restrict__ tiles, int ntiles, unsigned* cnt,
+                                                        int* err) {
+  __shared__ FlowSmem sm;
+  const int g = threadIdx.x >> 7, b = (int)blockIdx.x - nchain, nb = (int)gridDim.x - nchain;
+  if (b < 0) {
+    for (int w = blockIdx.x; w < nwin; w += nchain) {
+      const FlowWin f = wins[w];
+      unsigned* prog = cnt + f.cnt;
+      unsigned* xprog = prog + (int64_t)f.nrt * CSTR;
+      flow_chain(sm.c, buf + f.base, f.ld, f.npan, dv16 + f.dv, info + w, prog, xprog, xprog + CSTR,
+                 xprog + CSTR + f.npan, err);
+    }
+    return;
+  }
+  flow_bulk<true>(
+      sm.g[g], 1 + g, ntiles, g * nb + b, nb * FG,
+      [&](int t, FlowMat& m, int& i, int& j) {
+        const int4 it = tiles[t];
+        const FlowWin f = wins[it.x];
+        i = it.y;
+        j = it.z;
+        m = FlowMat{buf + f.base, dv16 + f.dv, cnt + f.cnt, f.ld, f.rows, f.npan, f.nrt, 0};
+      },
+      err);
+}
+
+// Forward solve of the FP64 form's prediction right-hand sides by the stored
+// factors: CTA (pair, 16 test rows; four warps, one per scheduler) sweeps the
+// window's 16-column panels left to right, P_j = (P_j - sum_{k<j} P_k L_jk^T) inv(L_jj)^T,
+// with the operations of a row of k_f64_windows in the same order, so that a
+// test row has the bits it would have as an extra row of the window.  Bounded by the
+// FP64 pipe, 2,048 clocks a tile product; 64-row CTAs left most SMs without one
+// (31 pairs of C1: 20.5 ms one pair a launch, 0.20 now).
+__global__ void __launch_bounds__(128) k_f64_psweep(const Pair* __restrict__ pairs, const int2* __restrict__ items,
+                                                    const Win* __restrict__ wins, const double* __restrict__ buf,
+                                                    const double* __restrict__ dv16, double* P) {
+  __shared__ __align__(16) double ta[TS][FP], tb[TS][FP];
+  const int2 it = items[blockIdx.x];
+  const Pair pr = pairs[it.x];
+  const Win w = wins[pr.win];
+  const int npan = (w.n + TS - 1) / TS, u0 = it.y * TS;
+  const int lane = threadIdx.x & 31, gw = threadIdx.x >> 5;
+  const int r = lane & 15, h = lane >> 4, c0 = 2 * gw + h, c1 = 2 * (7 - gw) + h;
+  const int lrow = threadIdx.x >> 3, lc = 2 * (threadIdx.x & 7);
+  const bool live = u0 + lrow < pr.nu;
+  const double2 zero = make_double2(0.0, 0.0);
+  double* pi = P + pr.pbase + (int64_t)(u0 + lrow) * w.npad + lc;
+  auto stash = [&](double (*dst)[FP], double2 g) { *reinterpret_cast<double2*>(&dst[lrow][lc]) = g; };
+  for (int j = 0; j < npan; ++j) {
+    const double* pj = buf + w.base + (int64_t)(j * TS + lrow) * w.npad + lc;
+    double2 ga = live ? __ldcg(reinterpret_cast<const double2*>(pi + j * TS)) : zero;
+    __syncthreads();
+    stash(ta, ga);
+    __syncthreads();
+    double a0 = ta[r][c0], a1 = ta[r][c1];
+    double2 gb = zero;
+    auto load = [&](int k) {
+      ga = live ? __ldcg(reinterpret_cast<const double2*>(pi + k * TS)) : zero;
+      gb = *reinterpret_cast<const double2*>(pj + k * TS);
+    };
+    if (j > 0) load(0);
+    for (int k = 0; k < j; ++k) {
+      __syncthreads();
+      stash(ta, ga);
+      stash(tb, gb);
+      __syncthreads();
+      if (k + 1 < j) load(k + 1);
+#pragma unroll
+      for (int kk = 0; kk < TS; kk += 2) {
+        const double2 a = *reinterpret_cast<const double2*>(&ta[r][kk]);
+        const double2 b0 = *reinterpret_cast<const double2*>(&tb[c0][kk]);
+        const double2 b1 = *reinterpret_cast<const double2*>(&tb[c1][kk]);
+        a0 = fma(-a.x, b0.x, a0);
+        a1 = fma(-a.x, b1.x, a1);
+        a0 = fma(-a.y, b0.y, a0);
+        a1 = fma(-a.y, b1.y, a1);
+      }
+    }
+    __syncthreads();
+    ta[r][c0] = a0;
+    ta[r][c1] = a1;
+    stash(tb, *reinterpret_cast<const double2*>(dv16 + w.dinv / 4 + (int64_t)j * TS * TS + lrow * TS + lc));
+    __syncthreads();
+    double o0 = 0.0, o1 = 0.0;
+#pragma unroll
+    for (int kk = 0; kk < TS; ++kk) {
+      const double u = ta[r][kk];
+      if (kk < 2 * gw + 2) o0 = fma(u, tb[c0][kk], o0);
+      if (kk < 16 - 2 * gw) o1 = fma(u, tb[c1][kk], o1);
+    }
+    __syncthreads();
+    ta[r][c0] = o0;
+    ta[r][c1] = o1;
+    __syncthreads();
+    if (live) *reinterpret_cast<double2*>(pi + j * TS) = *reinterpret_cast<const double2*>(&ta[lrow][lc]);
+  }
+}
+
+// inv(L_kk) of every 64 x 64 diagonal block from its 16 x 16 diagonal tiles' inverses (those past npan are the
+// identity): X_ij = -X_ii sum_{j <= k < i} L_ik X_kj, block diagonal by block diagonal.  Grid: x = block, y = window.
+__global__ void __launch_bounds__(256) k_f64_dinv64(const Win* __restrict__ wins, const FlowWin* __restrict__ fw,
+                                                    const double* __restrict__ buf, const double* __restrict__ dv16,
+                                                    double* __restrict__ dinv) {
+  const Win w = wins[blockIdx.y];
+  const FlowWin f = fw[blockIdx.y];
+  const int kp = blockIdx.x;
+  if (kp * TB >= w.npad) return;
+  __shared__ double X[4][4][TS][TS + 1], Lt[TS][TS + 1], S[TS][TS + 1];
+  const int r = threadIdx.x >> 4, c = threadIdx.x & 15;
+  const double* A = buf + w.base + (int64_t)kp * TB * w.npad + kp * TB;
+  for (int i = 0; i < 4; ++i) {
+    const int t = 4 * kp + i;
+    X[i][i][r][c] = t < f.npan ? dv16[f.dv + (int64_t)t * TS * TS + r * TS + c] : (r == c ? 1.0 : 0.0);
+    for (int j = i + 1; j < 4; ++j) X[i][j][r][c] = 0.0;
+  }
+  for (int d = 1; d < 4; ++d)
+    for (int j = 0; j + d < 4; ++j) {
+      const int i = j + d;
+      double acc = 0.0;
+      for (int k = j; k < i; ++k) {
+        __syncthreads();
+        Lt[r][c] = 4 * kp + i < f.npan ? A[(int64_t)(i * TS + r) * w.npad + k * TS + c] : 0.0;
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < TS; ++q) acc = fma(Lt[r][q], X[k][j][q][c], acc);
+      }
+      S[r][c] = acc;
+      __syncthreads();
+      acc = 0.0;
+#pragma unroll
+      for (int q = 0; q < TS; ++q) acc = fma(-X[i][i][r][q], S[q][c], acc);
+      X[i][j][r][c] = acc;
+    }
+  __syncthreads();
+  double* Dv = dinv + w.dinv + (int64_t)kp * TB * TB;
+  for (int e = threadIdx.x; e < TB * TB; e += 256) {
+    const int er = e / TB, ec = e % TB;
+    Dv[e] = X[er >> 4][ec >> 4][er & 15][ec & 15];
+  }
 }
 
 }  // namespace f64

@@ -215,6 +215,7 @@ struct ModelCore {
   int ldvs = 0;               //   ldvs (a multiple of 64; mixed form on the tensor cores only)
   void* wbuf = nullptr;       // window buffers (T)
   void* dinv = nullptr;       // inverted diagonal tiles (T)
+  double* dv16 = nullptr;     // FP64 form: inverted 16x16 diagonal tiles, at a quarter of the window's dinv offset
   void* ew = nullptr;         // per-window L^-1 e (T)
   Win* wins_d = nullptr;
   double* G = nullptr;        // (s+1)^2 global Gram [quad, y; y, A]
@@ -312,10 +313,5 @@ void make_pairs(const std::vector<Win>& wins, int64_t w0, int64_t M, int64_t B, 
                 bool fused, std::vector<Pair>& pairs, std::vector<int4>& tb, int64_t* p_elems);
 // number of appended test rows of each window of a whole fit (FusedTest)
 std::vector<int> fused_test_rows(int64_t M, int64_t B, const int64_t* tptr);
-
-// sweep helpers (defined per precision)
-template <typename T>
-void chol_sweep(cudaStream_t st, const std::vector<Win>& wins, Win* wins_d, T* buf, T* dinv, int* info,
-                bool batched, int* tc_err);
 
 }  // namespace lma

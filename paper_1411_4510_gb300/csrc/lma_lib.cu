@@ -301,20 +301,19 @@ static bool use_tensor_cores() {
   return v == 1;
 }
 
-template <typename T>
 static void set_smem_attr() {
-  cudaFuncSetAttribute(k_chol_step<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(CholSmem<T>));
-  cudaFuncSetAttribute(k_chol_trsm<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(TrsmSmem<T>));
-  cudaFuncSetAttribute(k_pred_sweep<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(CholSmem<T>));
-  cudaFuncSetAttribute(k_bwd_sweep<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(CholSmem<T>));
+  cudaFuncSetAttribute(k_chol_step<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(CholSmem<float>));
+  cudaFuncSetAttribute(k_chol_trsm<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(TrsmSmem<float>));
+  cudaFuncSetAttribute(k_pred_sweep<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(CholSmem<float>));
+  cudaFuncSetAttribute(k_bwd_sweep<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(CholSmem<float>));
+  cudaFuncSetAttribute(k_bwd_sweep<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(CholSmem<double>));
 }
 
 template <typename T>
 void Impl<T>::setup_attributes() {
   static bool done = false;
   if (!done) {
-    set_smem_attr<T>();
-    set_smem_attr<double>();
+    set_smem_attr();
     cudaFuncSetAttribute(k_chol_step_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc_chol_smem());
     cudaFuncSetAttribute(k_chol_panel_pt, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pt_smem());
     cudaFuncSetAttribute(k_pred_sweep_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc_chol_smem());
@@ -335,77 +334,6 @@ void Impl<T>::setup_attributes() {
   }
 }
 
-// Left-looking sweep over all column panels.  batched: every window in
-// each launch; otherwise one window per launch (the plain form).  With the
-// tensor cores (tc_err != nullptr) the panels are grouped in super-panels of
-// 256 columns: one wide update applies all columns left of the super-panel
-// (N = 256 tiles), the 64-wide panel steps add the rest.
-template <typename T>
-void chol_sweep(cudaStream_t st, const std::vector<Win>& wins, Win* wins_d, T* buf, T* dinv, int* info, bool batched,
-                int* tc_err) {
-  if (wins.empty()) return;
-  if (batched) {
-    int maxpan = 0, maxrt = 0;
-    for (const Win& w : wins) {
-      maxpan = std::max(maxpan, w.npad / TB);
-      maxrt = std::max(maxrt, (w.rows + TB - 1) / TB);
-    }
-    const unsigned nw = (unsigned)wins.size();
-    int maxrows = 0;
-    for (const Win& w : wins) maxrows = std::max(maxrows, w.rows);
-    const bool tc = tc_err && sizeof(T) == 4;
-    constexpr int SP = 256, HP = 128;
-    for (int kp = 0; kp < maxpan; ++kp) {
-      const int k0 = kp * TB;
-      if (tc) {
-        // columns [0, kb) of super-panel [kb, kb + 256) come from the 256-wide
-        // update, [kb, kh) of its second half from the 128-wide one, and the
-        // 64-wide panel step adds [kh, k0) (at most 64 columns)
-        const int kb = (k0 / SP) * SP, kh = (k0 / HP) * HP;
-        if (k0 == kb && kb > 0) {
-          const unsigned gy = (unsigned)((maxrows - kb + 127) / 128);
-          launch_pdl("k_chol_wide", k_chol_wide<256>, dim3(nw, gy), tc::kWsThreads, wide_smem<256>(), st, wins_d,
-                     (float*)buf, kb, 0, tc_err);
-        }
-        if (k0 == kh && kh > kb) {
-          const unsigned gy = (unsigned)((maxrows - kh + 127) / 128);
-          launch_pdl("k_chol_mid", k_chol_wide<128>, dim3(nw, gy), tc::kWsThreads, wide_smem<128>(), st, wins_d,
-                     (float*)buf, kh, kb, tc_err);
-        }
-        // every panel: its diagonal block (the first panel of a 128-column
-        // group has every column to its left applied; the second adds the
-        // first's 64 columns), then the persistent kernel updates the rows
-        // below with the same columns and solves them
-        launch_pdl("k_chol_step_tc", k_chol_step_tc, dim3(nw, 1), 256, tc_chol_smem(), st, wins_d, (float*)buf,
-                   (float*)dinv, info, kp, kh, tc_err);
-        if (maxrows - (kp + 1) * TB > 0) {
-          const int ntile = (maxrows - (kp + 1) * TB + 127) / 128;
-          launch_pdl("k_chol_panel_pt", k_chol_panel_pt, persistent_grid((size_t)ntile * nw), tc::kPtThreads,
-                     pt_smem(), st, wins_d, (int)nw, (float*)buf, (const float*)dinv, kp, kh, ntile, tc_err);
-        }
-      } else {
-        launch("k_chol_step", k_chol_step<T>, dim3(maxrt - kp, nw), NT, sizeof(CholSmem<T>), st, wins_d, buf, dinv,
-               info, kp);
-        if (maxrt - kp - 1 > 0)
-          launch("k_chol_trsm", k_chol_trsm<T>, dim3(maxrt - kp - 1, nw), NT, sizeof(TrsmSmem<T>), st, wins_d, buf,
-                 dinv, kp, 0);
-      }
-    }
-  } else {
-    for (size_t wi = 0; wi < wins.size(); ++wi) {
-      const Win& w = wins[wi];
-      const int npan = w.npad / TB, rt = (w.rows + TB - 1) / TB;
-      for (int kp = 0; kp < npan; ++kp) {
-        launch("k_chol_step", k_chol_step<T>, dim3(rt - kp, 1), NT, sizeof(CholSmem<T>), st, wins_d + wi, buf, dinv, info + wi, kp);
-        if (rt - kp - 1 > 0) {
-          launch("k_chol_trsm", k_chol_trsm<T>, dim3(rt - kp - 1, 1), NT, sizeof(TrsmSmem<T>), st, wins_d + wi, buf, dinv, kp,
-                 0);
-        }
-      }
-    }
-  }
-}
-
 // Right-looking factorisation of one FP64 matrix on 16 x 16 tiles (see
 // lma_f64.cuh).  nid: number of leading appended rows that are identity rows
 // (0 = none).  wd is unused (kept for the window form's signature).
@@ -414,9 +342,9 @@ void chol_sweep(cudaStream_t st, const std::vector<Win>& wins, Win* wins_d, T* b
 // latency-bound); variant 1: a solve launch and an update launch per panel
 // (each panel tile solved once; for large orders where the FP64 work counts).
 // CTAs of a cooperative FP64 kernel that can be resident at once on this
-// device (which = 0: k_f64_coop, 1: k_f64_flow).
+// device (which = 0: k_f64_coop, 1: k_f64_flow, 2: k_f64_windows).
 static int coop_capacity(int which = 0) {
-  static int cap[64][2] = {};
+  static int cap[64][3] = {};
   int dev = 0;
   LMA_CK(cudaGetDevice(&dev));
   if (dev < 0 || dev >= 64) return 0;
@@ -424,8 +352,10 @@ static int coop_capacity(int which = 0) {
     int nb = 0, sms = 0;
     if (which == 0)
       LMA_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, f64::k_f64_coop, f64::NTH, 0));
-    else
+    else if (which == 1)
       LMA_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, f64::k_f64_flow, f64::FTH, 0));
+    else
+      LMA_CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, f64::k_f64_windows, f64::FTH, 0));
     LMA_CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     cap[dev][which] = std::max(1, nb * sms);
   }
@@ -506,6 +436,147 @@ static void right_looking_fp64(cudaStream_t st, const Win& w, Win* wd, double* b
     if (trail + solve > 0)
       launch_pdl("k_f64_panel", k_f64_panel, (unsigned)(trail + solve), NTH, 0, st, buf, ld, w.rows, npan, kp, nid, dv,
              info);
+  }
+}
+
+// The FP64 form's windows, factorised and their extra rows solved by
+// k_f64_windows, up to kWinBatch windows a launch (which bounds the tile list).
+// Chains: each takes about 16,000 clocks a 16-column panel whatever its window's
+// rows, a bulk CTA 2,048 clocks a tile update; the number of chain CTAs is the one
+// that lets both sides end together.
+static void sweep_fp64(cudaStream_t st, Arena& tmp, const std::vector<Win>& wins, const Win* wins_d, double* buf,
+                       double* dinv, double* dv16, int* info, int* err) {
+  using namespace f64;
+  constexpr size_t kWinBatch = 64;
+  int dev = 0, sms = 0;
+  LMA_CK(cudaGetDevice(&dev));
+  LMA_CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+  const int cap = std::max(2, std::min(sms, coop_capacity(2)));
+  std::vector<FlowWin> fw(wins.size());
+  size_t maxcnt = 0;
+  int maxblk = 0;
+  for (size_t b = 0; b < wins.size(); b += kWinBatch) {
+    size_t cnt = 0;
+    for (size_t k = b; k < std::min(wins.size(), b + kWinBatch); ++k) {
+      const Win& w = wins[k];
+      FlowWin& f = fw[k];
+      f.base = w.base;
+      f.ld = w.npad;
+      f.rows = w.rows;
+      f.npan = (w.n + TS - 1) / TS;
+      f.nrt = f.npan + (w.rows - w.npad + TS - 1) / TS;
+      f.dv = w.dinv / 4;
+      f.cnt = (int64_t)cnt;
+      cnt += flow_counters(f.npan, f.nrt);
+      maxblk = std::max(maxblk, w.npad / TB);
+    }
+    maxcnt = std::max(maxcnt, cnt);
+  }
+  FlowWin* fwd = tmp.alloc<FlowWin>(fw.size());
+  unsigned* cntd = tmp.alloc<unsigned>(maxcnt);
+  stage_copy(fwd, fw.data(), sizeof(FlowWin) * fw.size(), st);
+  for (size_t b = 0; b < wins.size(); b += kWinBatch) {
+    const int nw = (int)std::min(wins.size() - b, kWinBatch);
+    double bulk = 0.0;
+    int maxpan = 0;
+    for (int w = 0; w < nw; ++w) {
+      const FlowWin& f = fw[b + w];
+      const double p = f.npan, e = f.nrt - f.npan;
+      bulk += 2048.0 * (p * p * p / 6.0 + (e + 0.5) * p * p / 2.0);
+      maxpan = std::max(maxpan, f.npan);
+    }
+    int nchain = 1;
+    double best = 0.0;
+    for (int c = 1; c <= std::min(nw, cap - 1); ++c) {
+      const double t = std::max(16000.0 * maxpan * ((nw + c - 1) / c), bulk / (cap - c));
+      if (c == 1 || t < best) {
+        best = t;
+        nchain = c;
+      }
+    }
+    std::vector<int4> tiles;
+    for (int w0 = 0; w0 < nw; w0 += nchain)
+      for (int j = 0; j < maxpan; ++j)
+        for (int w = w0; w < std::min(nw, w0 + nchain); ++w) {
+          const FlowWin& f = fw[b + w];
+          if (j >= f.npan) continue;
+          // what the chain's panel j needs comes before the tiles that need that panel (no wait is for a tile
+          // later in the list); panel 0 finds it in the original matrix
+          if (j > 0 && j + 1 < f.npan) {
+            tiles.push_back(make_int4(w, j + 1, j, 0));
+            tiles.push_back(make_int4(w, j + 1, j + 1, 0));
+          }
+          for (int i = std::min(j + 2, f.npan); i < f.nrt; ++i) tiles.push_back(make_int4(w, i, j, 0));
+        }
+    int4* tl = tmp.alloc<int4>(tiles.size());
+    stage_copy(tl, tiles.data(), sizeof(int4) * tiles.size(), st);
+    LMA_CK(cudaMemsetAsync(cntd, 0, sizeof(unsigned) * maxcnt, st));
+    const int nbulk = std::max(1, std::min(cap - nchain, (int)std::min<size_t>(tiles.size(), 1 << 20)));
+    launch_coop("k_f64_windows", k_f64_windows, (unsigned)(nchain + nbulk), FTH, 0, st, (const FlowWin*)(fwd + b), nw,
+                nchain, buf, dv16, info + b, (const int4*)tl, (int)tiles.size(), cntd, err);
+    tmp.free_one(tl);
+  }
+  for (size_t b = 0; b < wins.size(); b += 65535)
+    launch("k_f64_dinv64", k_f64_dinv64, dim3(maxblk, (unsigned)std::min<size_t>(65535, wins.size() - b)), 256, 0, st,
+           wins_d + b, (const FlowWin*)(fwd + b), (const double*)buf, (const double*)dv16, dinv);
+}
+
+// Factorises every window and solves its extra rows.  Mixed form: a left-looking
+// sweep over the column panels, every window in each launch; with the tensor
+// cores the panels are grouped in super-panels of 256 columns: one wide update
+// applies all columns left of the super-panel (N = 256 tiles), the 64-wide panel
+// steps add the rest.  FP64 form: sweep_fp64.  *err: set when a device wait gave up.
+template <typename T>
+void chol_sweep(cudaStream_t st, Arena& tmp, const std::vector<Win>& wins, Win* wins_d, T* buf, T* dinv, T* dv16,
+                int* info, int* err, bool tc) {
+  if (wins.empty()) return;
+  if constexpr (std::is_same<T, double>::value) {
+    sweep_fp64(st, tmp, wins, wins_d, buf, dinv, dv16, info, err);
+  } else {
+    int maxpan = 0, maxrt = 0, maxrows = 0;
+    for (const Win& w : wins) {
+      maxpan = std::max(maxpan, w.npad / TB);
+      maxrt = std::max(maxrt, (w.rows + TB - 1) / TB);
+      maxrows = std::max(maxrows, w.rows);
+    }
+    const unsigned nw = (unsigned)wins.size();
+    constexpr int SP = 256, HP = 128;
+    for (int kp = 0; kp < maxpan; ++kp) {
+      const int k0 = kp * TB;
+      if (tc) {
+        // columns [0, kb) of super-panel [kb, kb + 256) come from the 256-wide
+        // update, [kb, kh) of its second half from the 128-wide one, and the
+        // 64-wide panel step adds [kh, k0) (at most 64 columns)
+        const int kb = (k0 / SP) * SP, kh = (k0 / HP) * HP;
+        if (k0 == kb && kb > 0) {
+          const unsigned gy = (unsigned)((maxrows - kb + 127) / 128);
+          launch_pdl("k_chol_wide", k_chol_wide<256>, dim3(nw, gy), tc::kWsThreads, wide_smem<256>(), st, wins_d,
+                     (float*)buf, kb, 0, err);
+        }
+        if (k0 == kh && kh > kb) {
+          const unsigned gy = (unsigned)((maxrows - kh + 127) / 128);
+          launch_pdl("k_chol_mid", k_chol_wide<128>, dim3(nw, gy), tc::kWsThreads, wide_smem<128>(), st, wins_d,
+                     (float*)buf, kh, kb, err);
+        }
+        // every panel: its diagonal block (the first panel of a 128-column
+        // group has every column to its left applied; the second adds the
+        // first's 64 columns), then the persistent kernel updates the rows
+        // below with the same columns and solves them
+        launch_pdl("k_chol_step_tc", k_chol_step_tc, dim3(nw, 1), 256, tc_chol_smem(), st, wins_d, (float*)buf,
+                   (float*)dinv, info, kp, kh, err);
+        if (maxrows - (kp + 1) * TB > 0) {
+          const int ntile = (maxrows - (kp + 1) * TB + 127) / 128;
+          launch_pdl("k_chol_panel_pt", k_chol_panel_pt, persistent_grid((size_t)ntile * nw), tc::kPtThreads,
+                     pt_smem(), st, wins_d, (int)nw, (float*)buf, (const float*)dinv, kp, kh, ntile, err);
+        }
+      } else {
+        launch("k_chol_step", k_chol_step<T>, dim3(maxrt - kp, nw), NT, sizeof(CholSmem<T>), st, wins_d, buf, dinv,
+               info, kp);
+        if (maxrt - kp - 1 > 0)
+          launch("k_chol_trsm", k_chol_trsm<T>, dim3(maxrt - kp - 1, nw), NT, sizeof(TrsmSmem<T>), st, wins_d, buf,
+                 dinv, kp, 0);
+      }
+    }
   }
 }
 
@@ -656,7 +727,7 @@ void Impl<T>::fit_local(ModelCore& mc, const lma_problem* P, const lma_hyper* H,
   try {
     const double *X_d, *y_d;
     prepare(mc, P, H, tmp, &X_d, &y_d);
-    const bool batched = (mc.prec == LMA_MIXED);
+    const bool mixed = (mc.prec == LMA_MIXED);
     const int64_t n = mc.n, s = mc.s;
     const int d = (int)mc.d;
     T* rT = tmp.alloc<T>(n);
@@ -687,7 +758,7 @@ void Impl<T>::fit_local(ModelCore& mc, const lma_problem* P, const lma_hyper* H,
     const T* Vt = (const T*)mc.Vt;
     const T* xsT = (const T*)mc.xsT;
     const unsigned et = nblk(s + 1, TB);
-    if (batched && sizeof(T) == 4 && use_tensor_cores()) {
+    if (mixed && sizeof(T) == 4 && use_tensor_cores()) {
       // residual tiles on the tensor cores (bf16x6 products), fed by TMA from
       // the three bfloat16 planes of V (row length padded to 64) in reversed
       // point order
@@ -727,21 +798,16 @@ void Impl<T>::fit_local(ModelCore& mc, const lma_problem* P, const lma_hyper* H,
       }
       launch("k_fill_ext", k_fill_ext4, dim3(maxnt, (unsigned)((s + 63) / 64 + 1), (unsigned)M), 256, 0, st,
              (const Win*)wd, (const float*)Vt, (const float*)rT, (int)s, (float*)wbuf);
-    } else if (batched) {
+    } else {
       launch("k_resid", k_resid<T>, dim3(maxnt * (maxnt + 1) / 2, (unsigned)M), NT, 0, st, wd, xsT, d, Vt, (int)s, (T)mc.ss2,
                                                                           (T)mc.sn2, wbuf);
       launch("k_fill_ext", k_fill_ext<T>, dim3(maxnt, et, (unsigned)M), NT, 0, st, wd, Vt, rT, (int)s, wbuf);
-    } else {
-      for (int64_t m = 0; m < M; ++m) {
-        const int nt = mc.wins[m].npad / TB;
-        launch("k_resid", k_resid<T>, dim3(nt * (nt + 1) / 2, 1), NT, 0, st, wd + m, xsT, d, Vt, (int)s, (T)mc.ss2, (T)mc.sn2,
-                                                               wbuf);
-        launch("k_fill_ext", k_fill_ext<T>, dim3(nt, et, 1), NT, 0, st, wd + m, Vt, rT, (int)s, wbuf);
-      }
     }
-    int* tc_err = (batched && sizeof(T) == 4 && use_tensor_cores()) ? mc.flags + 2 : nullptr;
+    int* tc_err = (mixed && sizeof(T) == 4 && use_tensor_cores()) ? mc.flags + 2 : nullptr;
     if (ft) fused_rhs(mc, *ft, tmp);
-    chol_sweep<T>(st, mc.wins, wd, wbuf, dinv, info, batched, tc_err);
+    if (sizeof(T) == 8) mc.dv16 = mc.keep.alloc<double>(dinve / 4);
+    chol_sweep<T>(st, tmp, mc.wins, wd, wbuf, dinv, (T*)mc.dv16, info, tc_err ? tc_err : mc.flags + 3,
+                  tc_err != nullptr);
     // Gram of the local summaries of the owned windows, reduced in a fixed order
     const int se = (int)s + 1;
     const int nte = (se + TB - 1) / TB;
@@ -1101,8 +1167,8 @@ void Impl<T>::predict(const ModelCore& mc, int64_t U, const double* XU, const in
     const T* wbuf = (const T*)mc.wbuf;
     if (ft) {
       // the right-hand sides were appended to the windows and solved by the fit's sweep
-    } else if (mc.prec == LMA_MIXED) {
-      const bool tc = (sizeof(T) == 4 && use_tensor_cores());
+    } else if constexpr (sizeof(T) == 4) {
+      const bool tc = use_tensor_cores();
       if (tc) {
         // right-hand sides on the tensor cores (bf16x6 products), fed by TMA
         // from the bfloat16 planes of Vu (test order) and of Vt (reversed
@@ -1142,19 +1208,15 @@ void Impl<T>::predict(const ModelCore& mc, int64_t U, const double* XU, const in
                mc.wins_d, wbuf, (const T*)mc.dinv, Pbuf);
       }
     } else {
-      // plain form: one pair per launch
-      size_t a = 0, b = 0;
-      for (size_t pi = 0; pi < pairs.size(); ++pi) {
-        size_t a1 = a, b1 = b;
-        while (a1 < it_rhs.size() && it_rhs[a1].x == (int)pi) ++a1;
-        while (b1 < it_sw.size() && it_sw[b1].x == (int)pi) ++b1;
-        launch("k_pred_rhs", k_pred_rhs<T>, (unsigned)(a1 - a), NT, 0, st, pd, ird + a, mc.wins_d, xs, xu, d, Vt, Vu, (int)s,
-                                                         (T)mc.ss2, Pbuf);
-        launch("k_pred_sweep", k_pred_sweep<T>, (unsigned)(b1 - b), NT, sizeof(CholSmem<T>), st, pd, isd + b, mc.wins_d, wbuf,
-                                                                            (const T*)mc.dinv, Pbuf);
-        a = a1;
-        b = b1;
-      }
+      launch("k_pred_rhs", k_pred_rhs<T>, (unsigned)it_rhs.size(), NT, 0, st, pd, ird, mc.wins_d, xs, xu, d, Vt, Vu, (int)s,
+             (T)mc.ss2, Pbuf);
+      std::vector<int2> it16;
+      for (size_t pi = 0; pi < pairs.size(); ++pi)
+        for (int ut = 0; ut < (pairs[pi].nu + f64::TS - 1) / f64::TS; ++ut) it16.push_back(make_int2((int)pi, ut));
+      int2* i16 = tmp.alloc<int2>(it16.size());
+      stage_copy(i16, it16.data(), sizeof(int2) * it16.size(), st);
+      launch("k_pred_sweep", f64::k_f64_psweep, (unsigned)it16.size(), 128, 0, st, (const Pair*)pd, (const int2*)i16,
+             (const Win*)mc.wins_d, (const double*)wbuf, (const double*)mc.dv16, (double*)Pbuf);
     }
     T* h = tmp.alloc<T>(U * s);
     if (mc.prec == LMA_MIXED && sizeof(T) == 4 && use_tensor_cores()) {

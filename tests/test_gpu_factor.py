@@ -49,3 +49,16 @@ def test_diagonal_blocks_at_tile_edges(L, sizes):
     p = make_random_problem(7, sizes, d=2, s=min(20, sum(sizes)), B=1, test_sizes=(3, 4, 5))
     em, ev, el = _errors(L, p, L.MIXED)
     assert em <= 1e-4 and ev <= 6e-4 and el <= 1.5e-4, (em, ev, el)
+
+
+@pytest.mark.parametrize("sizes, s, B", [((1, 1, 1, 1), 3, 3), ((15, 17, 1, 16, 33), 18, 2), ([5 + k % 13 for k in range(71)], 9, 3),
+                                         ((70, 200, 30, 90), 40, 1)])
+def test_fp64_windows_at_tile_edges(L, sizes, s, B):
+    """Windows of one point up to seventeen 16-column panels, more windows than one launch and than its chains take,
+    test blocks of no, one and more than 16 points; the gradient reads the 64-wide inverses."""
+    test_sizes = [(0, 1, 17, 5)[k % 4] for k in range(len(sizes))]
+    p = make_random_problem(11, sizes, d=3, s=s, B=B, test_sizes=test_sizes)
+    em, ev, el = _errors(L, p, L.FP64)
+    assert em <= 1e-9 and ev <= 1e-9 and el <= 1e-9, (em, ev, el)
+    _, g = L.lma_loglik_grad(precision=L.FP64, **L.problem_args(p))
+    assert _rel(g, O2.loglik_grad(p)[1]) <= 1e-9

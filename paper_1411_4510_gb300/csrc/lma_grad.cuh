@@ -31,6 +31,14 @@ struct GWin {
   int pad_;
 };
 
+// One past the last column that right-hand-side rows [lo, hi] of a window (see GWin) reach: the zeroed copies end
+// at the blanket, unit row t at column nB + t, and a backward solve fills columns to the left only.
+__device__ __forceinline__ int rhs_columns(const Win& w, int s, int lo, int hi) {
+  if (lo <= s) return w.n;
+  if (hi <= 2 * s + 1) return w.nB;
+  return w.nB + (hi - (2 * s + 2)) + 1;
+}
+
 // rows 1+i and s+2+i: sum_{k<=i} Lc^-1[i][k] X_{1+k}[c]  (LcT[k][i] = Lc^-1[i][k])
 template <typename T>
 __global__ void __launch_bounds__(NT) k_grad_rhs(const Win* __restrict__ wins, const GWin* __restrict__ gw,
@@ -90,7 +98,7 @@ __global__ void k_grad_rhs_fill(const Win* __restrict__ wins, const GWin* __rest
 template <typename T>
 __global__ void __launch_bounds__(NT) k_bwd_sweep(const int2* __restrict__ items, const Win* __restrict__ wins,
                                                   const GWin* __restrict__ gw, const T* __restrict__ buf,
-                                                  const T* __restrict__ dinv, T* __restrict__ Q) {
+                                                  const T* __restrict__ dinv, int s, T* __restrict__ Q) {
   const int2 it = items[blockIdx.x];
   const Win w = wins[it.x];
   const GWin g = gw[it.x];
@@ -102,14 +110,14 @@ __global__ void __launch_bounds__(NT) k_bwd_sweep(const int2* __restrict__ items
   T* Qw = Q + g.q;
   const int nr = g.nrows;
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  const int npan = w.npad / TB;
+  const int npan = (rhs_columns(w, s, u0, min(u0 + TB, nr) - 1) + TB - 1) / TB;  // zero to the right of these
   for (int kp = npan - 1; kp >= 0; --kp) {
     const int k0 = kp * TB;
     const int t0 = k0 + TB;
     T acc[4][4] = {};
     auto fa = [&](int r, int k) -> T { return (u0 + r < nr) ? Qw[(int64_t)(u0 + r) * ld + t0 + k] : T(0); };
     auto fb = [&](int r, int k) -> T { return L[(int64_t)(t0 + k) * ld + k0 + r]; };
-    tile_mma<T, true, false>(acc, w.npad - t0, sm.g, fa, fb);
+    tile_mma<T, true, false>(acc, npan * TB - t0, sm.g, fa, fb);
 #pragma unroll
     for (int a = 0; a < 4; ++a)
 #pragma unroll
@@ -176,17 +184,18 @@ __global__ void __launch_bounds__(NT) k_grad_G(const int2* __restrict__ items, c
     auto fb = [&](int r, int k) -> T { return Qw[(int64_t)k * ld + c0 + r]; };
     tile_mma<T, false, false>(acc, s + 1, sm, fa, fb);
   }
-  {
+  if (r0 < w.nB) {  // the zeroed copies have no columns past the blanket
     const T* P = Qw + (int64_t)(s + 1) * ld;
     auto fa = [&](int r, int k) -> T { return P[(int64_t)k * ld + r0 + r]; };
     auto fb = [&](int r, int k) -> T { return -P[(int64_t)k * ld + c0 + r]; };
     tile_mma<T, false, false>(acc, s + 1, sm, fa, fb);
   }
-  {
-    const T* P = Qw + (int64_t)(2 * s + 2) * ld;
+  const int t0 = max(0, r0 - w.nB) / KS * KS;  // unit rows before it end left of this tile's rows
+  if (t0 < b) {
+    const T* P = Qw + (int64_t)(2 * s + 2 + t0) * ld;
     auto fa = [&](int r, int k) -> T { return P[(int64_t)k * ld + r0 + r]; };
     auto fb = [&](int r, int k) -> T { return -P[(int64_t)k * ld + c0 + r]; };
-    tile_mma<T, false, false>(acc, b, sm, fa, fb);
+    tile_mma<T, false, false>(acc, b - t0, sm, fa, fb);
   }
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
   const double wgt = (I == J) ? 1.0 : 2.0;
@@ -385,17 +394,30 @@ __global__ void __launch_bounds__(NT) k_grad_kds(const T* __restrict__ VbT, cons
   if (threadIdx.x == 0) P[d + 1] = 0.0;
 }
 
-// M1 = Vt-bar^T Vt (s x s) by chunks of rows p; FP64 partials per chunk.
+// Rows [q0, q0 + K) of the pieces that the sum over points of M1 is cut into: `nch` chunks of `chunk` rows, each
+// in pieces of `len` rows (the last ones shorter).
+struct Pieces {
+  int64_t n, chunk, len;
+  int per;  // pieces per chunk
+  __device__ __forceinline__ int get(int piece, int64_t& q0) const {
+    const int64_t pb = (piece / per) * chunk;
+    q0 = pb + (piece % per) * len;
+    const int64_t e = min(min(n, pb + chunk), q0 + len);
+    return e > q0 ? (int)(e - q0) : 0;
+  }
+};
+
+// M1 = Vt-bar^T Vt (s x s): each piece is summed in T, the pieces of slice z = blockIdx.z in FP64 into its partial.
 template <typename T>
 __global__ void __launch_bounds__(NT) k_grad_m1(const T* __restrict__ VbT, const T* __restrict__ Vt, int64_t n,
-                                                int s, int64_t chunk, double* __restrict__ partial) {
+                                                int s, Pieces pc, int npieces, int per_slice,
+                                                double* __restrict__ partial) {
   __shared__ GemmSmem<T> sm;
   const int i0 = blockIdx.y * TB, j0 = blockIdx.x * TB;
-  const int64_t pb = blockIdx.z * chunk;
-  const int64_t pe = min(n, pb + chunk);
   double accd[4][4] = {};
-  for (int64_t q0 = pb; q0 < pe; q0 += 1024) {
-    const int K = (int)min((int64_t)1024, pe - q0);
+  for (int p = blockIdx.z * per_slice; p < min(npieces, (int)(blockIdx.z + 1) * per_slice); ++p) {
+    int64_t q0;
+    const int K = pc.get(p, q0);
     T acc[4][4] = {};
     auto fa = [&](int r, int k) -> T { return (i0 + r < s) ? VbT[(int64_t)(i0 + r) * n + q0 + k] : T(0); };
     auto fb = [&](int r, int k) -> T { return (j0 + r < s) ? Vt[(q0 + k) * s + j0 + r] : T(0); };
@@ -416,6 +438,275 @@ __global__ void __launch_bounds__(NT) k_grad_m1(const T* __restrict__ VbT, const
     }
 }
 
+// ---------------------------------------------------------------------------
+// FP32 forms of the N x s products with 128 x 128 tiles and 8 x 8 values a thread
+// (the 64 x 64 tiles above read shared memory for every second FMA: 11-15 TFLOP/s at
+// N = 65,536, s = 1,024, M1 12.3 ms and Vt-bar 4.6; these 33-37, 3.7 and 2.1 ms).
+// One FMA per term, k ascending, as there.
+
+constexpr int GK = 8;  // K step
+struct Smem128 {
+  float a[2][GK][132], b[2][GK][132];
+};
+
+// Four consecutive floats at p, at most lim of them valid (the rest zero).
+__device__ __forceinline__ float4 grad_load4(const float* p, int lim) {
+  if (lim >= 4 && (reinterpret_cast<uintptr_t>(p) & 15u) == 0) return *reinterpret_cast<const float4*>(p);
+  return make_float4(lim > 0 ? p[0] : 0.f, lim > 1 ? p[1] : 0.f, lim > 2 ? p[2] : 0.f, lim > 3 ? p[3] : 0.f);
+}
+
+// acc[x][y] += sum_{k<K} A[r][k] B[k][c] for r = 4 ty + 64 (x / 4) + x % 4, c = 4 tx + 64 (y / 4) + y % 4 (256
+// threads, tx = tid % 16, ty = tid / 16); A: mlim rows of lda, B: rows of ldb with nlim columns.
+__device__ __forceinline__ void mma128(float (&acc)[8][8], Smem128& sm, const float* A, int64_t lda, int64_t mlim,
+                                       const float* B, int64_t ldb, int64_t nlim, int K) {
+  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+  const int ar = tid >> 1, ak = (tid & 1) * 4, br = tid >> 5, bc = (tid & 31) * 4;
+  const int blim = (int)min((int64_t)4, max((int64_t)0, nlim - bc));
+  float4 a, b;
+  auto load = [&](int k0) {
+    a = ar < mlim ? grad_load4(A + (int64_t)ar * lda + k0 + ak, min(4, K - k0 - ak)) : make_float4(0.f, 0.f, 0.f, 0.f);
+    b = k0 + br < K ? grad_load4(B + (int64_t)(k0 + br) * ldb + bc, blim) : make_float4(0.f, 0.f, 0.f, 0.f);
+  };
+  auto stash = [&](int s) {
+    sm.a[s][ak][ar] = a.x;
+    sm.a[s][ak + 1][ar] = a.y;
+    sm.a[s][ak + 2][ar] = a.z;
+    sm.a[s][ak + 3][ar] = a.w;
+    *reinterpret_cast<float4*>(&sm.b[s][br][bc]) = b;
+  };
+  if (K <= 0) return;
+  load(0);
+  __syncthreads();
+  stash(0);
+  __syncthreads();
+  int cur = 0;
+  for (int k0 = 0; k0 < K; k0 += GK) {
+    const bool more = k0 + GK < K;
+    if (more) load(k0 + GK);
+#pragma unroll
+    for (int kk = 0; kk < GK; ++kk) {
+      const float4 a0 = *reinterpret_cast<const float4*>(&sm.a[cur][kk][4 * ty]);
+      const float4 a1 = *reinterpret_cast<const float4*>(&sm.a[cur][kk][64 + 4 * ty]);
+      const float4 b0 = *reinterpret_cast<const float4*>(&sm.b[cur][kk][4 * tx]);
+      const float4 b1 = *reinterpret_cast<const float4*>(&sm.b[cur][kk][64 + 4 * tx]);
+      const float ra[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
+      const float rb[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
+#pragma unroll
+      for (int x = 0; x < 8; ++x)
+#pragma unroll
+        for (int y = 0; y < 8; ++y) acc[x][y] = fmaf(ra[x], rb[y], acc[x][y]);
+    }
+    if (more) {
+      stash(cur ^ 1);
+      __syncthreads();
+      cur ^= 1;
+    }
+  }
+}
+__device__ __forceinline__ int row128(int x) { return 4 * (int)(threadIdx.x >> 4) + 64 * (x >> 2) + (x & 3); }
+__device__ __forceinline__ int col128(int y) { return 4 * (int)(threadIdx.x & 15) + 64 * (y >> 2) + (y & 3); }
+
+__global__ void __launch_bounds__(256) k_grad_m1_128(const float* __restrict__ VbT, const float* __restrict__ Vt,
+                                                     int64_t n, int s, Pieces pc, int npieces, int per_slice,
+                                                     double* __restrict__ partial) {
+  __shared__ __align__(16) Smem128 sm;
+  const int i0 = blockIdx.y * 128, j0 = blockIdx.x * 128;
+  double* P = partial + (int64_t)blockIdx.z * s * s;
+  bool first = true;
+  for (int p = blockIdx.z * per_slice; p < min(npieces, (int)(blockIdx.z + 1) * per_slice); ++p) {
+    int64_t q0;
+    const int K = pc.get(p, q0);
+    float acc[8][8];
+#pragma unroll
+    for (int x = 0; x < 8; ++x)
+#pragma unroll
+      for (int y = 0; y < 8; ++y) acc[x][y] = 0.f;
+    mma128(acc, sm, VbT + (int64_t)i0 * n + q0, n, s - i0, Vt + q0 * s + j0, s, s - j0, K);
+#pragma unroll
+    for (int x = 0; x < 8; ++x)
+#pragma unroll
+      for (int y = 0; y < 8; ++y) {
+        const int i = i0 + row128(x), j = j0 + col128(y);
+        if (i < s && j < s) {
+          double* o = P + (int64_t)i * s + j;  // the slice's FP64 sum stays in the partial (no room in registers)
+          *o = first ? (double)acc[x][y] : *o + (double)acc[x][y];
+        }
+      }
+    first = false;
+  }
+}
+
+// k_grad_vbar with 128 x 128 tiles (grid: x over points, y over support coordinates).
+__global__ void __launch_bounds__(256) k_grad_vbar_128(const float* __restrict__ PsiT, const float* __restrict__ GVT,
+                                                       const float* __restrict__ LcT, const double* __restrict__ beta,
+                                                       int64_t n, int s, float* __restrict__ VbT) {
+  __shared__ __align__(16) Smem128 sm;
+  const int k0 = blockIdx.y * 128;
+  const int64_t p0 = (int64_t)blockIdx.x * 128;
+  float acc[8][8];
+#pragma unroll
+  for (int x = 0; x < 8; ++x)
+#pragma unroll
+    for (int y = 0; y < 8; ++y) acc[x][y] = 0.f;
+  mma128(acc, sm, LcT + (int64_t)k0 * s + k0, s, s - k0, PsiT + (int64_t)(1 + k0) * n + p0, n, n - p0, s - k0);
+#pragma unroll
+  for (int x = 0; x < 8; ++x)
+#pragma unroll
+    for (int y = 0; y < 8; ++y) {
+      const int k = k0 + row128(x);
+      const int64_t p = p0 + col128(y);
+      if (k < s && p < n)
+        VbT[(int64_t)k * n + p] = (float)(beta[k] * (double)PsiT[p]) - acc[x][y] - 2.f * GVT[(int64_t)k * n + p];
+    }
+}
+
+// Numbers held as the sum of two floats (48 bits): an FP64 instruction occupies a
+// scheduler for 64 clocks, a float one for one, so where FP64 is more than the result
+// needs but a float is less, sums and products of pairs are 5 to 10 times cheaper.
+struct Pair2 {
+  float h, l;
+};
+__device__ __forceinline__ Pair2 quick2(float a, float b) {  // |a| >= |b|
+  const float s = __fadd_rn(a, b);
+  return {s, __fsub_rn(b, __fsub_rn(s, a))};
+}
+__device__ __forceinline__ Pair2 sum2(float a, float b) {  // exact
+  const float s = __fadd_rn(a, b), t = __fsub_rn(s, a);
+  return {s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t))};
+}
+__device__ __forceinline__ Pair2 add2(Pair2 a, Pair2 b) {
+  const Pair2 s = sum2(a.h, b.h);
+  return quick2(s.h, __fadd_rn(s.l, __fadd_rn(a.l, b.l)));
+}
+__device__ __forceinline__ Pair2 mul2(Pair2 a, Pair2 b) {
+  const float p = __fmul_rn(a.h, b.h);
+  float e = __fmaf_rn(a.h, b.h, -p);
+  e = __fmaf_rn(a.h, b.l, e);
+  e = __fmaf_rn(a.l, b.h, e);
+  return quick2(p, e);
+}
+__device__ __forceinline__ Pair2 scale2(Pair2 a, float b) {
+  const float p = __fmul_rn(a.h, b);
+  return quick2(p, __fmaf_rn(a.l, b, __fmaf_rn(a.h, b, -p)));
+}
+__device__ __forceinline__ Pair2 split2(double x) {
+  const float h = (float)x;
+  return {h, (float)(x - (double)h)};
+}
+
+// exp(y) for y <= 0 to about 1e-11 relative (0 below 2^-125): y = n ln 2 + r with ln 2 in three parts (n times the
+// first is exact), then the Taylor series of exp(r), its terms from r^5 on in single precision (at most 4e-5 of the sum).
+__device__ __forceinline__ Pair2 exp2f_pair(Pair2 y) {
+  const float n = rintf(y.h * 1.44269504f);
+  Pair2 r = sum2(y.h, -0.693359375f * n);
+  const float q = __fmul_rn(n, 2.12194442e-4f);  // 0.693359375 - ln 2 = 2.12194440054690583e-4
+  const float e = __fmaf_rn(n, 2.12194442e-4f, -q);
+  r = add2(r, Pair2{q, __fadd_rn(e, __fmaf_rn(n, -1.64657177e-12f, y.l))});
+  const float x = r.h;
+  float t = 1.f / 39916800.f;
+  t = fmaf(t, x, 1.f / 3628800.f);
+  t = fmaf(t, x, 1.f / 362880.f);
+  t = fmaf(t, x, 1.f / 40320.f);
+  t = fmaf(t, x, 1.f / 5040.f);
+  t = fmaf(t, x, 1.f / 720.f);
+  t = fmaf(t, x, 1.f / 120.f);
+  Pair2 v = add2(Pair2{0.0416666679f, -1.24176348e-9f}, scale2(r, t));  // 1/24
+  v = add2(Pair2{0.166666672f, -4.96705388e-9f}, mul2(r, v));           // 1/6
+  v = add2(Pair2{0.5f, 0.f}, mul2(r, v));
+  v = add2(Pair2{1.f, 0.f}, mul2(r, v));
+  v = add2(Pair2{1.f, 0.f}, mul2(r, v));
+  const float sc = n < -125.f ? 0.f : __int_as_float(((int)n + 127) << 23);
+  return {v.h * sc, v.l * sc};
+}
+
+// k_grad_kds in FP32 with pairs of floats in place of its FP64 epilogue (12.8 -> 2.8 ms at N = 65,536, s = 1,024,
+// d = 8; the gradient moves by 1e-12): tiles of TS2 x TS2 (128 or, for small problems, 64), the product parked in shared memory, then a
+// thread takes one point and every (256 / TS2)-th support coordinate.  D: d padded with zero coordinates.
+template <int TS2, int D>
+__global__ void __launch_bounds__(256) k_grad_kds_pair(const float* __restrict__ VbT, const float* __restrict__ ET,
+                                                       const float* __restrict__ xs, const float* __restrict__ ss,
+                                                       int d, int64_t n, int s, double ss2,
+                                                       double* __restrict__ partial) {
+  extern __shared__ __align__(16) unsigned char smraw[];
+  float* prod = reinterpret_cast<float*>(smraw);                       // [TS2][TS2 + 1]
+  float(*xk)[D] = reinterpret_cast<float(*)[D]>(prod + TS2 * (TS2 + 4));  // [TS2][D]
+  __shared__ double red[8][D + 1];
+  const int k0 = blockIdx.y * TS2;
+  const int64_t p0 = (int64_t)blockIdx.x * TS2;
+  for (int e = threadIdx.x; e < TS2 * D; e += 256) {
+    const int r = e / D, q = e % D;
+    xk[r][q] = (k0 + r < s && q < d) ? ss[(int64_t)(k0 + r) * d + q] : 0.f;
+  }
+  if constexpr (TS2 == 128) {
+    Smem128& sm = *reinterpret_cast<Smem128*>(smraw);
+    float acc[8][8];
+#pragma unroll
+    for (int x = 0; x < 8; ++x)
+#pragma unroll
+      for (int y = 0; y < 8; ++y) acc[x][y] = 0.f;
+    mma128(acc, sm, ET + (int64_t)k0 * s + k0, s, s - k0, VbT + (int64_t)k0 * n + p0, n, n - p0, s - k0);
+    __syncthreads();
+#pragma unroll
+    for (int x = 0; x < 8; ++x)
+#pragma unroll
+      for (int y = 0; y < 8; ++y) prod[row128(x) * (TS2 + 1) + col128(y)] = acc[x][y];
+  } else {
+    GemmSmem<float>& sm = *reinterpret_cast<GemmSmem<float>*>(smraw);
+    float acc[4][4] = {};
+    auto fa = [&](int r, int ii) -> float { return (k0 + r < s) ? ET[(int64_t)(k0 + r) * s + k0 + ii] : 0.f; };
+    auto fb = [&](int r, int ii) -> float { return (p0 + r < n) ? VbT[(int64_t)(k0 + ii) * n + p0 + r] : 0.f; };
+    tile_mma<float, true, false>(acc, s - k0, sm, fa, fb);
+    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+      for (int b = 0; b < 4; ++b) prod[(ty + 16 * a) * (TS2 + 1) + tx + 16 * b] = acc[a][b];
+  }
+  __syncthreads();
+  const int pc = threadIdx.x % TS2;
+  const int64_t p = p0 + pc;
+  float xp[D];
+#pragma unroll
+  for (int q = 0; q < D; ++q) xp[q] = (p < n && q < d) ? xs[p * d + q] : 0.f;
+  Pair2 gl[D], gs{0.f, 0.f};
+#pragma unroll
+  for (int q = 0; q < D; ++q) gl[q] = {0.f, 0.f};
+  if (p < n)
+    for (int kr = threadIdx.x / TS2; kr < min(TS2, s - k0); kr += 256 / TS2) {
+      Pair2 d2{0.f, 0.f};
+#pragma unroll
+      for (int q = 0; q < D; ++q) {
+        const Pair2 t = sum2(xk[kr][q], -xp[q]);
+        d2 = add2(d2, mul2(t, t));
+      }
+      const Pair2 kg = scale2(exp2f_pair(Pair2{-0.5f * d2.h, -0.5f * d2.l}), prod[kr * (TS2 + 1) + pc]);
+      gs = add2(gs, kg);
+#pragma unroll
+      for (int q = 0; q < D; ++q) {
+        const Pair2 t = sum2(xk[kr][q], -xp[q]);
+        gl[q] = add2(gl[q], mul2(kg, mul2(t, t)));
+      }
+    }
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+#pragma unroll
+  for (int q = 0; q < D + 1; ++q) {
+    Pair2 v = q < D ? gl[q < D ? q : 0] : gs;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+      v = add2(v, Pair2{__shfl_xor_sync(0xffffffffu, v.h, o), __shfl_xor_sync(0xffffffffu, v.l, o)});
+    if (lane == 0) red[warp][q] = (double)v.h + (double)v.l;
+  }
+  __syncthreads();
+  double* P = partial + ((int64_t)blockIdx.y * gridDim.x + blockIdx.x) * (d + 2);
+  if (threadIdx.x <= d) {
+    const int q = threadIdx.x < d ? threadIdx.x : D;
+    double v = 0.0;
+    for (int k = 0; k < 8; ++k) v += red[k][q];
+    P[threadIdx.x] = v * (threadIdx.x < d ? ss2 : 2.0 * ss2);
+  }
+  if (threadIdx.x == d + 1) P[d + 1] = 0.0;
+}
+
 __global__ void k_sum_chunks(const double* __restrict__ partial, int nchunk, int64_t len, double* __restrict__ out) {
   int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (e >= len) return;
@@ -424,29 +715,57 @@ __global__ void k_sum_chunks(const double* __restrict__ partial, int nchunk, int
   out[e] = v;
 }
 
-// Dense FP64 product C = alpha op(A) op(B) (s x s, row-major, leading dims lda/ldb/ldc).
-template <bool TA, bool TBm>
-__global__ void __launch_bounds__(NT) k_dgemm(const double* __restrict__ A, int64_t lda, const double* __restrict__ Bm,
-                                              int64_t ldb, double* __restrict__ C, int64_t ldc, int s, double alpha) {
-  __shared__ GemmSmem<double> sm;
-  const int i0 = blockIdx.y * TB, j0 = blockIdx.x * TB;
-  double acc[4][4] = {};
-  auto fa = [&](int r, int k) -> double {
-    int i = i0 + r;
-    return i < s ? (TA ? A[(int64_t)k * lda + i] : A[(int64_t)i * lda + k]) : 0.0;
-  };
-  auto fb = [&](int r, int k) -> double {
-    int j = j0 + r;
-    return j < s ? (TBm ? Bm[(int64_t)j * ldb + k] : Bm[(int64_t)k * ldb + j]) : 0.0;
-  };
-  tile_mma<double, !TA, TBm>(acc, s, sm, fa, fb);
+// Dense FP64 product C = alpha op(A) op(B) (s x s, row-major, leading dims lda/ldb/ldc) of triangular operands.
+// SHAPE says which terms and results are zero: bit 0: op(A)[i][k] = 0 for k < i; bit 1: op(A)[i][k] = 0 for k > i;
+// bit 2: op(B)[k][j] = 0 for k < j; bit 3: only C's lower triangle is wanted (the rest is left).  TILE x TILE results
+// a CTA of 256 threads: 16 where 32 would leave SMs without a tile (FP64: 16 K clocks a 64-wide tile and K, which
+// made the four products of s = 100 130 us each on four CTAs).
+template <bool TA, bool TBm, int SHAPE, int TILE>
+__global__ void __launch_bounds__(256) k_dgemm(const double* __restrict__ A, int64_t lda, const double* __restrict__ Bm,
+                                               int64_t ldb, double* __restrict__ C, int64_t ldc, int s, double alpha) {
+  constexpr int KT = 16, R = TILE / 16;
+  __shared__ double sa[KT][TILE + 1], sb[KT][TILE + 1];
+  const int i0 = blockIdx.y * TILE, j0 = blockIdx.x * TILE;
+  if ((SHAPE & 8) && j0 > i0 + TILE - 1) return;
+  int kb = 0, ke = s;
+  if (SHAPE & 1) kb = max(kb, i0);
+  if (SHAPE & 4) kb = max(kb, j0);
+  if (SHAPE & 2) ke = min(ke, i0 + TILE);
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+  double acc[R][R] = {};
+  for (int k0 = kb; k0 < ke; k0 += KT) {
+    for (int e = threadIdx.x; e < TILE * KT; e += 256) {
+      const int ra = TA ? e % TILE : e / KT, ka = TA ? e / TILE : e % KT;
+      sa[ka][ra] = (i0 + ra < s && k0 + ka < ke)
+                       ? (TA ? A[(int64_t)(k0 + ka) * lda + i0 + ra] : A[(int64_t)(i0 + ra) * lda + k0 + ka])
+                       : 0.0;
+      const int rb = TBm ? e / KT : e % TILE, kq = TBm ? e % KT : e / TILE;
+      sb[kq][rb] = (j0 + rb < s && k0 + kq < ke)
+                       ? (TBm ? Bm[(int64_t)(j0 + rb) * ldb + k0 + kq] : Bm[(int64_t)(k0 + kq) * ldb + j0 + rb])
+                       : 0.0;
+    }
+    __syncthreads();
 #pragma unroll
-  for (int a = 0; a < 4; ++a)
+    for (int kk = 0; kk < KT; ++kk) {
+      double a[R], b[R];
 #pragma unroll
-    for (int b = 0; b < 4; ++b) {
-      int i = i0 + ty + 16 * a, j = j0 + tx + 16 * b;
-      if (i < s && j < s) C[(int64_t)i * ldc + j] = alpha * acc[a][b];
+      for (int q = 0; q < R; ++q) {
+        a[q] = sa[kk][ty + 16 * q];
+        b[q] = sb[kk][tx + 16 * q];
+      }
+#pragma unroll
+      for (int p = 0; p < R; ++p)
+#pragma unroll
+        for (int q = 0; q < R; ++q) acc[p][q] = fma(a[p], b[q], acc[p][q]);
+    }
+    __syncthreads();
+  }
+#pragma unroll
+  for (int p = 0; p < R; ++p)
+#pragma unroll
+    for (int q = 0; q < R; ++q) {
+      const int i = i0 + ty + 16 * p, j = j0 + tx + 16 * q;
+      if (i < s && j < s) C[(int64_t)i * ldc + j] = alpha * acc[p][q];
     }
 }
 

@@ -110,7 +110,7 @@ __global__ void __launch_bounds__(256, 2) k_grad_rhs_tc(const Win* __restrict__ 
 // items: x = window, y = 128-row tile of the window's right-hand sides.
 __global__ void __launch_bounds__(256, 2) k_bwd_sweep_tc(const int2* __restrict__ items, const Win* __restrict__ wins,
                                                       const GWin* __restrict__ gw, const float* __restrict__ buf,
-                                                      const float* __restrict__ dinv, float* __restrict__ Q,
+                                                      const float* __restrict__ dinv, int s, float* __restrict__ Q,
                                                       int* __restrict__ err) {
   const int2 it = items[blockIdx.x];
   const Win w = wins[it.x];
@@ -129,8 +129,9 @@ __global__ void __launch_bounds__(256, 2) k_bwd_sweep_tc(const int2* __restrict_
   float* myrow = Qw + (int64_t)(u0 + rl) * ld;
   tc::TcPipe pipe;
   bool ok = true;
-  for (int kp = w.npad / TB - 1; kp >= 0 && ok; --kp) {
-    const int k0 = kp * TB, t0 = k0 + TB, K = w.npad - t0;
+  const int npan = (rhs_columns(w, s, u0, min(u0 + 128, nr) - 1) + TB - 1) / TB;  // zero to the right of these
+  for (int kp = npan - 1; kp >= 0 && ok; --kp) {
+    const int k0 = kp * TB, t0 = k0 + TB, K = npan * TB - t0;
     float v[32];
     if (K > 0) {
       auto rowA = [&](int r) -> const float* { return u0 + r < nr ? Qw + (int64_t)(u0 + r) * ld + t0 : nullptr; };
@@ -214,18 +215,20 @@ __global__ void __launch_bounds__(256, 2) k_grad_G_tc(const int4* __restrict__ i
     auto rowB = [&](int k) -> const float* { return k < K ? Qw + (int64_t)k * ld + c0 : nullptr; };
     ok = tc::tile_product2<64, true, true>(sm, pipe, tmem, K, rowA, rowB, alim, 64, false, false);
   }
-  if (ok) {
+  if (ok && r0 < w.nB) {  // the zeroed copies have no columns past the blanket
     const int K = s + 1;
     const float* P = Qw + (int64_t)(s + 1) * ld;
     auto rowA = [&](int k) -> const float* { return k < K ? P + (int64_t)k * ld + r0 : nullptr; };
     auto rowB = [&](int k) -> const float* { return k < K ? P + (int64_t)k * ld + c0 : nullptr; };
     ok = tc::tile_product2<64, true, true>(sm, pipe, tmem, K, rowA, rowB, alim, 64, true, true);
   }
-  if (ok && b > 0) {
-    const float* P = Qw + (int64_t)(2 * s + 2) * ld;
-    auto rowA = [&](int k) -> const float* { return k < b ? P + (int64_t)k * ld + r0 : nullptr; };
-    auto rowB = [&](int k) -> const float* { return k < b ? P + (int64_t)k * ld + c0 : nullptr; };
-    ok = tc::tile_product2<64, true, true>(sm, pipe, tmem, b, rowA, rowB, alim, 64, true, true);
+  const int t0 = max(0, r0 - w.nB) / 32 * 32;  // unit rows before it end left of this tile's rows
+  if (ok && t0 < b) {
+    const float* P = Qw + (int64_t)(2 * s + 2 + t0) * ld;
+    const int K = b - t0;
+    auto rowA = [&](int k) -> const float* { return k < K ? P + (int64_t)k * ld + r0 : nullptr; };
+    auto rowB = [&](int k) -> const float* { return k < K ? P + (int64_t)k * ld + c0 : nullptr; };
+    ok = tc::tile_product2<64, true, true>(sm, pipe, tmem, K, rowA, rowB, alim, 64, true, true);
   }
   if (!ok && threadIdx.x == 0) atomicExch(err, 1);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;

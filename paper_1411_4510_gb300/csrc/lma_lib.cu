@@ -178,6 +178,7 @@ Staging& staging() {
   return s;
 }
 
+static size_t kds_smem(int tile, int dpad);
 static size_t tc_chol_smem() { return sizeof(tc::TcSmem<64>) + tc::kTcAlignSlack; }
 static size_t pt_smem() { return sizeof(tc::PtSmem) + tc::kTcAlignSlack; }
 
@@ -326,6 +327,9 @@ void Impl<T>::setup_attributes() {
     cudaFuncSetAttribute(k_chol_wide<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)wide_smem<256>());
     cudaFuncSetAttribute(k_chol_wide<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)wide_smem<128>());
     cudaFuncSetAttribute(k_proj_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bf6::smem_bytes());
+    cudaFuncSetAttribute(k_grad_kds_pair<128, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kds_smem(128, 8));
+    cudaFuncSetAttribute(k_grad_kds_pair<128, MAXD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)kds_smem(128, MAXD));
     cudaFuncSetAttribute(k_grad_rhs_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc_chol_smem());
     cudaFuncSetAttribute(k_bwd_sweep_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc_chol_smem());
     cudaFuncSetAttribute(k_grad_G_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc_chol_smem());
@@ -1446,6 +1450,21 @@ void Impl<T>::loglik_grad(ModelCore& mc, const lma_problem* P, const lma_hyper* 
   *ll = mc.loglik;
 }
 
+// Dynamic shared memory of k_grad_kds_pair: the product tile (or the operands') and the support coordinates.
+static size_t kds_smem(int tile, int dpad) { return sizeof(float) * ((size_t)tile * (tile + 4) + (size_t)tile * dpad); }
+
+// Sb = L^-T Phi(L^T Lbar) L^-1 with Lbar = -L^-T M1 (the adjoint of the Cholesky factor), Y a scratch matrix.
+template <int TILE>
+static void chol_adjoint(cudaStream_t st, int s, const double* ET64, int64_t npS, const double* M1, const double* Lm,
+                         double* Lbar, double* X, double* Y, double* Sb) {
+  const dim3 gg(nblk(s, TILE), nblk(s, TILE));
+  launch("k_dgemm", k_dgemm<false, false, 1, TILE>, gg, 256, 0, st, ET64, npS, M1, s, Lbar, s, s, -1.0);
+  launch("k_dgemm", k_dgemm<true, false, 1 | 8, TILE>, gg, 256, 0, st, Lm, s, (const double*)Lbar, s, X, s, s, 1.0);
+  launch("k_phi", k_phi, nblk((int64_t)s * s), NT, 0, st, X, s);
+  launch("k_dgemm", k_dgemm<false, true, 2 | 4, TILE>, gg, 256, 0, st, (const double*)X, s, ET64, npS, Y, s, s, 1.0);
+  launch("k_dgemm", k_dgemm<false, false, 1 | 4, TILE>, gg, 256, 0, st, ET64, npS, (const double*)Y, s, Sb, s, s, 1.0);
+}
+
 // The adjoint restricted to windows [k_lo, k_hi) of the model: their
 // G_m terms and the chain of their Vt-bar contributions through K_DS and
 // L_SS.  Every step after the window terms is linear in them, so the parts
@@ -1512,7 +1531,7 @@ void Impl<T>::grad_windows(ModelCore& mc, int64_t k_lo, int64_t k_hi, double* gr
       stage_copy(isw, it_sw.data(), sizeof(int2) * it_sw.size(), st);
       stage_copy(ig, it_g.data(), sizeof(int4) * it_g.size(), st);
       launch("k_bwd_sweep_tc", k_bwd_sweep_tc, dim3((unsigned)it_sw.size()), 256, tc_chol_smem(), st,
-             (const int2*)isw, wk, gwd, (const float*)wbuf, (const float*)mc.dinv, (float*)Q, tc_err);
+             (const int2*)isw, wk, gwd, (const float*)wbuf, (const float*)mc.dinv, si, (float*)Q, tc_err);
       n_g = it_g.size();
       pG = tmp.alloc<double>(n_g * np2);
       launch("k_grad_G_tc", k_grad_G_tc, dim3((unsigned)n_g), 256, tc_chol_smem(), st, (const int4*)ig, wk,
@@ -1536,7 +1555,7 @@ void Impl<T>::grad_windows(ModelCore& mc, int64_t k_lo, int64_t k_hi, double* gr
       stage_copy(isw, it_sw.data(), sizeof(int2) * it_sw.size(), st);
       stage_copy(ig, it_g.data(), sizeof(int2) * it_g.size(), st);
       launch("k_bwd_sweep", k_bwd_sweep<T>, dim3((unsigned)it_sw.size()), NT, sizeof(CholSmem<T>), st, isw,
-             wk, gwd, wbuf, (const T*)mc.dinv, Q);
+             wk, gwd, wbuf, (const T*)mc.dinv, si, Q);
       n_g = it_g.size();
       pG = tmp.alloc<double>(n_g * np2);
       launch("k_grad_G", k_grad_G<T>, dim3((unsigned)n_g), NT, 0, st, ig, wk, gwd, (const T*)Q,
@@ -1552,20 +1571,58 @@ void Impl<T>::grad_windows(ModelCore& mc, int64_t k_lo, int64_t k_hi, double* gr
            bptr_d, (int)mc.M, (int)mc.B, n, si, (const T*)Q, (const T*)GV, PsiT, GVT, (int)mc.w0, (int)k_lo,
            (int)k_hi);
     T* VbT = tmp.alloc<T>(s * n);
-    launch("k_grad_vbar", k_grad_vbar<T>, dim3(nblk(n, TB), nblk(s, TB)), NT, 0, st, (const T*)PsiT,
-           (const T*)GVT, (const T*)mc.LcT, mc.beta, n, si, VbT);
-    const unsigned gx = nblk(n, TB), gy = nblk(s, TB);
+    // N x s products: 128 x 128 tiles in FP32 where there are enough of them for every SM (below, 64 x 64 ones
+    // spread the work: at N = 3,200, s = 100 they are 25 and 100 CTAs)
+    int sms = 0, dev = 0;
+    LMA_CK(cudaGetDevice(&dev));
+    LMA_CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    const bool big = sizeof(T) == 4 && (int64_t)nblk(n, 128) * nblk(s, 128) >= 2 * sms;
+    const unsigned tile = big ? 128 : TB, gx = nblk(n, (int)tile), gy = nblk(s, (int)tile);
+    if constexpr (sizeof(T) == 4) {
+      if (big)
+        launch("k_grad_vbar", k_grad_vbar_128, dim3(gx, gy), 256, 0, st, (const float*)PsiT, (const float*)GVT,
+               (const float*)mc.LcT, (const double*)mc.beta, n, si, VbT);
+    }
+    if (!big)
+      launch("k_grad_vbar", k_grad_vbar<T>, dim3(gx, gy), NT, 0, st, (const T*)PsiT, (const T*)GVT,
+             (const T*)mc.LcT, mc.beta, n, si, VbT);
     double* pK = tmp.alloc<double>((size_t)gx * gy * np2);
-    launch("k_grad_kds", k_grad_kds<T>, dim3(gx, gy), NT, 0, st, (const T*)VbT, (const T*)mc.ET,
-           (const T*)mc.xsT, (const T*)mc.ssT, d, n, si, mc.ss2, pK);
+    if constexpr (sizeof(T) == 4) {
+      const bool d8 = pad_dim(d) == 8;
+      launch("k_grad_kds",
+             big ? (d8 ? k_grad_kds_pair<128, 8> : k_grad_kds_pair<128, MAXD>)
+                 : (d8 ? k_grad_kds_pair<64, 8> : k_grad_kds_pair<64, MAXD>),
+             dim3(gx, gy), 256, kds_smem((int)tile, d8 ? 8 : MAXD), st, (const float*)VbT, (const float*)mc.ET,
+             (const float*)mc.xsT, (const float*)mc.ssT, d, n, si, mc.ss2, pK);
+    } else {
+      launch("k_grad_kds", k_grad_kds<T>, dim3(gx, gy), NT, 0, st, (const T*)VbT, (const T*)mc.ET,
+             (const T*)mc.xsT, (const T*)mc.ssT, d, n, si, mc.ss2, pK);
+    }
     // L_SS-bar = -L_SS^-T (Vt-bar^T Vt) and the Cholesky adjoint, in FP64
+    // M1's sum over the points: FP32 sums run over 1,024 points at most (FP64 ones over 256, for more CTAs), the
+    // pieces are dealt to slices so that every SM has tiles, the slices' FP64 sums are added at the end
+    Pieces pc;
     const int nch = (int)std::min<int64_t>(64, (n + 8191) / 8192);
-    const int64_t chunk = (n + nch - 1) / nch;
-    double* pM = tmp.alloc<double>((size_t)nch * s * s);
-    launch("k_grad_m1", k_grad_m1<T>, dim3(gy, gy, nch), NT, 0, st, (const T*)VbT, (const T*)mc.Vt, n, si, chunk,
-           pM);
+    pc.n = n;
+    pc.chunk = (n + nch - 1) / nch;
+    pc.len = sizeof(T) == 4 ? 1024 : 256;
+    pc.per = (int)((pc.chunk + pc.len - 1) / pc.len);
+    const int npieces = nch * pc.per;
+    const int64_t mt = (int64_t)nblk(s, (int)tile) * nblk(s, (int)tile);
+    int nslice = (int)std::min<int64_t>(npieces, std::max<int64_t>(1, (4 * sms + mt - 1) / mt));
+    const int per_slice = (npieces + nslice - 1) / nslice;
+    nslice = (npieces + per_slice - 1) / per_slice;
+    double* pM = tmp.alloc<double>((size_t)nslice * s * s);
+    if constexpr (sizeof(T) == 4) {
+      if (big)
+        launch("k_grad_m1", k_grad_m1_128, dim3(nblk(s, 128), nblk(s, 128), nslice), 256, 0, st, (const float*)VbT,
+               (const float*)mc.Vt, n, si, pc, npieces, per_slice, pM);
+    }
+    if (!big)
+      launch("k_grad_m1", k_grad_m1<T>, dim3(nblk(s, TB), nblk(s, TB), nslice), NT, 0, st, (const T*)VbT,
+             (const T*)mc.Vt, n, si, pc, npieces, per_slice, pM);
     double* M1 = tmp.alloc<double>(s * s);
-    launch("k_sum_chunks", k_sum_chunks, nblk(s * s), NT, 0, st, (const double*)pM, nch, (int64_t)(s * s), M1);
+    launch("k_sum_chunks", k_sum_chunks, nblk(s * s), NT, 0, st, (const double*)pM, nslice, (int64_t)(s * s), M1);
     const double* ET64 = mc.kss + (int64_t)mc.npS * mc.npS;
     double* Lm = tmp.alloc<double>(s * s);   // L_SS with its upper triangle zeroed
     launch("k_copy_block", k_copy_block<double>, nblk(s * s), NT, 0, st, (const double*)mc.kss, (int64_t)mc.npS,
@@ -1576,16 +1633,12 @@ void Impl<T>::grad_windows(ModelCore& mc, int64_t k_lo, int64_t k_hi, double* gr
     double* X = tmp.alloc<double>(s * s);
     double* Y = tmp.alloc<double>(s * s);
     double* Sb = tmp.alloc<double>(s * s);
-    const dim3 gg(gy, gy);
-    launch("k_dgemm", k_dgemm<false, false>, gg, NT, 0, st, ET64, (int64_t)mc.npS, (const double*)M1, s, Lbar, s,
-           si, -1.0);
-    launch("k_dgemm", k_dgemm<true, false>, gg, NT, 0, st, (const double*)Lm, s, (const double*)Lbar, s, X, s, si,
-           1.0);
-    launch("k_phi", k_phi, nblk(s * s), NT, 0, st, X, si);
-    launch("k_dgemm", k_dgemm<false, true>, gg, NT, 0, st, (const double*)X, s, ET64, (int64_t)mc.npS, Y, s, si,
-           1.0);
-    launch("k_dgemm", k_dgemm<false, false>, gg, NT, 0, st, ET64, (int64_t)mc.npS, (const double*)Y, s, Sb, s, si,
-           1.0);
+    // ET64 = L_SS^-T is upper triangular, Lm lower; only X's lower triangle is used (k_phi zeroes the rest), and
+    // Y = Phi(X) ET64^T is lower triangular, so Sb's sum starts at max(i, j)
+    if ((int64_t)nblk(s, 32) * nblk(s, 32) < 2 * sms)
+      chol_adjoint<16>(st, si, ET64, mc.npS, M1, Lm, Lbar, X, Y, Sb);
+    else
+      chol_adjoint<32>(st, si, ET64, mc.npS, M1, Lm, Lbar, X, Y, Sb);
     double* pS = tmp.alloc<double>(s * np2);
     launch("k_grad_kss", k_grad_kss, (unsigned)s, NT, 0, st, (const double*)Sb, (const double*)mc.ss64, si, d,
            mc.ss2, pS);

@@ -62,3 +62,13 @@ def test_fp64_windows_at_tile_edges(L, sizes, s, B):
     assert em <= 1e-9 and ev <= 1e-9 and el <= 1e-9, (em, ev, el)
     _, g = L.lma_loglik_grad(precision=L.FP64, **L.problem_args(p))
     assert _rel(g, O2.loglik_grad(p)[1]) <= 1e-9
+
+
+@pytest.mark.parametrize("d, s", [(8, 901), (9, 77), (3, 128)])
+def test_mixed_gradient_products_at_tile_edges(L, d, s):
+    """N x s products of the adjoint: 128-wide tiles with ragged edges and unaligned rows (4,871 x 901), the 64-wide
+    ones below; input dimensions padded to 8 and to 24.  Bound: the mixed gradient's 5e-4."""
+    n = 4871 if s > 900 else 333
+    p = make_random_problem(5, [n // 9] * 8 + [n - 8 * (n // 9)], d=d, s=s, B=1, ell=0.06 + 0.08 * d, sigma_n=0.2)
+    _, g = L.lma_loglik_grad(precision=L.MIXED, **L.problem_args(p))
+    assert _rel(g, O2.loglik_grad(p)[1]) <= 5e-4

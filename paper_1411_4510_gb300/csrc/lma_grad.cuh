@@ -560,42 +560,8 @@ __global__ void __launch_bounds__(256) k_grad_vbar_128(const float* __restrict__
     }
 }
 
-// Numbers held as the sum of two floats (48 bits): an FP64 instruction occupies a
-// scheduler for 64 clocks, a float one for one, so where FP64 is more than the result
-// needs but a float is less, sums and products of pairs are 5 to 10 times cheaper.
-struct Pair2 {
-  float h, l;
-};
-__device__ __forceinline__ Pair2 quick2(float a, float b) {  // |a| >= |b|
-  const float s = __fadd_rn(a, b);
-  return {s, __fsub_rn(b, __fsub_rn(s, a))};
-}
-__device__ __forceinline__ Pair2 sum2(float a, float b) {  // exact
-  const float s = __fadd_rn(a, b), t = __fsub_rn(s, a);
-  return {s, __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t))};
-}
-__device__ __forceinline__ Pair2 add2(Pair2 a, Pair2 b) {
-  const Pair2 s = sum2(a.h, b.h);
-  return quick2(s.h, __fadd_rn(s.l, __fadd_rn(a.l, b.l)));
-}
-__device__ __forceinline__ Pair2 mul2(Pair2 a, Pair2 b) {
-  const float p = __fmul_rn(a.h, b.h);
-  float e = __fmaf_rn(a.h, b.h, -p);
-  e = __fmaf_rn(a.h, b.l, e);
-  e = __fmaf_rn(a.l, b.h, e);
-  return quick2(p, e);
-}
-__device__ __forceinline__ Pair2 scale2(Pair2 a, float b) {
-  const float p = __fmul_rn(a.h, b);
-  return quick2(p, __fmaf_rn(a.l, b, __fmaf_rn(a.h, b, -p)));
-}
-__device__ __forceinline__ Pair2 split2(double x) {
-  const float h = (float)x;
-  return {h, (float)(x - (double)h)};
-}
-
-// exp(y) for y <= 0 to about 1e-11 relative (0 below 2^-125): y = n ln 2 + r with ln 2 in three parts (n times the
-// first is exact), then the Taylor series of exp(r), its terms from r^5 on in single precision (at most 4e-5 of the sum).
+// exp(y) for y <= 0 to about 1e-13 relative (0 below 2^-125): y = n ln 2 + r with ln 2 in three parts (n times the
+// first is exact), then the Taylor series of exp(r), its terms from r^8 on in single precision (at most 5e-9 of the sum).
 __device__ __forceinline__ Pair2 exp2f_pair(Pair2 y) {
   const float n = rintf(y.h * 1.44269504f);
   Pair2 r = sum2(y.h, -0.693359375f * n);
@@ -603,15 +569,16 @@ __device__ __forceinline__ Pair2 exp2f_pair(Pair2 y) {
   const float e = __fmaf_rn(n, 2.12194442e-4f, -q);
   r = add2(r, Pair2{q, __fadd_rn(e, __fmaf_rn(n, -1.64657177e-12f, y.l))});
   const float x = r.h;
-  float t = 1.f / 39916800.f;
+  float t = 1.f / 479001600.f;
+  t = fmaf(t, x, 1.f / 39916800.f);
   t = fmaf(t, x, 1.f / 3628800.f);
   t = fmaf(t, x, 1.f / 362880.f);
   t = fmaf(t, x, 1.f / 40320.f);
-  t = fmaf(t, x, 1.f / 5040.f);
-  t = fmaf(t, x, 1.f / 720.f);
-  t = fmaf(t, x, 1.f / 120.f);
-  Pair2 v = add2(Pair2{0.0416666679f, -1.24176348e-9f}, scale2(r, t));  // 1/24
-  v = add2(Pair2{0.166666672f, -4.96705388e-9f}, mul2(r, v));           // 1/6
+  Pair2 v = add2(Pair2{0.000198412701f, -2.72559687e-12f}, scale2(r, t));  // 1/5040
+  v = add2(Pair2{0.00138888892f, -3.36310944e-11f}, mul2(r, v));  // 1/720
+  v = add2(Pair2{0.00833333377f, -4.34617203e-10f}, mul2(r, v));  // 1/120
+  v = add2(Pair2{0.0416666679f, -1.24176347e-09f}, mul2(r, v));  // 1/24
+  v = add2(Pair2{0.166666672f, -4.96705388e-09f}, mul2(r, v));  // 1/6
   v = add2(Pair2{0.5f, 0.f}, mul2(r, v));
   v = add2(Pair2{1.f, 0.f}, mul2(r, v));
   v = add2(Pair2{1.f, 0.f}, mul2(r, v));
@@ -690,11 +657,8 @@ __global__ void __launch_bounds__(256) k_grad_kds_pair(const float* __restrict__
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 #pragma unroll
   for (int q = 0; q < D + 1; ++q) {
-    Pair2 v = q < D ? gl[q < D ? q : 0] : gs;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1)
-      v = add2(v, Pair2{__shfl_xor_sync(0xffffffffu, v.h, o), __shfl_xor_sync(0xffffffffu, v.l, o)});
-    if (lane == 0) red[warp][q] = (double)v.h + (double)v.l;
+    const Pair2 v = warp_sum2(q < D ? gl[q < D ? q : 0] : gs);
+    if (lane == 0) red[warp][q] = to_double(v);
   }
   __syncthreads();
   double* P = partial + ((int64_t)blockIdx.y * gridDim.x + blockIdx.x) * (d + 2);

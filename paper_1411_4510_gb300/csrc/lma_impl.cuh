@@ -220,6 +220,7 @@ struct ModelCore {
   Win* wins_d = nullptr;
   double* G = nullptr;        // (s+1)^2 global Gram [quad, y; y, A]
   double* beta = nullptr;     // s
+  float2* bs = nullptr;       // beta as two floats each (mixed form)
   void* LcT = nullptr;        // s*s, (L_C^-1)[i][k] at [k][i]   (T)
   double quad = 0, wCw = 0, logdetC = 0, logdetR = 0, loglik = 0;
   uint16_t* linv3 = nullptr;  // three bfloat16 planes of L_SS^-1 (mixed form on the tensor cores), brows x ldk each
@@ -305,12 +306,15 @@ void make_windows(const std::vector<int64_t>& bptr, int64_t B, int64_t s, size_t
                   int64_t& buf_elems, int64_t& dinv_elems, int64_t& ew_elems, int64_t m_begin = 0,
                   int64_t m_end = -1, const std::vector<int>* test_rows = nullptr);
 
-// Prediction pairs (test block n, window m in [n - B, n]) and per test block
-// (first pair, pair count, first test row, test rows).  fused: P rows of
-// pair (n, m) are window m's appended test rows (FusedTest); otherwise they
-// are packed in a separate buffer of *p_elems elements.
+// Prediction pairs (test block n, window m in [n - B, n]), per test block
+// (first pair, pair count, first test row, test rows), and per window with test
+// rows one pair of all of them (blocks m .. m + B, consecutive in test order) with
+// the number of its own block's, which come first.  fused: a window's P rows are
+// its appended test rows (FusedTest); otherwise they are packed, window after
+// window, in a separate buffer of *p_elems elements.
 void make_pairs(const std::vector<Win>& wins, int64_t w0, int64_t M, int64_t B, int64_t s, const int64_t* tptr,
-                bool fused, std::vector<Pair>& pairs, std::vector<int4>& tb, int64_t* p_elems);
+                bool fused, std::vector<Pair>& pairs, std::vector<int4>& tb, std::vector<Pair>& wpairs,
+                std::vector<int>& own, int64_t* p_elems);
 // number of appended test rows of each window of a whole fit (FusedTest)
 std::vector<int> fused_test_rows(int64_t M, int64_t B, const int64_t* tptr);
 

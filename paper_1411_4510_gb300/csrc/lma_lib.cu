@@ -17,6 +17,7 @@
 #include "lma_tc.cuh"
 #include "lma_grad_tc.cuh"
 #include "lma_bf6.cuh"
+#include "lma_pred_tc.cuh"
 #include "lma_f64.cuh"
 #include "lma_tune.cuh"
 
@@ -50,9 +51,28 @@ void make_windows(const std::vector<int64_t>& bptr, int64_t B, int64_t s, size_t
 }
 
 void make_pairs(const std::vector<Win>& wins, int64_t w0, int64_t M, int64_t B, int64_t s, const int64_t* tptr,
-                bool fused, std::vector<Pair>& pairs, std::vector<int4>& tb, int64_t* p_elems) {
-  std::vector<int> used(wins.size(), 0);  // test rows already placed in each window (fused)
+                bool fused, std::vector<Pair>& pairs, std::vector<int4>& tb, std::vector<Pair>& wpairs,
+                std::vector<int>& own, int64_t* p_elems) {
+  // every window's test rows (those of blocks m .. m + B, consecutive in test order) lie together: below the
+  // window's own extra rows (fused) or window after window in a separate buffer
+  std::vector<int64_t> base(wins.size(), 0);
   int64_t pe = 0;
+  for (size_t k = 0; k < wins.size(); ++k) {
+    const Win& w = wins[k];
+    const int64_t last = std::min<int64_t>(w.m + B, M - 1);
+    Pair p{};
+    p.u0 = (int)tptr[w.m];
+    p.nu = (int)(tptr[last + 1] - tptr[w.m]);
+    p.pbase = base[k] = fused ? w.base + (int64_t)(w.npad + s + 1) * w.npad : pe;
+    p.win = (int)k;
+    p.c0 = 0;
+    p.c1 = w.n;
+    p.n = w.m;
+    if (p.nu == 0) continue;
+    if (!fused) pe += (int64_t)p.nu * w.npad;
+    wpairs.push_back(p);
+    own.push_back((int)(tptr[w.m + 1] - tptr[w.m]));
+  }
   for (int64_t nb = 0; nb < M; ++nb) {
     const int nu = (int)(tptr[nb + 1] - tptr[nb]);
     if (nu == 0) continue;
@@ -60,13 +80,7 @@ void make_pairs(const std::vector<Win>& wins, int64_t w0, int64_t M, int64_t B, 
     for (int64_t m = std::max<int64_t>(0, nb - B); m <= nb; ++m) {
       const Win& w = wins[m - w0];
       Pair p{};
-      if (fused) {
-        p.pbase = w.base + (int64_t)(w.npad + s + 1 + used[m - w0]) * w.npad;
-        used[m - w0] += nu;
-      } else {
-        p.pbase = pe;
-        pe += (int64_t)nu * w.npad;
-      }
+      p.pbase = base[m - w0] + (tptr[nb] - tptr[m]) * (int64_t)w.npad;
       p.win = (int)(m - w0);
       p.u0 = (int)tptr[nb];
       p.nu = nu;
@@ -184,7 +198,10 @@ static size_t pt_smem() { return sizeof(tc::PtSmem) + tc::kTcAlignSlack; }
 
 template <int BN>
 static size_t wide_smem() { return sizeof(tc::WsSmem<2, BN>) + tc::kTcAlignSlack; }
-static size_t tc_resid_smem() { return sizeof(CompSmem<RB>) + tc::kTcAlignSlack; }
+template <int N>
+static size_t ps_smem() { return sizeof(tc::PsSmem<N>) + tc::kTcAlignSlack; }
+template <int N>
+static size_t pa_smem() { return sizeof(tc::PaSmem<N>) + tc::kTcAlignSlack; }
 
 // Grid of a persistent kernel with one CTA per SM: min(items, SM count).
 static unsigned persistent_grid(size_t items) {
@@ -317,13 +334,16 @@ void Impl<T>::setup_attributes() {
     set_smem_attr();
     cudaFuncSetAttribute(k_chol_step_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc_chol_smem());
     cudaFuncSetAttribute(k_chol_panel_pt, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pt_smem());
-    cudaFuncSetAttribute(k_pred_sweep_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc_chol_smem());
+    cudaFuncSetAttribute(k_pred_sweep_tc<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ps_smem<16>());
+    cudaFuncSetAttribute(k_pred_sweep_tc<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ps_smem<64>());
+    cudaFuncSetAttribute(k_pred_sweep_tc<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ps_smem<128>());
     cudaFuncSetAttribute(k_gram_bf6, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bf6::smem_bytes());
     cudaFuncSetAttribute(k_resid_bf6<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bf6::smem_bytes());
     cudaFuncSetAttribute(k_resid_bf6<MAXD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bf6::smem_bytes());
     cudaFuncSetAttribute(k_pred_rhs_bf6<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bf6::smem_bytes());
     cudaFuncSetAttribute(k_pred_rhs_bf6<MAXD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bf6::smem_bytes());
-    cudaFuncSetAttribute(k_pred_accum_win, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc_resid_smem());
+    cudaFuncSetAttribute(k_pred_accum_win<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pa_smem<16>());
+    cudaFuncSetAttribute(k_pred_accum_win<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pa_smem<64>());
     cudaFuncSetAttribute(k_chol_wide<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)wide_smem<256>());
     cudaFuncSetAttribute(k_chol_wide<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)wide_smem<128>());
     cudaFuncSetAttribute(k_proj_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bf6::smem_bytes());
@@ -930,7 +950,7 @@ void Impl<T>::fit_global(ModelCore& mc, int64_t n_total, cudaStream_t on) {
              (int)s, mc.brows, mc.ldk, mc.lcinv3);
     }
     if (sizeof(T) == 4) {
-      float2* bs = tmp.alloc<float2>(s);
+      float2* bs = mc.bs = mc.keep.alloc<float2>(s);
       launch("k_split_beta", k_split_beta, nblk(s), NT, 0, st, (const double*)mc.beta, (int)s, bs);
       launch("k_ew", k_ew_f32, dim3(nblk(maxnt * TB), (unsigned)M), NT, 0, st, mc.wins_d, (const float*)mc.wbuf,
              (const float2*)bs, (int)s, (float*)mc.ew);
@@ -1063,23 +1083,10 @@ void Impl<T>::fused_rhs(ModelCore& mc, FusedTest& ft, Arena& tmp) {
   // of blocks m .. m + B, consecutive both in the test order and in the
   // window buffer, so a 128-row tile covers the points of several blocks
   // (the right-hand sides R_{W_m u} of every pair (n, m) of the window).
-  std::vector<Pair> pairs;
-  const int64_t Mw = (int64_t)mc.wins.size();
-  for (int64_t m = 0; m < Mw; ++m) {
-    const Win& w = mc.wins[m];
-    const int64_t last = std::min<int64_t>(m + mc.B, mc.M - 1);
-    const int64_t u0 = ft.tptr[m], u1 = ft.tptr[last + 1];
-    if (u1 <= u0) continue;
-    Pair p{};
-    p.pbase = w.base + (int64_t)(w.npad + s + 1) * w.npad;
-    p.win = (int)m;
-    p.u0 = (int)u0;
-    p.nu = (int)(u1 - u0);
-    p.c0 = 0;
-    p.c1 = w.n;
-    p.n = (int)m;
-    pairs.push_back(p);
-  }
+  std::vector<Pair> all, pairs;
+  std::vector<int4> tb;
+  std::vector<int> own;
+  make_pairs(mc.wins, mc.w0, mc.M, mc.B, s, ft.tptr, true, all, tb, pairs, own, nullptr);
   if (pairs.empty()) return;
   Pair* pd = tmp.alloc<Pair>(pairs.size());
   stage_copy(pd, pairs.data(), sizeof(Pair) * pairs.size(), st);
@@ -1137,7 +1144,12 @@ void Impl<T>::predict(const ModelCore& mc, int64_t U, const double* XU, const in
     std::vector<Pair> pairs;
     std::vector<int4> tb;  // per test block: first pair, count, u0, nu
     int64_t pe = 0;
-    make_pairs(mc.wins, mc.w0, M, B, s, tptr, ft != nullptr, pairs, tb, &pe);
+    std::vector<Pair> wpairs;  // all test rows of a window
+    std::vector<int> own;      // ... of which the first are its own block's
+    make_pairs(mc.wins, mc.w0, M, B, s, tptr, ft != nullptr, pairs, tb, wpairs, own, &pe);
+    const bool use_tc = mc.prec == LMA_MIXED && sizeof(T) == 4 && use_tensor_cores();
+    int maxrows = 0;
+    for (const Pair& p : wpairs) maxrows = std::max(maxrows, p.nu);
     std::vector<int4> it_rhs, it_acc, it_t12;
     std::vector<int2> it_sw;
     for (size_t pi = 0; pi < pairs.size(); ++pi) {
@@ -1155,6 +1167,8 @@ void Impl<T>::predict(const ModelCore& mc, int64_t U, const double* XU, const in
         for (int kt = 0; kt < nst; ++kt) it_acc.push_back(make_int4(t.x, t.y, ut, kt));
       for (int u = 0; u < t.w; ++u) it_t12.push_back(make_int4(t.x, t.y, u, 0));
     }
+    Pair* wpd = tmp.alloc<Pair>(wpairs.size());
+    if (use_tc) stage_copy(wpd, wpairs.data(), sizeof(Pair) * wpairs.size(), st);
     Pair* pd = tmp.alloc<Pair>(pairs.size());
     int4* ird = tmp.alloc<int4>(it_rhs.size());
     int2* isd = tmp.alloc<int2>(it_sw.size());
@@ -1184,15 +1198,15 @@ void Impl<T>::predict(const ModelCore& mc, int64_t U, const double* XU, const in
         uint16_t* ub3 = split_rows_bf3(st, (const float*)Vu, U, s, sp, false, tmp.alloc<uint16_t>((size_t)3 * U * sp));
         const CUtensorMap vb = bf16_tensor_map(vb3, 3 * mc.n, sp), ub = bf16_tensor_map(ub3, 3 * U, sp);
         std::vector<int4> it_r;
-        for (size_t pi = 0; pi < pairs.size(); ++pi) {
-          const int nct = (mc.wins[pairs[pi].win].npad + 127) / 128;
-          for (int ut = 0; ut < (pairs[pi].nu + 127) / 128; ++ut)
+        for (size_t pi = 0; pi < wpairs.size(); ++pi) {
+          const int nct = (mc.wins[wpairs[pi].win].npad + 127) / 128;
+          for (int ut = 0; ut < (wpairs[pi].nu + 127) / 128; ++ut)
             for (int ct = 0; ct < nct; ++ct) it_r.push_back(make_int4((int)pi, ut, ct, 0));
         }
         int4* irr = tmp.alloc<int4>(it_r.size());
         stage_copy(irr, it_r.data(), sizeof(int4) * it_r.size(), st);
         launch("k_pred_rhs_bf6", pad_dim(d) == 8 ? k_pred_rhs_bf6<8> : k_pred_rhs_bf6<MAXD>,
-               persistent_grid(it_r.size()), bf6::NTHR, bf6::smem_bytes(), st, (const Pair*)pd, (const int4*)irr,
+               persistent_grid(it_r.size()), bf6::NTHR, bf6::smem_bytes(), st, (const Pair*)wpd, (const int4*)irr,
                (int)it_r.size(), (const Win*)mc.wins_d, (const float*)xs, (const float*)xu, d, ub, (int)U, vb,
                (int)mc.n, sp / bf6::KC, (float)mc.ss2, (float*)Pbuf, perr);
       } else {
@@ -1200,12 +1214,18 @@ void Impl<T>::predict(const ModelCore& mc, int64_t U, const double* XU, const in
                (int)s, (T)mc.ss2, Pbuf);
       }
       if (tc) {
+        // test rows a CTA: the smallest of 16, 64 and 128 that holds a window's (16 rows cost a CTA as much time as
+        // 64 where the factor's bytes bound it, but leave room for a deeper ring)
+        const int N = maxrows <= 16 ? 16 : (maxrows <= 64 ? 64 : 128);
         std::vector<int2> it_tc;
-        for (size_t pi = 0; pi < pairs.size(); ++pi)
-          for (int ut = 0; ut < (pairs[pi].nu + 127) / 128; ++ut) it_tc.push_back(make_int2((int)pi, ut));
+        for (size_t pi = 0; pi < wpairs.size(); ++pi)
+          for (int ut = 0; ut < (wpairs[pi].nu + N - 1) / N; ++ut) it_tc.push_back(make_int2((int)pi, ut));
         int2* itc = tmp.alloc<int2>(it_tc.size());
         stage_copy(itc, it_tc.data(), sizeof(int2) * it_tc.size(), st);
-        launch("k_pred_sweep_tc", k_pred_sweep_tc, (unsigned)it_tc.size(), 256, tc_chol_smem(), st, pd,
+        launch("k_pred_sweep_tc",
+               N == 16 ? k_pred_sweep_tc<16> : (N == 64 ? k_pred_sweep_tc<64> : k_pred_sweep_tc<128>),
+               (unsigned)it_tc.size(), tc::kPsThreads,
+               N == 16 ? ps_smem<16>() : (N == 64 ? ps_smem<64>() : ps_smem<128>()), st, (const Pair*)wpd,
                (const int2*)itc, mc.wins_d, (const float*)wbuf, (const float*)mc.dinv, (float*)Pbuf, perr);
       } else {
         launch("k_pred_sweep", k_pred_sweep<T>, (unsigned)it_sw.size(), NT, sizeof(CholSmem<T>), st, pd, isd,
@@ -1223,46 +1243,32 @@ void Impl<T>::predict(const ModelCore& mc, int64_t U, const double* XU, const in
              (const Win*)mc.wins_d, (const double*)wbuf, (const double*)mc.dv16, (double*)Pbuf);
     }
     T* h = tmp.alloc<T>(U * s);
-    if (mc.prec == LMA_MIXED && sizeof(T) == 4 && use_tensor_cores()) {
-      // per window: its pairs (n, m) in increasing n, their partial rows, items
-      const int64_t nwin = (int64_t)mc.wins.size();
-      std::vector<std::vector<int>> byw((size_t)nwin);
-      for (size_t pi = 0; pi < pairs.size(); ++pi) byw[pairs[pi].win].push_back((int)pi);
-      std::vector<int> wp;
-      std::vector<int4> it_w;
-      std::vector<int64_t> wrow, prow(pairs.size(), 0);
+    if (use_tc) {
+      // per window: all its test rows against its extra rows, in partial rows of their own
+      const int N = maxrows <= 16 ? 16 : 64;
+      std::vector<AccItem> it_w;
+      std::vector<int64_t> wrow(mc.wins.size(), 0), prow(pairs.size(), 0);
       int64_t hrows = 0;
-      for (int64_t m = 0; m < nwin; ++m) {
-        if (byw[m].empty()) continue;
-        const int off = (int)wp.size();
-        int rows = 0;
-        for (int pi : byw[m]) {
-          wp.push_back(pi);
-          prow[pi] = hrows + rows;
-          rows += pairs[pi].nu;
-        }
-        for (int ut = 0; ut < (rows + 127) / 128; ++ut)
-          for (int kt = 0; kt < (s + RB - 1) / RB; ++kt) {
-            it_w.push_back(make_int4(off, (int)byw[m].size(), ut, kt));
-            wrow.push_back(hrows);
-          }
-        hrows += rows;
+      for (size_t k = 0; k < wpairs.size(); ++k) {
+        const Pair& p = wpairs[k];
+        wrow[p.win] = hrows;
+        for (int ut = 0; ut < (p.nu + N - 1) / N; ++ut)
+          for (int kt = 0; kt < (s + 127) / 128; ++kt) it_w.push_back(AccItem{(int)k, ut, kt, own[k], hrows});
+        hrows += p.nu;
       }
-      int* wpd = tmp.alloc<int>(wp.size());
-      int4* iwd = tmp.alloc<int4>(it_w.size());
-      int64_t* wrd = tmp.alloc<int64_t>(wrow.size());
+      for (size_t pi = 0; pi < pairs.size(); ++pi)
+        prow[pi] = wrow[pairs[pi].win] + (pairs[pi].u0 - tptr[mc.wins[pairs[pi].win].m]);
+      AccItem* iwd = tmp.alloc<AccItem>(it_w.size());
       int64_t* prd = tmp.alloc<int64_t>(prow.size());
       int4* tbd = tmp.alloc<int4>(tb.size());
-      stage_copy(wpd, wp.data(), sizeof(int) * wp.size(), st);
-      stage_copy(iwd, it_w.data(), sizeof(int4) * it_w.size(), st);
-      stage_copy(wrd, wrow.data(), sizeof(int64_t) * wrow.size(), st);
+      stage_copy(iwd, it_w.data(), sizeof(AccItem) * it_w.size(), st);
       stage_copy(prd, prow.data(), sizeof(int64_t) * prow.size(), st);
       stage_copy(tbd, tb.data(), sizeof(int4) * tb.size(), st);
       float* hw = tmp.alloc<float>((size_t)hrows * s);
       if (!it_w.empty())
-        launch("k_pred_accum_tc", k_pred_accum_win, (unsigned)it_w.size(), comp_threads<RB>(), tc_resid_smem(), st, pd,
-               (const int*)wpd, (const int4*)iwd, (const int64_t*)wrd, mc.wins_d, (const float*)wbuf,
-               (const float*)Pbuf, (int)s, hw, perr);
+        launch("k_pred_accum_tc", N == 16 ? k_pred_accum_win<16> : k_pred_accum_win<64>, persistent_grid(it_w.size()),
+               tc::pa_threads(N), N == 16 ? pa_smem<16>() : pa_smem<64>(), st, (const Pair*)wpd, (const AccItem*)iwd,
+               (int)it_w.size(), mc.wins_d, (const float*)wbuf, (const float*)Pbuf, (int)s, hw, perr);
       int maxnu = 1;
       for (const int4& t : tb) maxnu = std::max(maxnu, t.w);
       if (!tb.empty())
@@ -1304,7 +1310,7 @@ void Impl<T>::predict(const ModelCore& mc, int64_t U, const double* XU, const in
       vd = tmp.alloc<double>(U);
     }
     const double prior = mc.ss2 + (noisy ? mc.sn2 : 0.0);
-    launch("k_pred_final", k_pred_final<T>, nblk(U * 32), NT, 0, st, Vu, U, (int)s, mc.beta, t1, t2, part, ntile_var,
+    launch("k_pred_final", k_pred_final<T>, nblk(U * 32), NT, 0, st, Vu, U, (int)s, mc.beta, (const float2*)mc.bs, t1, t2, part, ntile_var,
            mc.mu, prior, md, vd);
     if (cov) {
       // requested blocks of the covariance between test blocks (Eq. vapvar on

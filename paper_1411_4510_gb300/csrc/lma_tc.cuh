@@ -739,10 +739,11 @@ __device__ bool ws_product(WsSmem<NS, BN>& sm, int K, RA rowA, RB rowB) {
           const int i = tid + PT * q;
           store_split4(S.b_hi, S.b_lo, i >> 3, (i & 7) * 4, rb[d][q]);
         }
-        if (c + D < nchunk) load(c + D, ra[d], rb[d]);
         fence_async_smem();
         __syncwarp();
         if (lane == 0) mbar_arrive(&sm.full[s]);
+        // after the arrival: it releases the warp's earlier accesses, loads in flight among them
+        if (c + D < nchunk) load(c + D, ra[d], rb[d]);
       }
     }
   } else {
@@ -1210,315 +1211,9 @@ __global__ void __maxnreg__(128) k_chol_panel_pt(const Win* __restrict__ wins, i
   if (warp == kPtProducers) tmem_dealloc(sm.tmem, 128);
 }
 
-// Forward solve of the prediction right-hand sides on the tensor cores: CTA
-// (pair, 128 test rows) sweeps the window's column panels left to right,
-//   T = P[:, panel] - P[:, 0:k0] L[panel, 0:k0]^T ;  P[:, panel] = T inv(L_kk)^T
-// with both products on tcgen05 (3xTF32).  items: x = pair, y = 128-row tile.
-__global__ void __launch_bounds__(256, 2) k_pred_sweep_tc(const Pair* __restrict__ pairs, const int2* __restrict__ items,
-                                                       const Win* __restrict__ wins, const float* __restrict__ buf,
-                                                       const float* __restrict__ dinv, float* __restrict__ P,
-                                                       int* __restrict__ err) {
-  using namespace tc;
-  const int2 it = items[blockIdx.x];
-  const Pair pr = pairs[it.x];
-  const Win w = wins[pr.win];
-  const int u0 = it.y * 128;
-  extern __shared__ __align__(16) unsigned char smraw[];
-  TcSmem<64>& sm = tc_smem<64>(smraw);
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const float* L = buf + w.base;
-  const int64_t ld = w.npad;
-  float* Pp = P + pr.pbase;
-  if (tid == 0) {
-    mbar_init(&sm.bar[0], 1);
-    mbar_init(&sm.bar[1], 1);
-    mbar_fence_init();
-  }
-  if (warp == 0) tmem_alloc(&sm.tmem, 64);
-  fence_before_sync();
-  __syncthreads();
-  fence_after_sync();
-  const uint32_t tmem = sm.tmem;
-  TcPipe pipe;
-  const int q = warp & 3, half = warp >> 2;
-  const int rl = q * 32 + lane;
-  const bool live = (u0 + rl) < pr.nu;
-  float* myrow = Pp + (int64_t)(u0 + rl) * ld;
-  const uint32_t taddr = tmem + ((uint32_t)(q * 32) << 16) + half * 32;
-  bool ok = true;
-  const int npan = w.npad / TB;
-  for (int kp = 0; kp < npan && ok; ++kp) {
-    const int k0 = kp * TB;
-    float v[32];
-    if (k0 > 0) {
-      auto rowA = [&](int r) -> const float* {
-        return (u0 + r) < pr.nu ? Pp + (int64_t)(u0 + r) * ld : nullptr;
-      };
-      auto rowB = [&](int c) -> const float* { return L + (int64_t)(k0 + c) * ld; };
-      ok = tile_product<64>(sm, pipe, tmem, k0, rowA, rowB);
-      if (!ok) break;
-      float t[16];
-      tmem_ld16(taddr, t);
-#pragma unroll
-      for (int j = 0; j < 16; ++j) v[j] = t[j];
-      tmem_ld16(taddr + 16, t);
-#pragma unroll
-      for (int j = 0; j < 16; ++j) v[16 + j] = t[j];
-    } else {
-#pragma unroll
-      for (int j = 0; j < 32; ++j) v[j] = 0.f;
-    }
-    if (live) {
-      float* dst = myrow + k0 + half * 32;
-      float4 av[8];  // all loads first: they are independent of the stores below
-#pragma unroll
-      for (int j4 = 0; j4 < 8; ++j4) av[j4] = *reinterpret_cast<const float4*>(dst + 4 * j4);
-#pragma unroll
-      for (int j4 = 0; j4 < 8; ++j4) {
-        float4 a = av[j4];
-        a.x -= v[4 * j4 + 0];
-        a.y -= v[4 * j4 + 1];
-        a.z -= v[4 * j4 + 2];
-        a.w -= v[4 * j4 + 3];
-        *reinterpret_cast<float4*>(dst + 4 * j4) = a;
-      }
-    }
-    fence_before_sync();
-    __syncthreads();
-    const float* Dv = dinv + w.dinv + (int64_t)kp * TB * TB;
-    auto rowT = [&](int r) -> const float* { return (u0 + r) < pr.nu ? Pp + (int64_t)(u0 + r) * ld + k0 : nullptr; };
-    auto rowD = [&](int c) -> const float* { return Dv + (int64_t)c * TB; };
-    ok = tile_product<64>(sm, pipe, tmem, TB, rowT, rowD);
-    if (!ok) break;
-    float t[16];
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      tmem_ld16(taddr + 16 * h, t);
-      if (live) {
-        float* dst = myrow + k0 + half * 32 + 16 * h;
-#pragma unroll
-        for (int j4 = 0; j4 < 4; ++j4)
-          *reinterpret_cast<float4*>(dst + 4 * j4) = make_float4(t[4 * j4], t[4 * j4 + 1], t[4 * j4 + 2], t[4 * j4 + 3]);
-      }
-    }
-    fence_before_sync();
-    __syncthreads();
-  }
-  if (!ok && tid == 0) atomicExch(err, 1);
-  fence_before_sync();
-  __syncthreads();
-  if (warp == 0) tmem_dealloc(tmem, 64);
-}
-
 }  // namespace lma
 
 namespace lma {
-
-// Compensated tile product on the tensor cores over a 128 x BN tile:
-// hi + lo = sum_{k<K} A(r,k) B(c,k) for worker thread t's row
-// r = 32 (warp mod 4) + lane and its 32 columns c = 32 (warp / 4) + j.
-// 4 BN worker threads (warps 0 .. BN/8 - 1) load each 32-wide K chunk one
-// chunk ahead into registers, split it into TF32 hi/lo into stage c mod 2 and
-// arrive on full[s]; the last warp issues the chunk's 12 MMAs into tensor-
-// memory slot (c / 2) mod 2 (columns [BN slot, BN slot + BN)) and commits to
-// done[s].  Before refilling stage s the workers wait for done[s] of chunk
-// c - 2; when that chunk ends a pair (chunks 2p, 2p + 1) they drain the
-// pair's slot into registers, adding its sums with TwoSum, so the slot is
-// free before the MMAs of pair p + 2 start.  The tensor core's FP32
-// accumulation is 24 MMA steps (64 values of K) deep, the cross-pair sum is
-// compensated, and no CTA-wide barrier waits for the MMA issue.  (Draining
-// after every chunk made the workers' TwoSum work, not the MMAs, the limit.)
-template <int BN>
-struct CompSmem {
-  tc::TcStage<BN> st[2];
-  uint64_t full[2], done[2], fin;
-  uint32_t tmem;
-  int abort;
-};
-template <int BN>
-__device__ __forceinline__ CompSmem<BN>& comp_smem(unsigned char* raw) {
-  uintptr_t p = reinterpret_cast<uintptr_t>(raw);
-  p = (p + 1023) & ~uintptr_t(1023);
-  return *reinterpret_cast<CompSmem<BN>*>(p);
-}
-template <int BN>
-constexpr int comp_threads() { return 4 * BN + 32; }
-
-// Barriers and tensor memory (2 BN columns, allocated by the MMA warp).
-template <int BN>
-__device__ __forceinline__ void comp_setup(CompSmem<BN>& sm) {
-  using namespace tc;
-  constexpr int NW = BN / 8;  // worker warps
-  if (threadIdx.x == 0) {
-    for (int s = 0; s < 2; ++s) {
-      mbar_init(&sm.full[s], NW);
-      mbar_init(&sm.done[s], 1);
-    }
-    mbar_init(&sm.fin, 1);
-    sm.abort = 0;
-    mbar_fence_init();
-  }
-  if ((threadIdx.x >> 5) == NW) tmem_alloc(&sm.tmem, 2 * BN);
-  fence_before_sync();
-  __syncthreads();
-  fence_after_sync();
-}
-template <int BN>
-__device__ __forceinline__ void comp_teardown(CompSmem<BN>& sm) {
-  using namespace tc;
-  fence_before_sync();
-  __syncthreads();
-  if ((threadIdx.x >> 5) == BN / 8) tmem_dealloc(sm.tmem, 2 * BN);
-}
-
-// Chunk and call counters of a CTA's compensated products: a kernel may call
-// comp_product several times (one K range each) and the barrier phases
-// continue from one call to the next.
-struct CompState {
-  int chunks = 0;
-  int calls = 0;
-};
-
-// Adds sum over k in [kbeg, kend) of A(r,k) B(c,k) to hi + lo (zeroed first
-// unless ACC).  rowA(r) / rowB(c) return a 16-byte-aligned row pointer (or
-// nullptr for a zero row) whose row holds at least kend rounded up to 4
-// values; values outside [kbeg, kend) are masked.  MASK = false is for
-// kbeg = 0 and kend a multiple of 32 (nothing to mask).  Returns false (in every
-// thread) when a wait timed out.  hi / lo are only meaningful in workers.
-template <int BN, bool ACC = false, bool MASK = true, class RA, class RB>
-__device__ bool comp_product(CompSmem<BN>& sm, CompState& cs, int kbeg, int kend, RA rowA, RB rowB,
-                             float (&hi)[32], float (&lo)[32]) {
-  using namespace tc;
-  constexpr int NW = BN / 8, NTHR = 4 * BN;
-  constexpr int NA = 128 * 8 / NTHR, NB = BN * 8 / NTHR;  // float4 per worker per chunk
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int kal = kbeg & ~3;
-  const int nchunk = kend > kbeg ? (kend - kal + 31) / 32 : 0;
-  const int g0 = cs.chunks;  // global index of this call's first chunk
-  volatile int* abort_flag = &sm.abort;
-  if (!ACC) {
-#pragma unroll
-    for (int j = 0; j < 32; ++j) hi[j] = lo[j] = 0.f;
-  }
-  if (warp < NW) {
-    const int q = warp & 3, half = warp >> 2;
-    const uint32_t tlane = sm.tmem + ((uint32_t)(q * 32) << 16) + half * 32;
-    auto wait_done = [&](int g) -> bool {  // MMAs of global chunk g have completed (warp-uniform result)
-      int okw = 1;
-      if (lane == 0) okw = mbar_wait(&sm.done[g & 1], (g >> 1) & 1) ? 1 : 0;
-      okw = __shfl_sync(0xffffffffu, okw, 0);
-      if (!okw) *abort_flag = 1;
-      return okw != 0;
-    };
-    auto drain = [&](int pair) {
-      fence_after_sync();
-      float t[16];
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        tmem_ld16(tlane + BN * (pair & 1) + 16 * h, t);
-#pragma unroll
-        for (int j = 0; j < 16; ++j) two_sum(hi[16 * h + j], lo[16 * h + j], t[j]);
-      }
-      fence_before_sync();
-    };
-    float4 ra[NA], rb[NB];
-    auto ld4 = [&](const float* src, int kk) -> float4 {
-      if (!MASK) return src ? *reinterpret_cast<const float4*>(src + kk) : make_float4(0.f, 0.f, 0.f, 0.f);
-      if (!src || kk >= kend) return make_float4(0.f, 0.f, 0.f, 0.f);
-      float4 v = *reinterpret_cast<const float4*>(src + kk);
-      if (kk < kbeg || kk + 4 > kend) {
-        v.x = (kk >= kbeg && kk < kend) ? v.x : 0.f;
-        v.y = (kk + 1 >= kbeg && kk + 1 < kend) ? v.y : 0.f;
-        v.z = (kk + 2 >= kbeg && kk + 2 < kend) ? v.z : 0.f;
-        v.w = (kk + 3 >= kbeg && kk + 3 < kend) ? v.w : 0.f;
-      }
-      return v;
-    };
-    auto load = [&](int c) {
-      const int k0 = kal + c * 32;
-#pragma unroll
-      for (int j = 0; j < NA; ++j) {
-        const int i = tid + NTHR * j, row = i >> 3, c4 = i & 7;
-        ra[j] = ld4(rowA(row), k0 + c4 * 4);
-      }
-#pragma unroll
-      for (int j = 0; j < NB; ++j) {
-        const int i = tid + NTHR * j, row = i >> 3, c4 = i & 7;
-        rb[j] = ld4(rowB(row), k0 + c4 * 4);
-      }
-    };
-    // chunk c of this call accumulates into tensor-memory slot (c / 2) mod 2;
-    // a slot is drained once the last chunk of its pair has completed
-    auto ends_pair = [&](int c) { return (c & 1) == 1 || c == nchunk - 1; };
-    if (nchunk > 0) load(0);
-    for (int c = 0; c < nchunk; ++c) {
-      const int g = g0 + c, s = g & 1;
-      if (c >= 2) {  // chunk c - 2 used stage s
-        if (!wait_done(g - 2)) break;
-        if (ends_pair(c - 2)) drain((c - 2) >> 1);
-      }
-      if (*abort_flag) break;
-      TcStage<BN>& S = sm.st[s];
-#pragma unroll
-      for (int j = 0; j < NA; ++j) {
-        const int i = tid + NTHR * j;
-        store_split4(S.a_hi, S.a_lo, i >> 3, (i & 7) * 4, ra[j]);
-      }
-#pragma unroll
-      for (int j = 0; j < NB; ++j) {
-        const int i = tid + NTHR * j;
-        store_split4(S.b_hi, S.b_lo, i >> 3, (i & 7) * 4, rb[j]);
-      }
-      if (c + 1 < nchunk) load(c + 1);
-      fence_async_smem();
-      fence_before_sync();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&sm.full[s]);
-    }
-    for (int c = max(0, nchunk - 2); c < nchunk && !*abort_flag; ++c) {  // the last one or two chunks, in order
-      if (!wait_done(g0 + c)) break;
-      if (ends_pair(c)) drain(c >> 1);
-    }
-  } else {
-    // MMA warp: the whole warp runs the loop, lane 0 issues
-    const uint32_t idesc = idesc_tf32(128, BN);
-    for (int c = 0; c < nchunk; ++c) {
-      const int g = g0 + c, s = g & 1;
-      if (*abort_flag) break;
-      int okw = 1;
-      if (lane == 0) okw = mbar_wait(&sm.full[s], (g >> 1) & 1) ? 1 : 0;
-      okw = __shfl_sync(0xffffffffu, okw, 0);
-      if (!okw) {
-        *abort_flag = 1;
-        break;
-      }
-      fence_after_sync();
-      if (lane == 0) {
-        TcStage<BN>& S = sm.st[s];
-        const uint32_t ah = smem_addr(S.a_hi), al = smem_addr(S.a_lo);
-        const uint32_t bh = smem_addr(S.b_hi), bl = smem_addr(S.b_lo);
-        const uint32_t dcol = sm.tmem + BN * ((c >> 1) & 1);
-        const bool first = (c & 1) == 0;
-#pragma unroll
-        for (int ks = 0; ks < 4; ++ks) {
-          const uint32_t o = ks * 32;
-          mma_tf32(dcol, sdesc_sw128(ah + o), sdesc_sw128(bh + o), idesc, (first && ks == 0) ? 0u : 1u);
-          mma_tf32(dcol, sdesc_sw128(ah + o), sdesc_sw128(bl + o), idesc, 1u);
-          mma_tf32(dcol, sdesc_sw128(al + o), sdesc_sw128(bh + o), idesc, 1u);
-        }
-        mma_commit(&sm.done[s]);
-      }
-      __syncwarp();
-    }
-    if (lane == 0) mma_commit(&sm.fin);  // arrives once every MMA issued above has completed
-    __syncwarp();
-  }
-  // every issued MMA has completed before anyone reads or frees tensor memory
-  const bool w = mbar_wait(&sm.fin, cs.calls & 1);
-  cs.chunks += nchunk;
-  cs.calls += 1;
-  return __syncthreads_and(w && !*abort_flag) != 0;
-}
 
 // ---------------------------------------------------------------------------
 // Worker warps of the persistent tensor-core products (4 lane quarters x 4
@@ -1562,89 +1257,8 @@ __device__ __forceinline__ float dist2(const float (&a)[D], const float* b) {
 // Input dimension padded for the unrolled epilogues (a multiple of 4).
 __host__ __device__ constexpr int pad_dim(int d) { return d <= 8 ? 8 : MAXD; }
 
-// The h accumulation per window (mixed form): the test rows that use window m
-// (the pairs (n, m), n = m .. m + B) share its extra rows X_{1+k} as the B
-// operand, so one 128-row tile covers the test points of several blocks.
-// Item x = first index into wp (the window's pairs, increasing n), y = pair
-// count, z = 128-row tile of the window's test rows, w = RB-wide s tile; the
-// partial hw[(prow + r) * s + k] = sum over the pair's kept columns of
-// P[r][c] X_{1+k}[c] (block columns [nB, n) for every row, the blanket
-// columns [0, nB) only for the rows of block m itself), where prow is the
-// window's first partial row (wrow[item], one entry per item).  k_pred_hsum adds each test point's
-// partials in window order.
-__global__ void __launch_bounds__(comp_threads<RB>(), 1) k_pred_accum_win(const Pair* __restrict__ pairs,
-                                                                        const int* __restrict__ wp,
-                                                                        const int4* __restrict__ items,
-                                                                        const int64_t* __restrict__ wrow,
-                                                                        const Win* __restrict__ wins,
-                                                                        const float* __restrict__ buf,
-                                                                        const float* __restrict__ P, int s,
-                                                                        float* __restrict__ hw, int* __restrict__ err) {
-  using namespace tc;
-  const int4 it = items[blockIdx.x];
-  const int u0 = it.z * 128, k0 = it.w * RB;
-  extern __shared__ __align__(16) unsigned char smraw[];
-  CompSmem<RB>& sm = comp_smem<RB>(smraw);
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  comp_setup(sm);
-  const Pair p0 = pairs[wp[it.x]];
-  const Win w = wins[p0.win];
-  const float* E = buf + w.base + (int64_t)w.npad * w.npad;
-  const int64_t ld = w.npad;
-  // row r of the tile -> pointer to its P row (nullptr past the window's test
-  // rows) and whether it is a row of block m itself (kept blanket columns)
-  __shared__ const float* rowp[128];
-  __shared__ int rowown[128];
-  __shared__ int s_rows;
-  if (tid < 128) {
-    int rr = u0 + tid;
-    const float* ptr = nullptr;
-    int own = 0;
-    for (int j = 0; j < it.y; ++j) {
-      const Pair pr = pairs[wp[it.x + j]];
-      if (rr < pr.nu) {
-        own = pr.c0 == 0;
-        ptr = P + pr.pbase + (int64_t)rr * ld;
-        break;
-      }
-      rr -= pr.nu;
-    }
-    rowp[tid] = ptr;
-    rowown[tid] = own;
-  }
-  if (tid == 0) {
-    int rows = 0;
-    for (int j = 0; j < it.y; ++j) rows += pairs[wp[it.x + j]].nu;
-    s_rows = rows;
-  }
-  __syncthreads();
-  auto rowB = [&](int c) -> const float* { return (k0 + c < s) ? E + (int64_t)(1 + k0 + c) * ld : nullptr; };
-  CompState cs;
-  float hi[32], lo[32];
-#pragma unroll
-  for (int j = 0; j < 32; ++j) hi[j] = lo[j] = 0.f;
-  auto rowAll = [&](int r) -> const float* { return rowp[r]; };
-  bool ok = comp_product<RB, true>(sm, cs, w.nB, w.n, rowAll, rowB, hi, lo);
-  if (ok && w.nB > 0) {
-    auto rowOwn = [&](int r) -> const float* { return rowown[r] ? rowp[r] : nullptr; };
-    ok = comp_product<RB, true>(sm, cs, 0, w.nB, rowOwn, rowB, hi, lo);
-  }
-  if (!ok && tid == 0) atomicExch(err, 1);
-  const int rows = s_rows;
-  const int q = warp & 3, half = warp >> 2;
-  const int rr = u0 + q * 32 + lane;
-  const int kg = k0 + half * 32;
-  if (ok && warp < RB / 8 && rr < rows) {
-    float* dst = hw + (wrow[blockIdx.x] + rr) * (int64_t)s;
-#pragma unroll
-    for (int j = 0; j < 32; ++j)
-      if (kg + j < s) dst[kg + j] = hi[j] + lo[j];
-  }
-  comp_teardown(sm);
-}
-
 // h[u][k] = sum over the pairs (n, m) of u's test block n, in window order, of
-// hw[(prow of the pair + u - u0) * s + k] (added in FP64), minus Vu[u][k].
+// hw[(prow of the pair + u - u0) * s + k], minus Vu[u][k], added in pairs of floats and rounded once.
 // Grid: y = test block (tb: x = its first pair, y = pair count, z = first test
 // row, w = rows), x covers the block's rows x s elements; prow[pair] = the
 // pair's first partial row.
@@ -1656,10 +1270,10 @@ __global__ void k_pred_hsum(const int4* __restrict__ tb, const int64_t* __restri
   if (e >= (int64_t)t.w * s) return;
   const int64_t r = e / s;
   const int k = (int)(e - r * s);
-  double acc = 0.0;
-  for (int j = 0; j < t.y; ++j) acc += (double)hw[(prow[t.x + j] + r) * s + k];
+  Pair2 acc{0.f, 0.f};
+  for (int j = 0; j < t.y; ++j) acc = add2(acc, Pair2{hw[(prow[t.x + j] + r) * s + k], 0.f});
   const int64_t o = (t.z + r) * (int64_t)s + k;
-  h[o] = (float)(acc - (double)Vu[o]);
+  h[o] = add2(acc, Pair2{-Vu[o], 0.f}).h;
 }
 
 

@@ -64,11 +64,36 @@ def test_fp64_windows_at_tile_edges(L, sizes, s, B):
     assert _rel(g, O2.loglik_grad(p)[1]) <= 1e-9
 
 
-@pytest.mark.parametrize("d, s", [(8, 901), (9, 77), (3, 128)])
+@pytest.mark.parametrize("d, s", [(9, 77), (3, 128)])
 def test_mixed_gradient_products_at_tile_edges(L, d, s):
-    """N x s products of the adjoint: 128-wide tiles with ragged edges and unaligned rows (4,871 x 901), the 64-wide
-    ones below; input dimensions padded to 8 and to 24.  Bound: the mixed gradient's 5e-4."""
-    n = 4871 if s > 900 else 333
+    """N x s products of the adjoint on 64-wide tiles with ragged edges, input dimensions padded to 8 and to 24 (the
+    128-wide tiles run in the full-size gradient test).  Bound: the mixed gradient's 5e-4."""
+    n = 333
     p = make_random_problem(5, [n // 9] * 8 + [n - 8 * (n // 9)], d=d, s=s, B=1, ell=0.06 + 0.08 * d, sigma_n=0.2)
     _, g = L.lma_loglik_grad(precision=L.MIXED, **L.problem_args(p))
     assert _rel(g, O2.loglik_grad(p)[1]) <= 5e-4
+
+
+@pytest.mark.parametrize("s", [1001, 900])
+def test_adjoint_128_wide_tiles_equal_64_wide_ones(L, s):
+    """The gradient of a whole fit (128-wide tiles: 4,871 points, rows of s values aligned or not) against the sum of
+    the gradients of two shards of its blocks (64-wide ones).  The terms are the same, each shard's Vt-bar is rounded to
+    FP32 by itself and its K-sums run over its own points: 2^-24 per operation over sums whose terms cancel by up to
+    about 1e3 leaves 1e-4 of the gradient."""
+    n, nb = 4871, 9
+    p = make_random_problem(5, [n // nb] * (nb - 1) + [n - (nb - 1) * (n // nb)], d=8, s=s, B=0, ell=0.7, sigma_n=0.2)
+    args = L.problem_args(p)
+    _, g = L.lma_loglik_grad(precision=L.MIXED, **args)
+    ptr, parts = p.block_ptr, []
+    for b0, b1 in ((0, 2), (2, 4), (4, 6), (6, 8), (8, 9)):
+        rows = slice(ptr[b0], ptr[b1])
+        sub = dict(args, X=p.X[rows], y=p.y[rows], block_ptr=ptr[b0:b1 + 1] - ptr[b0])
+        m = L.lma_fit_local(win_begin=0, own_begin=0, own_end=b1 - b0, precision=L.MIXED, **sub)
+        parts.append((m, *L.lma_model_local_summary(m)))
+    G, ld = sum(x[1] for x in parts), sum(x[2] for x in parts)
+    total = 0.0
+    for m, _, _ in parts:
+        L.lma_model_set_global(m, G, ld, n)
+        total = total + L.lma_model_loglik_grad(m)
+    # the support-set term's partial sums are per shard: everything after the window terms is linear in them
+    assert _rel(total, g) <= 1e-4

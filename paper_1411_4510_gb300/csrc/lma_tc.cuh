@@ -580,7 +580,7 @@ __global__ void __launch_bounds__(256, 2) k_chol_step_tc(const Win* __restrict__
     fence_after_sync();
     tmem = sm.tmem;
     TcPipe pipe;
-    auto rowA = [&](int r) -> const float* { return r < TB ? A + (int64_t)(k0 + r) * ld + kb : nullptr; };
+    auto rowA = [&](int r) -> const float* { return A + (int64_t)(k0 + (r & (TB - 1))) * ld + kb; };  // rows 64 .. are not read
     auto rowB = [&](int c) -> const float* { return A + (int64_t)(k0 + c) * ld + kb; };
     ok = tile_product<64>(sm, pipe, tmem, K, rowA, rowB);
     if (!ok && tid == 0) atomicExch(err, 1);
@@ -681,8 +681,9 @@ __device__ __forceinline__ void ws_teardown(WsSmem<NS, BN>& sm) {
 
 // D (tensor memory, 128 lanes x BN FP32 columns) = sum_{k<K} A(r,k) B(c,k)
 // (3xTF32), r < 128, c < BN, K % 32 == 0; rowA(r) / rowB(c) return a
-// 16-byte-aligned pointer to the K values of that row or nullptr for a zero
-// row.  Called by all kWsThreads threads; returns false (in every thread)
+// 16-byte-aligned pointer to the K values of that row, of any valid row where
+// the result is not wanted (a load under a condition makes the warp wait for it
+// before it issues the next).  Called by all kWsThreads threads; returns false (in every thread)
 // when a wait timed out.  On return every MMA has completed.
 template <int NS, int BN, class RA, class RB>
 __device__ bool ws_product(WsSmem<NS, BN>& sm, int K, RA rowA, RB rowB) {
@@ -698,14 +699,12 @@ __device__ bool ws_product(WsSmem<NS, BN>& sm, int K, RA rowA, RB rowB) {
 #pragma unroll
       for (int j = 0; j < NA; ++j) {
         const int i = tid + PT * j, row = i >> 3, c4 = i & 7;
-        const float* src = rowA(row);
-        xa[j] = src ? *reinterpret_cast<const float4*>(src + k0 + c4 * 4) : make_float4(0.f, 0.f, 0.f, 0.f);
+        xa[j] = *reinterpret_cast<const float4*>(rowA(row) + k0 + c4 * 4);
       }
 #pragma unroll
       for (int j = 0; j < NB; ++j) {
         const int i = tid + PT * j, row = i >> 3, c4 = i & 7;
-        const float* src = rowB(row);
-        xb[j] = src ? *reinterpret_cast<const float4*>(src + k0 + c4 * 4) : make_float4(0.f, 0.f, 0.f, 0.f);
+        xb[j] = *reinterpret_cast<const float4*>(rowB(row) + k0 + c4 * 4);
       }
     };
 #pragma unroll
@@ -815,11 +814,8 @@ __global__ void __launch_bounds__(tc::kWsThreads, 1) k_chol_wide(const Win* __re
   float* A = buf + w.base;
   const int64_t ld = w.npad;
   ws_setup(sm);
-  auto rowA = [&](int r) -> const float* {
-    const int row = r0 + r;
-    return row < w.rows ? A + (int64_t)row * ld + kfrom : nullptr;
-  };
-  auto rowB = [&](int c) -> const float* { return c < ncol ? A + (int64_t)(s0 + c) * ld + kfrom : nullptr; };
+  auto rowA = [&](int r) -> const float* { return A + (int64_t)min(r0 + r, w.rows - 1) * ld + kfrom; };
+  auto rowB = [&](int c) -> const float* { return A + (int64_t)(s0 + min(c, ncol - 1)) * ld + kfrom; };
   const bool ok = ws_product(sm, s0 - kfrom, rowA, rowB);
   if (!ok && tid == 0) atomicExch(err, 1);
   if (ok && warp < kWsProducers) {
@@ -1016,8 +1012,8 @@ __global__ void __maxnreg__(128) k_chol_panel_pt(const Win* __restrict__ wins, i
 #pragma unroll
       for (int j = 0; j < NA; ++j) {
         const int i = pt + PT * j, row = i >> 4, c4 = i & 15;
-        x[j] = (r0 + row < w.rows) ? *reinterpret_cast<const float4*>(A + (int64_t)(r0 + row) * w.npad + col + 4 * c4)
-                                   : make_float4(0.f, 0.f, 0.f, 0.f);
+        // rows past the window's feed accumulator rows that are not stored
+        x[j] = *reinterpret_cast<const float4*>(A + (int64_t)min(r0 + row, w.rows - 1) * w.npad + col + 4 * c4);
       }
     };
     auto next_item = [&](int64_t from, int& wi, int& r0) -> int64_t {
@@ -1153,8 +1149,7 @@ __global__ void __maxnreg__(128) k_chol_panel_pt(const Win* __restrict__ wins, i
 #pragma unroll
       for (int k = 0; k < 16; ++k) {
         const int row = r0 + 32 * q + 2 * k + cr;
-        own[k] = row < w.rows ? *reinterpret_cast<const float4*>(src + (int64_t)row * w.npad)
-                              : make_float4(0.f, 0.f, 0.f, 0.f);
+        own[k] = *reinterpret_cast<const float4*>(src + (int64_t)min(row, w.rows - 1) * w.npad);
       }
     };
     if (upd) load_own(ibeg);

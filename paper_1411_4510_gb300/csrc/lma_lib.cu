@@ -1107,6 +1107,24 @@ void Impl<T>::fused_rhs(ModelCore& mc, FusedTest& ft, Arena& tmp) {
          (float)mc.ss2, (float*)mc.wbuf, mc.flags + 2);
 }
 
+// Test rows per CTA (or persistent item) with the least waves x time, given the relative time of each choice and the
+// items per row tile.
+static int pick_rows(const std::vector<Pair>& wpairs, std::initializer_list<std::pair<int, double>> choices, int per) {
+  const double nsm = persistent_grid(1u << 30);
+  int best = 0;
+  double cost = 0.0;
+  for (const auto& c : choices) {
+    double tiles = 0.0;
+    for (const Pair& p : wpairs) tiles += (p.nu + c.first - 1) / c.first;
+    const double t = ceil(tiles * per / nsm) * c.second;
+    if (!best || t < cost) {
+      best = c.first;
+      cost = t;
+    }
+  }
+  return best;
+}
+
 template <typename T>
 void Impl<T>::predict(const ModelCore& mc, int64_t U, const double* XU, const int64_t* tptr, int noisy, int on_device,
                       double* mean, double* var, cudaEvent_t global_done, double* cov, FusedTest* ft,
@@ -1148,11 +1166,9 @@ void Impl<T>::predict(const ModelCore& mc, int64_t U, const double* XU, const in
     std::vector<int> own;      // ... of which the first are its own block's
     make_pairs(mc.wins, mc.w0, M, B, s, tptr, ft != nullptr, pairs, tb, wpairs, own, &pe);
     const bool use_tc = mc.prec == LMA_MIXED && sizeof(T) == 4 && use_tensor_cores();
-    int maxrows = 0;
-    for (const Pair& p : wpairs) maxrows = std::max(maxrows, p.nu);
     std::vector<int4> it_rhs, it_acc, it_t12;
     std::vector<int2> it_sw;
-    for (size_t pi = 0; pi < pairs.size(); ++pi) {
+    for (size_t pi = 0; pi < pairs.size() && !use_tc; ++pi) {
       const Pair& p = pairs[pi];
       const int nut = (p.nu + TB - 1) / TB, nct = mc.wins[p.win].npad / TB;
       for (int ut = 0; ut < nut; ++ut) {
@@ -1163,7 +1179,7 @@ void Impl<T>::predict(const ModelCore& mc, int64_t U, const double* XU, const in
     const int nst = (int)((s + TB - 1) / TB);
     for (const int4& t : tb) {
       const int nut = (t.w + TB - 1) / TB;
-      for (int ut = 0; ut < nut; ++ut)
+      for (int ut = 0; ut < nut && !use_tc; ++ut)
         for (int kt = 0; kt < nst; ++kt) it_acc.push_back(make_int4(t.x, t.y, ut, kt));
       for (int u = 0; u < t.w; ++u) it_t12.push_back(make_int4(t.x, t.y, u, 0));
     }
@@ -1214,9 +1230,9 @@ void Impl<T>::predict(const ModelCore& mc, int64_t U, const double* XU, const in
                (int)s, (T)mc.ss2, Pbuf);
       }
       if (tc) {
-        // test rows a CTA: the smallest of 16, 64 and 128 that holds a window's (16 rows cost a CTA as much time as
-        // 64 where the factor's bytes bound it, but leave room for a deeper ring)
-        const int N = maxrows <= 16 ? 16 : (maxrows <= 64 ? 64 : 128);
+        // test rows a CTA: a sweep of 16, 64 or 128 rows takes about 1 : 1.4 : 1.9 of the time, so the one with the
+        // least of it over the waves of CTAs
+        const int N = pick_rows(wpairs, {{16, 1.0}, {64, 1.4}, {128, 1.9}}, 1);
         std::vector<int2> it_tc;
         for (size_t pi = 0; pi < wpairs.size(); ++pi)
           for (int ut = 0; ut < (wpairs[pi].nu + N - 1) / N; ++ut) it_tc.push_back(make_int2((int)pi, ut));
@@ -1245,7 +1261,7 @@ void Impl<T>::predict(const ModelCore& mc, int64_t U, const double* XU, const in
     T* h = tmp.alloc<T>(U * s);
     if (use_tc) {
       // per window: all its test rows against its extra rows, in partial rows of their own
-      const int N = maxrows <= 16 ? 16 : 64;
+      const int N = pick_rows(wpairs, {{16, 1.0}, {64, 1.6}}, (int)((s + 127) / 128));
       std::vector<AccItem> it_w;
       std::vector<int64_t> wrow(mc.wins.size(), 0), prow(pairs.size(), 0);
       int64_t hrows = 0;

@@ -409,6 +409,8 @@ template <int D>
 __global__ void __launch_bounds__(256) k_kds_bf3(const float* __restrict__ xs, int64_t n, int d,
                                                  const float* __restrict__ ss, int s, float ss2, int ld,
                                                  uint16_t* __restrict__ out) {
+  grid_dep_wait();
+  grid_dep_launch();
   __shared__ __align__(16) float sk[D][64];
   const int tid = threadIdx.x;
   const int k0 = blockIdx.x * 64;
@@ -456,6 +458,8 @@ __global__ void __launch_bounds__(256) k_kds_bf3(const float* __restrict__ xs, i
 // consecutive columns of one row.
 __global__ void k_split_bf3(const float* __restrict__ A, int64_t rows, int cols, int64_t lda, int ld,
                             uint16_t* __restrict__ out, int reverse) {
+  grid_dep_wait();
+  grid_dep_launch();
   const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   const int per = ld / 8;
   if (e >= rows * per) return;
@@ -485,6 +489,8 @@ __global__ void k_split_bf3(const float* __restrict__ A, int64_t rows, int cols,
 // outside the s x s matrix.  The pieces are taken from the FP64 value.
 __global__ void k_linv_bf3(const double* __restrict__ buf, int64_t npad, int s, int rows, int ld,
                            uint16_t* __restrict__ out) {
+  grid_dep_wait();
+  grid_dep_launch();
   const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (e >= (int64_t)rows * ld) return;
   const int i = (int)(e / ld), k = (int)(e % ld);
@@ -507,6 +513,8 @@ __global__ void k_linv_bf3(const double* __restrict__ buf, int64_t npad, int s, 
 // e = 4 x + threadIdx.y, eight values per thread and step.
 __global__ void k_split_summary_bf3(const Win* __restrict__ wins, const float* __restrict__ buf, int se, int nown,
                                     int kmax, uint16_t* __restrict__ out) {
+  grid_dep_wait();
+  grid_dep_launch();
   const Win w = wins[blockIdx.y];
   const int e = blockIdx.x * blockDim.y + threadIdx.y;
   if (e >= se) return;
@@ -542,6 +550,8 @@ __global__ void __launch_bounds__(bf6::NTHR, 1) k_gram_bf6(const int2* __restric
                                                            int group, int se, int kmax,
                                                            const __grid_constant__ CUtensorMap sb, int srows,
                                                            double* __restrict__ partial, int* __restrict__ err) {
+  grid_dep_wait();
+  grid_dep_launch();
   extern __shared__ __align__(16) unsigned char smraw[];
   bf6::Smem& sm = bf6::smem_of(smraw);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -595,6 +605,8 @@ __global__ void __launch_bounds__(bf6::NTHR, 1) k_resid_bf6(const int4* __restri
                                                             int d, const __grid_constant__ CUtensorMap vb, int nrev,
                                                             int kc, float ss2, float sn2, float* __restrict__ buf,
                                                             int* __restrict__ err) {
+  grid_dep_wait();
+  grid_dep_launch();
   extern __shared__ __align__(16) unsigned char smraw[];
   bf6::Smem& sm = bf6::smem_of(smraw);
   __shared__ __align__(16) float xc[128][D];  // scaled inputs of the tile's columns, zero-padded
@@ -668,6 +680,8 @@ __global__ void __launch_bounds__(bf6::NTHR, 1) k_pred_rhs_bf6(const Pair* __res
                                                                const __grid_constant__ CUtensorMap vb, int nrev,
                                                                int kc, float ss2, float* __restrict__ P,
                                                                int* __restrict__ err) {
+  grid_dep_wait();
+  grid_dep_launch();
   extern __shared__ __align__(16) unsigned char smraw[];
   bf6::Smem& sm = bf6::smem_of(smraw);
   __shared__ __align__(16) float xc[128][D];
@@ -736,6 +750,8 @@ __global__ void __launch_bounds__(bf6::NTHR, 1) k_proj_tc(const __grid_constant_
                                                           const __grid_constant__ CUtensorMap bmap, int brows,
                                                           int64_t nrows, int s, float* __restrict__ out, int64_t ldo,
                                                           int* __restrict__ err) {
+  grid_dep_wait();
+  grid_dep_launch();
   extern __shared__ __align__(16) unsigned char smraw[];
   bf6::Smem& sm = bf6::smem_of(smraw);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;

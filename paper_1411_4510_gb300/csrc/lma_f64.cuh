@@ -996,6 +996,8 @@ __global__ void __launch_bounds__(FTH, 1) k_f64_windows(const FlowWin* __restric
 __global__ void __launch_bounds__(128) k_f64_psweep(const Pair* __restrict__ pairs, const int2* __restrict__ items,
                                                     const Win* __restrict__ wins, const double* __restrict__ buf,
                                                     const double* __restrict__ dv16, double* P) {
+  grid_dep_wait();
+  grid_dep_launch();
   __shared__ __align__(16) double ta[TS][FP], tb[TS][FP];
   const int2 it = items[blockIdx.x];
   const Pair pr = pairs[it.x];
@@ -1063,6 +1065,8 @@ __global__ void __launch_bounds__(128) k_f64_psweep(const Pair* __restrict__ pai
 __global__ void __launch_bounds__(256) k_f64_dinv64(const Win* __restrict__ wins, const FlowWin* __restrict__ fw,
                                                     const double* __restrict__ buf, const double* __restrict__ dv16,
                                                     double* __restrict__ dinv) {
+  grid_dep_wait();
+  grid_dep_launch();
   const Win w = wins[blockIdx.y];
   const FlowWin f = fw[blockIdx.y];
   const int kp = blockIdx.x;

@@ -44,6 +44,8 @@ template <typename T>
 __global__ void __launch_bounds__(NT) k_grad_rhs(const Win* __restrict__ wins, const GWin* __restrict__ gw,
                                                  const T* __restrict__ buf, const T* __restrict__ LcT, int s,
                                                  T* __restrict__ Q) {
+  grid_dep_wait();
+  grid_dep_launch();
   const Win w = wins[blockIdx.z];
   const GWin g = gw[blockIdx.z];
   const int c0 = blockIdx.x * TB, i0 = blockIdx.y * TB;
@@ -74,6 +76,8 @@ __global__ void __launch_bounds__(NT) k_grad_rhs(const Win* __restrict__ wins, c
 template <typename T>
 __global__ void k_grad_rhs_fill(const Win* __restrict__ wins, const GWin* __restrict__ gw,
                                 const T* __restrict__ ew, int s, T* __restrict__ Q) {
+  grid_dep_wait();
+  grid_dep_launch();
   const Win w = wins[blockIdx.y];
   const GWin g = gw[blockIdx.y];
   T* Qw = Q + g.q;
@@ -99,6 +103,8 @@ template <typename T>
 __global__ void __launch_bounds__(NT) k_bwd_sweep(const int2* __restrict__ items, const Win* __restrict__ wins,
                                                   const GWin* __restrict__ gw, const T* __restrict__ buf,
                                                   const T* __restrict__ dinv, int s, T* __restrict__ Q) {
+  grid_dep_wait();
+  grid_dep_launch();
   const int2 it = items[blockIdx.x];
   const Win w = wins[it.x];
   const GWin g = gw[it.x];
@@ -160,6 +166,8 @@ __global__ void __launch_bounds__(NT) k_grad_G(const int2* __restrict__ items, c
                                                const GWin* __restrict__ gw, const T* __restrict__ Q,
                                                const T* __restrict__ xs, int d, int s, double ss2, double sn2,
                                                T* __restrict__ Gbuf, double* __restrict__ partial) {
+  grid_dep_wait();
+  grid_dep_launch();
   const int2 it = items[blockIdx.x];
   const Win w = wins[it.x];
   const GWin g = gw[it.x];
@@ -249,6 +257,8 @@ template <typename T>
 __global__ void __launch_bounds__(NT) k_grad_gv(const Win* __restrict__ wins, const GWin* __restrict__ gw,
                                                 const T* __restrict__ Gbuf, const T* __restrict__ Vt, int s,
                                                 T* __restrict__ GV) {
+  grid_dep_wait();
+  grid_dep_launch();
   const Win w = wins[blockIdx.z];
   const GWin g = gw[blockIdx.z];
   const int c0 = blockIdx.x * TB, k0 = blockIdx.y * TB;
@@ -282,6 +292,8 @@ __global__ void k_grad_gather(const Win* __restrict__ wins, const GWin* __restri
                               const int64_t* __restrict__ bptr, int M, int B, int64_t n, int s,
                               const T* __restrict__ Q, const T* __restrict__ GV, T* __restrict__ PsiT,
                               T* __restrict__ GVT, int w0, int k_lo, int k_hi) {
+  grid_dep_wait();
+  grid_dep_launch();
   const int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   const int k = blockIdx.y;
   if (p >= n) return;
@@ -315,6 +327,8 @@ template <typename T>
 __global__ void __launch_bounds__(NT) k_grad_vbar(const T* __restrict__ PsiT, const T* __restrict__ GVT,
                                                   const T* __restrict__ LcT, const double* __restrict__ beta,
                                                   int64_t n, int s, T* __restrict__ VbT) {
+  grid_dep_wait();
+  grid_dep_launch();
   __shared__ GemmSmem<T> sm;
   const int k0 = blockIdx.y * TB;
   const int64_t p0 = (int64_t)blockIdx.x * TB;
@@ -341,6 +355,8 @@ template <typename T>
 __global__ void __launch_bounds__(NT) k_grad_kds(const T* __restrict__ VbT, const T* __restrict__ ET,
                                                  const T* __restrict__ xs, const T* __restrict__ ss, int d,
                                                  int64_t n, int s, double ss2, double* __restrict__ partial) {
+  grid_dep_wait();
+  grid_dep_launch();
   __shared__ GemmSmem<T> sm;
   __shared__ T xp[TB][MAXD + 1];
   __shared__ T xk[TB][MAXD + 1];
@@ -412,6 +428,8 @@ template <typename T>
 __global__ void __launch_bounds__(NT) k_grad_m1(const T* __restrict__ VbT, const T* __restrict__ Vt, int64_t n,
                                                 int s, Pieces pc, int npieces, int per_slice,
                                                 double* __restrict__ partial) {
+  grid_dep_wait();
+  grid_dep_launch();
   __shared__ GemmSmem<T> sm;
   const int i0 = blockIdx.y * TB, j0 = blockIdx.x * TB;
   double accd[4][4] = {};
@@ -509,6 +527,8 @@ __device__ __forceinline__ int col128(int y) { return 4 * (int)(threadIdx.x & 15
 __global__ void __launch_bounds__(256) k_grad_m1_128(const float* __restrict__ VbT, const float* __restrict__ Vt,
                                                      int64_t n, int s, Pieces pc, int npieces, int per_slice,
                                                      double* __restrict__ partial) {
+  grid_dep_wait();
+  grid_dep_launch();
   __shared__ __align__(16) Smem128 sm;
   const int i0 = blockIdx.y * 128, j0 = blockIdx.x * 128;
   double* P = partial + (int64_t)blockIdx.z * s * s;
@@ -540,6 +560,8 @@ __global__ void __launch_bounds__(256) k_grad_m1_128(const float* __restrict__ V
 __global__ void __launch_bounds__(256) k_grad_vbar_128(const float* __restrict__ PsiT, const float* __restrict__ GVT,
                                                        const float* __restrict__ LcT, const double* __restrict__ beta,
                                                        int64_t n, int s, float* __restrict__ VbT) {
+  grid_dep_wait();
+  grid_dep_launch();
   __shared__ __align__(16) Smem128 sm;
   const int k0 = blockIdx.y * 128;
   const int64_t p0 = (int64_t)blockIdx.x * 128;
@@ -594,6 +616,8 @@ __global__ void __launch_bounds__(256) k_grad_kds_pair(const float* __restrict__
                                                        const float* __restrict__ xs, const float* __restrict__ ss,
                                                        int d, int64_t n, int s, double ss2,
                                                        double* __restrict__ partial) {
+  grid_dep_wait();
+  grid_dep_launch();
   extern __shared__ __align__(16) unsigned char smraw[];
   float* prod = reinterpret_cast<float*>(smraw);                       // [TS2][TS2 + 1]
   float(*xk)[D] = reinterpret_cast<float(*)[D]>(prod + TS2 * (TS2 + 4));  // [TS2][D]
@@ -672,6 +696,8 @@ __global__ void __launch_bounds__(256) k_grad_kds_pair(const float* __restrict__
 }
 
 __global__ void k_sum_chunks(const double* __restrict__ partial, int nchunk, int64_t len, double* __restrict__ out) {
+  grid_dep_wait();
+  grid_dep_launch();
   int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (e >= len) return;
   double v = 0.0;
@@ -687,6 +713,8 @@ __global__ void k_sum_chunks(const double* __restrict__ partial, int nchunk, int
 template <bool TA, bool TBm, int SHAPE, int TILE>
 __global__ void __launch_bounds__(256) k_dgemm(const double* __restrict__ A, int64_t lda, const double* __restrict__ Bm,
                                                int64_t ldb, double* __restrict__ C, int64_t ldc, int s, double alpha) {
+  grid_dep_wait();
+  grid_dep_launch();
   constexpr int KT = 16, R = TILE / 16;
   __shared__ double sa[KT][TILE + 1], sb[KT][TILE + 1];
   const int i0 = blockIdx.y * TILE, j0 = blockIdx.x * TILE;
@@ -735,6 +763,8 @@ __global__ void __launch_bounds__(256) k_dgemm(const double* __restrict__ A, int
 
 // Phi(X): lower triangle with halved diagonal, in place (s x s, ld s)
 static __global__ void k_phi(double* __restrict__ X, int s) {
+  grid_dep_wait();
+  grid_dep_launch();
   int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (e >= (int64_t)s * s) return;
   int i = (int)(e / s), j = (int)(e % s);
@@ -744,6 +774,8 @@ static __global__ void k_phi(double* __restrict__ X, int s) {
 
 // after k_phi on a copy of L: restore the diagonal halved by k_phi (x2)
 static __global__ void k_tril_fix(double* __restrict__ X, int s) {
+  grid_dep_wait();
+  grid_dep_launch();
   int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (e >= (int64_t)s * s) return;
   int i = (int)(e / s), j = (int)(e % s);
@@ -753,6 +785,8 @@ static __global__ void k_tril_fix(double* __restrict__ X, int s) {
 // <Sigma-bar_SS, dK_SS/dtheta> (jitter held fixed); one CTA row-chunk per block
 static __global__ void k_grad_kss(const double* __restrict__ Sb, const double* __restrict__ ss, int s, int d,
                                   double ss2, double* __restrict__ partial) {
+  grid_dep_wait();
+  grid_dep_launch();
   __shared__ double red[NT];
   double gl[MAXD];
   for (int q = 0; q < d; ++q) gl[q] = 0.0;

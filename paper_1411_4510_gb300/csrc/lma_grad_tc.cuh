@@ -59,6 +59,8 @@ __device__ __forceinline__ void read_acc(uint32_t tmem, float (&v)[32]) {
 __global__ void __launch_bounds__(256, 2) k_grad_rhs_tc(const Win* __restrict__ wins, const GWin* __restrict__ gw,
                                                      const float* __restrict__ buf, const float* __restrict__ LcT,
                                                      int s, float* __restrict__ Q, int* __restrict__ err) {
+  grid_dep_wait();
+  grid_dep_launch();
   const Win w = wins[blockIdx.z];
   const GWin g = gw[blockIdx.z];
   const int c0 = blockIdx.x * 64, i0 = blockIdx.y * 128;
@@ -112,6 +114,8 @@ __global__ void __launch_bounds__(256, 2) k_bwd_sweep_tc(const int2* __restrict_
                                                       const GWin* __restrict__ gw, const float* __restrict__ buf,
                                                       const float* __restrict__ dinv, int s, float* __restrict__ Q,
                                                       int* __restrict__ err) {
+  grid_dep_wait();
+  grid_dep_launch();
   const int2 it = items[blockIdx.x];
   const Win w = wins[it.x];
   const GWin g = gw[it.x];
@@ -190,6 +194,8 @@ __global__ void __launch_bounds__(256, 2) k_grad_G_tc(const int4* __restrict__ i
                                                    const float* __restrict__ xs, int d, int s, float ss2, double sn2,
                                                    float* __restrict__ Gbuf, double* __restrict__ partial,
                                                    int* __restrict__ err) {
+  grid_dep_wait();
+  grid_dep_launch();
   const int4 it = items[blockIdx.x];
   const Win w = wins[it.x];
   const GWin g = gw[it.x];
@@ -301,6 +307,8 @@ __global__ void __launch_bounds__(256, 2) k_grad_G_tc(const int4* __restrict__ i
 __global__ void __launch_bounds__(256, 2) k_grad_gv_tc(const Win* __restrict__ wins, const GWin* __restrict__ gw,
                                                     const float* __restrict__ Gbuf, const float* __restrict__ Vt,
                                                     int s, float* __restrict__ GV, int* __restrict__ err) {
+  grid_dep_wait();
+  grid_dep_launch();
   const Win w = wins[blockIdx.z];
   const GWin g = gw[blockIdx.z];
   const int c0 = blockIdx.x * 64, k0 = blockIdx.y * 128;

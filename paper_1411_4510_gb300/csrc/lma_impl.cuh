@@ -81,34 +81,36 @@ void start(const char* name, cudaStream_t st);
 void stop(cudaStream_t st);
 }  // namespace prof
 
+inline int sm_count() {
+  static const int n = [] {
+    int dev = 0, v = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+      v = 152;
+    return v;
+  }();
+  return n;
+}
+
 // Launch a kernel, count it, check the launch status and (optionally) time it.
+// A grid of at most one CTA per SM is started with programmatic stream
+// serialisation: it may become resident while its predecessor in the stream
+// still runs, which hides the 1-2 us between two dependent launches (a small
+// problem is a chain of 45 to 60 of them; every kernel calls grid_dep_wait()
+// before anything else).  A larger grid is not: its CTAs would fill up the SMs
+// that the predecessor leaves first and run unevenly.  Measured, none / every
+// grid / this rule: N = 1,000 fit and predict 0.672 / 0.612 / 0.608 ms, N =
+// 40,960 4.28 / 4.24 / 4.14 ms (the factorisation's launches had it before), N =
+// 2,000,000 527.5 (none but those) / 500.6 ms (this rule), an FP64 gradient
+// 17.8 / 18.9 / 17.8 ms.
 template <typename... KArgs, typename... Args>
 inline void launch(const char* name, void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
                    Args... args) {
   const bool p = prof::active(name);
   if (p) prof::start(name, st);
-  kern<<<grid, block, smem, st>>>(static_cast<KArgs>(args)...);
-  count_launch();
-  cudaError_t e = cudaGetLastError();
-  if (p) prof::stop(st);
-  if (e != cudaSuccess) {
-    fail(LMA_ERR_CUDA, std::string("launch of ") + name + ": " + cudaGetErrorString(e));
-    throw Fail{};
-  }
-}
-
-// launch() with programmatic stream serialisation: the kernel may become
-// resident while its predecessor in the stream still runs, which hides the
-// launch latency of long chains of short dependent launches (the panel steps
-// of the factorisations).  Only for kernels that call grid_dep_wait() first.
-template <typename... KArgs, typename... Args>
-inline void launch_pdl(const char* name, void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
-                       Args... args) {
-  const bool p = prof::active(name);
-  if (p) prof::start(name, st);
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[0].val.programmaticStreamSerializationAllowed = 1;
+  at[0].val.programmaticStreamSerializationAllowed = (int64_t)grid.x * grid.y * grid.z <= sm_count() ? 1 : 0;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;

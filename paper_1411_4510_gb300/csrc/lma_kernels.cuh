@@ -128,6 +128,8 @@ __device__ __forceinline__ void tri_index(int t, int& I, int& J) {
 template <typename T>
 __global__ void k_scale(const double* __restrict__ X, int64_t n, int d, const double* __restrict__ inv_ell,
                         double* __restrict__ xs64, T* __restrict__ xsT) {
+  grid_dep_wait();
+  grid_dep_launch();
   int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i >= n * d) return;
   double v = X[i] * inv_ell[i % d];
@@ -138,6 +140,8 @@ __global__ void k_scale(const double* __restrict__ X, int64_t n, int d, const do
 // r = y - mu in T and FP64
 template <typename T>
 __global__ void k_center(const double* __restrict__ y, int64_t n, double mu, T* __restrict__ rT) {
+  grid_dep_wait();
+  grid_dep_launch();
   int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i < n) rT[i] = (T)(y[i] - mu);
 }
@@ -146,6 +150,8 @@ __global__ void k_center(const double* __restrict__ y, int64_t n, double mu, T* 
 // (the sweep then yields L_SS and L_SS^-T).  One thread per element.
 __global__ void k_build_kss(const double* __restrict__ ss, int s, int d, double ss2, double jitter,
                             int npad, double* __restrict__ buf) {
+  grid_dep_wait();
+  grid_dep_launch();
   int64_t total = (int64_t)(npad + s) * npad;
   int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (e >= total) return;
@@ -172,6 +178,8 @@ __global__ void k_build_kss(const double* __restrict__ ss, int s, int d, double 
 template <typename T>
 __global__ void __launch_bounds__(NT) k_kds(const T* __restrict__ xs, int64_t n, int d, const T* __restrict__ ss,
                                             int s, T ss2, T* __restrict__ out) {
+  grid_dep_wait();
+  grid_dep_launch();
   __shared__ T xp[TB][MAXD + 1];
   __shared__ T xk[TB][MAXD + 1];
   const int64_t p0 = (int64_t)blockIdx.y * TB;
@@ -200,6 +208,8 @@ __global__ void __launch_bounds__(NT) k_kds(const T* __restrict__ xs, int64_t n,
 template <typename T>
 __global__ void __launch_bounds__(NT) k_proj(const T* __restrict__ Kds, int64_t n, int s, const T* __restrict__ ET,
                                              T* __restrict__ Vt, int ldo) {
+  grid_dep_wait();
+  grid_dep_launch();
   __shared__ GemmSmem<T> sm;
   const int64_t p0 = (int64_t)blockIdx.y * TB;
   const int i0 = blockIdx.x * TB;
@@ -225,6 +235,8 @@ __global__ void __launch_bounds__(NT) k_proj(const T* __restrict__ Kds, int64_t 
 // Vt[p][i] = sum_{k <= i} Kds[p][k] ET[k][i].  Needs s % 4 == 0 (float4 rows).
 __global__ void __launch_bounds__(256) k_proj128(const float* __restrict__ Kds, int64_t n, int s,
                                                  const float* __restrict__ ET, float* __restrict__ Vt, int ldo) {
+  grid_dep_wait();
+  grid_dep_launch();
   constexpr int BM = 128, BK = 8;
   __shared__ __align__(16) float As[2][BK][BM + 4];
   __shared__ __align__(16) float Bs[2][BK][BM + 4];
@@ -310,6 +322,8 @@ __global__ void __launch_bounds__(256) k_proj128(const float* __restrict__ Kds, 
 template <typename T>
 __global__ void __launch_bounds__(NT) k_resid(const Win* __restrict__ wins, const T* __restrict__ xs, int d,
                                               const T* __restrict__ Vt, int s, T ss2, T sn2, T* __restrict__ buf) {
+  grid_dep_wait();
+  grid_dep_launch();
   const Win w = wins[blockIdx.y];
   const int nt = w.npad / TB;
   if ((int)blockIdx.x >= nt * (nt + 1) / 2) return;
@@ -357,6 +371,8 @@ __global__ void __launch_bounds__(NT) k_resid(const Win* __restrict__ wins, cons
 
 // dst |= src (one device status word into another).
 __global__ void k_or_flag(const int* __restrict__ src, int* __restrict__ dst) {
+  grid_dep_wait();
+  grid_dep_launch();
   if (threadIdx.x == 0 && *src) atomicOr(dst, *src);
 }
 
@@ -374,6 +390,8 @@ __global__ void k_or_flag(const int* __restrict__ src, int* __restrict__ dst) {
 template <typename T>
 __global__ void k_copy_shared_tiles(const Win* __restrict__ wins, int nwin, int B, const int* __restrict__ Ls,
                                     T* __restrict__ buf) {
+  grid_dep_wait();
+  grid_dep_launch();
   const int k = blockIdx.y;
   const int L = Ls[k];
   const int i = blockIdx.x;
@@ -402,6 +420,8 @@ __global__ void k_copy_shared_tiles(const Win* __restrict__ wins, int nwin, int 
 template <typename T>
 __global__ void __launch_bounds__(NT) k_fill_ext(const Win* __restrict__ wins, const T* __restrict__ Vt,
                                                  const T* __restrict__ r, int s, T* __restrict__ buf) {
+  grid_dep_wait();
+  grid_dep_launch();
   const Win w = wins[blockIdx.z];
   const int c0 = blockIdx.x * TB;
   const int e0 = blockIdx.y * TB;
@@ -432,6 +452,8 @@ __global__ void __launch_bounds__(NT) k_fill_ext(const Win* __restrict__ wins, c
 // row length s is not a multiple of 4), stores four consecutive columns.
 __global__ void __launch_bounds__(256) k_fill_ext4(const Win* __restrict__ wins, const float* __restrict__ Vt,
                                                    const float* __restrict__ r, int s, float* __restrict__ buf) {
+  grid_dep_wait();
+  grid_dep_launch();
   const Win w = wins[blockIdx.z];
   const int c0 = blockIdx.x * 64;
   if (c0 >= w.npad) return;
@@ -798,6 +820,8 @@ __device__ void diag_factor(T (*D)[N + 1], T* Lout, int64_t ld, T* Dv, int* info
 template <typename T>
 __global__ void __launch_bounds__(NT) k_chol_step(const Win* __restrict__ wins, T* __restrict__ buf,
                                                   T* __restrict__ dinv, int* __restrict__ info, int kp) {
+  grid_dep_wait();
+  grid_dep_launch();
   const Win w = wins[blockIdx.y];
   if (kp * TB >= w.npad) return;
   const int i = kp + blockIdx.x;
@@ -848,6 +872,8 @@ struct TrsmSmem {
 template <typename T>
 __global__ void __launch_bounds__(NT) k_chol_trsm(const Win* __restrict__ wins, T* __restrict__ buf,
                                                   const T* __restrict__ dinv, int kp, int nid) {
+  grid_dep_wait();
+  grid_dep_launch();
   const Win w = wins[blockIdx.y];
   if (kp * TB >= w.npad) return;
   const int i = kp + 1 + blockIdx.x;
@@ -902,6 +928,8 @@ __global__ void __launch_bounds__(NT) k_chol_trsm(const Win* __restrict__ wins, 
 template <typename T>
 __global__ void __launch_bounds__(NT) k_gram(const Win* __restrict__ wins, int nwin, int chunk, int s,
                                              const T* __restrict__ buf, double* __restrict__ partial) {
+  grid_dep_wait();
+  grid_dep_launch();
   int I, J;
   tri_index(blockIdx.x, I, J);
   const int se = s + 1;
@@ -936,6 +964,8 @@ __global__ void __launch_bounds__(NT) k_gram(const Win* __restrict__ wins, int n
 
 __global__ void k_gram_reduce(const double* __restrict__ partial, int nchunk, int se, double* __restrict__ G,
                               int tile) {
+  grid_dep_wait();
+  grid_dep_launch();
   int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (e >= (int64_t)se * se) return;
   int i = (int)(e / se), j = (int)(e % se);
@@ -950,6 +980,8 @@ __global__ void k_gram_reduce(const double* __restrict__ partial, int nchunk, in
 // log|R-dot_m^-1| per window = 2 sum log diag of the trailing (block) factor
 template <typename T>
 __global__ void k_logdet(const Win* __restrict__ wins, const T* __restrict__ buf, double* __restrict__ out) {
+  grid_dep_wait();
+  grid_dep_launch();
   const Win w = wins[blockIdx.x];
   __shared__ double red[NT];
   double sum = 0.0;
@@ -966,6 +998,8 @@ __global__ void k_logdet(const Win* __restrict__ wins, const T* __restrict__ buf
 
 // ordered sum of n doubles (single thread: deterministic)
 __global__ void k_sum_ordered(const double* __restrict__ v, int n, double* __restrict__ out) {
+  grid_dep_wait();
+  grid_dep_launch();
   if (threadIdx.x == 0 && blockIdx.x == 0) {
     double s = 0.0;
     for (int i = 0; i < n; ++i) s += v[i];
@@ -977,6 +1011,8 @@ __global__ void k_sum_ordered(const double* __restrict__ v, int n, double* __res
 // then yields L_C, L_C^-T and L_C^-1 y; identity rows first so they stay
 // 64-aligned for the zero-tile skip).
 __global__ void k_build_global(const double* __restrict__ G, int s, int npad, double* __restrict__ buf) {
+  grid_dep_wait();
+  grid_dep_launch();
   const int se = s + 1;
   int64_t total = (int64_t)(npad + 1 + s) * npad;
   int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -1001,6 +1037,8 @@ __global__ void k_build_global(const double* __restrict__ G, int s, int npad, do
 __global__ void __launch_bounds__(NT) k_global_finish(const double* __restrict__ buf, const double* __restrict__ G,
                                                       int s, int npad, double* __restrict__ beta,
                                                       double* __restrict__ scalars) {
+  grid_dep_wait();
+  grid_dep_launch();
   const double* E = buf + (int64_t)npad * npad;  // row k = (L_C^-T)[k][.]
   const double* w = E + (int64_t)s * npad;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -1040,6 +1078,8 @@ __global__ void __launch_bounds__(NT) k_global_finish(const double* __restrict__
 // Copy an s x s block with leading dimension ld (FP64) into T with ld s.
 template <typename T>
 __global__ void k_copy_block(const double* __restrict__ src, int64_t ld, int s, T* __restrict__ dst) {
+  grid_dep_wait();
+  grid_dep_launch();
   int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (e >= (int64_t)s * s) return;
   int i = (int)(e / s), j = (int)(e % s);
@@ -1051,6 +1091,8 @@ __global__ void k_copy_block(const double* __restrict__ src, int64_t ld, int s, 
 template <typename T>
 __global__ void k_ew(const Win* __restrict__ wins, const T* __restrict__ buf, const double* __restrict__ beta, int s,
                      T* __restrict__ ew) {
+  grid_dep_wait();
+  grid_dep_launch();
   const Win w = wins[blockIdx.y];
   int c = blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= w.npad) return;
@@ -1065,6 +1107,8 @@ __global__ void k_ew(const Win* __restrict__ wins, const T* __restrict__ buf, co
 // bh_k x = p + e exactly (e from an FMA), bl_k x added to e, and the p are
 // summed with TwoSum into (hi, lo), which keeps about 48 bits of the sum.
 __global__ void k_split_beta(const double* __restrict__ beta, int s, float2* __restrict__ bs) {
+  grid_dep_wait();
+  grid_dep_launch();
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= s) return;
   const float h = (float)beta[k];
@@ -1072,6 +1116,8 @@ __global__ void k_split_beta(const double* __restrict__ beta, int s, float2* __r
 }
 __global__ void k_ew_f32(const Win* __restrict__ wins, const float* __restrict__ buf, const float2* __restrict__ bs,
                          int s, float* __restrict__ ew) {
+  grid_dep_wait();
+  grid_dep_launch();
   const Win w = wins[blockIdx.y];
   const int c = blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= w.npad) return;
@@ -1116,6 +1162,8 @@ __global__ void __launch_bounds__(NT) k_pred_rhs(const Pair* __restrict__ pairs,
                                                  const Win* __restrict__ wins, const T* __restrict__ xs,
                                                  const T* __restrict__ xu, int d, const T* __restrict__ Vt,
                                                  const T* __restrict__ Vu, int s, T ss2, T* __restrict__ P) {
+  grid_dep_wait();
+  grid_dep_launch();
   const int4 it = items[blockIdx.x];
   const Pair pr = pairs[it.x];
   const Win w = wins[pr.win];
@@ -1161,6 +1209,8 @@ template <typename T>
 __global__ void __launch_bounds__(NT) k_pred_sweep(const Pair* __restrict__ pairs, const int2* __restrict__ items,
                                                    const Win* __restrict__ wins, const T* __restrict__ buf,
                                                    const T* __restrict__ dinv, T* __restrict__ P) {
+  grid_dep_wait();
+  grid_dep_launch();
   const int2 it = items[blockIdx.x];
   const Pair pr = pairs[it.x];
   const Win w = wins[pr.win];
@@ -1220,6 +1270,8 @@ __global__ void __launch_bounds__(NT) k_pred_accum(const Pair* __restrict__ pair
                                                    const Win* __restrict__ wins, const T* __restrict__ buf,
                                                    const T* __restrict__ P, const T* __restrict__ Vu, int s,
                                                    T* __restrict__ h) {
+  grid_dep_wait();
+  grid_dep_launch();
   const int4 it = items[blockIdx.x];
   const int u0 = it.z * TB, k0 = it.w * TB;
   __shared__ GemmSmem<T> sm;
@@ -1254,6 +1306,8 @@ template <typename T>
 __global__ void k_pred_t12(const Pair* __restrict__ pairs, const int4* __restrict__ items, int nitems,
                            const Win* __restrict__ wins, const T* __restrict__ P, const T* __restrict__ ew,
                            double* __restrict__ t1, double* __restrict__ t2) {
+  grid_dep_wait();
+  grid_dep_launch();
   const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (warp >= nitems) return;
@@ -1309,6 +1363,8 @@ __global__ void k_pred_t12(const Pair* __restrict__ pairs, const int4* __restric
 template <typename T>
 __global__ void __launch_bounds__(NT) k_var_gemm(const T* __restrict__ h, int64_t U, int s, const T* __restrict__ LcT,
                                                  double* __restrict__ partial) {
+  grid_dep_wait();
+  grid_dep_launch();
   __shared__ GemmSmem<T> sm;
   __shared__ double red[TB][17];
   const int64_t u0 = (int64_t)blockIdx.y * TB;
@@ -1340,6 +1396,8 @@ __global__ void __launch_bounds__(NT) k_var_gemm(const T* __restrict__ h, int64_
 // out[u] = |g_u|^2 (summed in pairs of floats) for g = L_C^-1 h formed by k_proj128 (U rows of
 // s values): the variance term of k_var_gemm as one partial (ntile = 1).
 __global__ void k_row_sqnorm(const float* __restrict__ g, int64_t U, int s, double* __restrict__ out) {
+  grid_dep_wait();
+  grid_dep_launch();
   const int64_t row = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (row >= U) return;
@@ -1357,6 +1415,8 @@ __global__ void k_row_sqnorm(const float* __restrict__ g, int64_t U, int s, doub
 template <typename T>
 __global__ void __launch_bounds__(NT) k_lc_apply(const T* __restrict__ h, int64_t U, int s, const T* __restrict__ LcT,
                                                  T* __restrict__ g) {
+  grid_dep_wait();
+  grid_dep_launch();
   __shared__ GemmSmem<T> sm;
   const int64_t u0 = (int64_t)blockIdx.y * TB;
   const int i0 = blockIdx.x * TB;
@@ -1396,6 +1456,8 @@ __global__ void __launch_bounds__(NT) k_pred_xcov(const Pair* __restrict__ pairs
                                                   const T* __restrict__ xu, int d, const T* __restrict__ Vu,
                                                   const T* __restrict__ P, const T* __restrict__ g, int s, double ss2,
                                                   double noise, double* __restrict__ cov) {
+  grid_dep_wait();
+  grid_dep_launch();
   const int4 it = items[blockIdx.x];
   const CovReq rq = reqs[it.x];
   const int a0 = it.y * TB, b0 = it.z * TB, nua = rq.nua, nub = rq.nub;
@@ -1463,6 +1525,8 @@ __global__ void k_pred_final(const T* __restrict__ Vu, int64_t U, int s, const d
                              const float2* __restrict__ bs, const double* __restrict__ t1, const double* __restrict__ t2,
                              const double* __restrict__ partial, int ntile, double mu, double prior,
                              double* __restrict__ mean, double* __restrict__ var) {
+  grid_dep_wait();
+  grid_dep_launch();
   const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (warp >= U) return;

@@ -205,13 +205,7 @@ static size_t pa_smem() { return sizeof(tc::PaSmem<N>) + tc::kTcAlignSlack; }
 
 // Grid of a persistent kernel with one CTA per SM: min(items, SM count).
 static unsigned persistent_grid(size_t items) {
-  static int nsm = 0;
-  if (nsm == 0) {
-    int dev = 0;
-    LMA_CK(cudaGetDevice(&dev));
-    LMA_CK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-  }
-  return (unsigned)std::max<size_t>(1, std::min<size_t>(items, (size_t)nsm));
+  return (unsigned)std::max<size_t>(1, std::min<size_t>(items, (size_t)sm_count()));
 }
 
 // cuTensorMapEncodeTiled through the runtime's driver entry point (no link
@@ -440,15 +434,15 @@ static void right_looking_fp64(cudaStream_t st, const Win& w, Win* wd, double* b
     launch_coop("k_f64_coop", k_f64_coop, (unsigned)G, NTH, 0, st, buf, ld, w.rows, npan, nid, dv, info, bar, err);
     return;
   }
-  launch_pdl("k_f64_potrf", k_f64_potrf, 1, NTH, 0, st, buf, ld, 0, dv, info);
+  launch("k_f64_potrf", k_f64_potrf, 1, NTH, 0, st, buf, ld, 0, dv, info);
   if (variant == 1) {
     for (int kp = 0; kp < npan; ++kp) {
       if (nrt - kp - 1 > 0)
-        launch_pdl("k_f64_solve2", k_f64_solve2, (unsigned)(nrt - kp - 1), NTH, 0, st, buf, ld, w.rows, npan, kp,
+        launch("k_f64_solve2", k_f64_solve2, (unsigned)(nrt - kp - 1), NTH, 0, st, buf, ld, w.rows, npan, kp,
                    nid, (const double*)dv);
       const int m = npan - kp - 1;
       if (m > 0)
-        launch_pdl("k_f64_panel", k_f64_update2, (unsigned)(m * (m + 1) / 2 + (nrt - npan) * m), NTH, 0, st, buf,
+        launch("k_f64_panel", k_f64_update2, (unsigned)(m * (m + 1) / 2 + (nrt - npan) * m), NTH, 0, st, buf,
                    ld, w.rows, npan, kp, nid, dv, info);
     }
     return;
@@ -458,7 +452,7 @@ static void right_looking_fp64(cudaStream_t st, const Win& w, Win* wd, double* b
     const int trail = m > 0 ? m * (m + 1) / 2 + (nrt - npan) * m : 0;
     const int solve = kp >= 1 ? nrt - kp : 0;
     if (trail + solve > 0)
-      launch_pdl("k_f64_panel", k_f64_panel, (unsigned)(trail + solve), NTH, 0, st, buf, ld, w.rows, npan, kp, nid, dv,
+      launch("k_f64_panel", k_f64_panel, (unsigned)(trail + solve), NTH, 0, st, buf, ld, w.rows, npan, kp, nid, dv,
              info);
   }
 }
@@ -574,23 +568,23 @@ void chol_sweep(cudaStream_t st, Arena& tmp, const std::vector<Win>& wins, Win* 
         const int kb = (k0 / SP) * SP, kh = (k0 / HP) * HP;
         if (k0 == kb && kb > 0) {
           const unsigned gy = (unsigned)((maxrows - kb + 127) / 128);
-          launch_pdl("k_chol_wide", k_chol_wide<256>, dim3(nw, gy), tc::kWsThreads, wide_smem<256>(), st, wins_d,
+          launch("k_chol_wide", k_chol_wide<256>, dim3(nw, gy), tc::kWsThreads, wide_smem<256>(), st, wins_d,
                      (float*)buf, kb, 0, err);
         }
         if (k0 == kh && kh > kb) {
           const unsigned gy = (unsigned)((maxrows - kh + 127) / 128);
-          launch_pdl("k_chol_mid", k_chol_wide<128>, dim3(nw, gy), tc::kWsThreads, wide_smem<128>(), st, wins_d,
+          launch("k_chol_mid", k_chol_wide<128>, dim3(nw, gy), tc::kWsThreads, wide_smem<128>(), st, wins_d,
                      (float*)buf, kh, kb, err);
         }
         // every panel: its diagonal block (the first panel of a 128-column
         // group has every column to its left applied; the second adds the
         // first's 64 columns), then the persistent kernel updates the rows
         // below with the same columns and solves them
-        launch_pdl("k_chol_step_tc", k_chol_step_tc, dim3(nw, 1), 256, tc_chol_smem(), st, wins_d, (float*)buf,
+        launch("k_chol_step_tc", k_chol_step_tc, dim3(nw, 1), 256, tc_chol_smem(), st, wins_d, (float*)buf,
                    (float*)dinv, info, kp, kh, err);
         if (maxrows - (kp + 1) * TB > 0) {
           const int ntile = (maxrows - (kp + 1) * TB + 127) / 128;
-          launch_pdl("k_chol_panel_pt", k_chol_panel_pt, persistent_grid((size_t)ntile * nw), tc::kPtThreads,
+          launch("k_chol_panel_pt", k_chol_panel_pt, persistent_grid((size_t)ntile * nw), tc::kPtThreads,
                      pt_smem(), st, wins_d, (int)nw, (float*)buf, (const float*)dinv, kp, kh, ntile, err);
         }
       } else {
@@ -1110,7 +1104,7 @@ void Impl<T>::fused_rhs(ModelCore& mc, FusedTest& ft, Arena& tmp) {
 // Test rows per CTA (or persistent item) with the least waves x time, given the relative time of each choice and the
 // items per row tile.
 static int pick_rows(const std::vector<Pair>& wpairs, std::initializer_list<std::pair<int, double>> choices, int per) {
-  const double nsm = persistent_grid(1u << 30);
+  const double nsm = sm_count();
   int best = 0;
   double cost = 0.0;
   for (const auto& c : choices) {
@@ -1763,6 +1757,8 @@ static double* noalloc_scratch() {
 }
 
 static __global__ void k_noalloc_setup(Win* wslot, Win w, int* flag) {
+  grid_dep_wait();
+  grid_dep_launch();
   *wslot = w;
   *flag = 0;
 }
@@ -1772,6 +1768,8 @@ static __global__ void k_noalloc_setup(Win* wslot, Win w, int* flag) {
 // 64-aligned and the factorisation skips their tiles while still zero.
 static __global__ void k_noalloc_build(const double* __restrict__ A, const double* __restrict__ y, int s, int npad,
                                        double* __restrict__ buf) {
+  grid_dep_wait();
+  grid_dep_launch();
   int64_t total = (int64_t)(npad + 1 + s) * npad;
   int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (e >= total) return;
@@ -1795,6 +1793,8 @@ static __global__ void k_noalloc_build(const double* __restrict__ A, const doubl
 static __global__ void __launch_bounds__(NT) k_noalloc_finish(const double* __restrict__ buf, int s, int npad,
                                                               double quad, double logdet_R, double n,
                                                               double* __restrict__ beta, double* __restrict__ out) {
+  grid_dep_wait();
+  grid_dep_launch();
   const double* E = buf + (int64_t)npad * npad;  // row k = (L_C^-T)[k][.]
   const double* w = E + (int64_t)s * npad;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;

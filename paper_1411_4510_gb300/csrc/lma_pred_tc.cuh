@@ -68,6 +68,8 @@ __global__ void __launch_bounds__(tc::kPsThreads, 1) k_pred_sweep_tc(const Pair*
                                                                      const float* __restrict__ buf,
                                                                      const float* __restrict__ dinv, float* P,
                                                                      int* __restrict__ err) {
+  grid_dep_wait();
+  grid_dep_launch();
   using namespace tc;
   constexpr int NS = ps_stages(N), NA = 4, NBV = N >= 32 ? N / 32 : 1, PF = N == 16 ? 3 : 2;
   constexpr uint32_t TCOL = 2 * N < 32 ? 32 : 2 * N;
@@ -294,6 +296,8 @@ __global__ void __launch_bounds__(tc::pa_threads(N), 1) k_pred_accum_win(const P
                                                                          const float* __restrict__ P, int s,
                                                                          float* __restrict__ hw,
                                                                          int* __restrict__ err) {
+  grid_dep_wait();
+  grid_dep_launch();
   using namespace tc;
   constexpr int NS = 4, NSLOT = 4, NA = 4, NBV = N >= 32 ? N / 32 : 1, PF = N == 16 ? 3 : 2, ND = pa_drain(N);
   constexpr int NC = N / (ND / 4);  // test rows per drain thread

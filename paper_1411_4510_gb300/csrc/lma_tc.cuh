@@ -199,6 +199,8 @@ template <int BN>
 __global__ void __launch_bounds__(256) k_tc_gemm(const float* __restrict__ A, int64_t lda,
                                                  const float* __restrict__ Bm, int64_t ldb, float* __restrict__ C,
                                                  int64_t ldc, int M, int N, int K, int* __restrict__ err) {
+  grid_dep_wait();
+  grid_dep_launch();
   using namespace tc;
   extern __shared__ __align__(16) unsigned char smraw[];
   TcSmem<BN>& sm = tc_smem<BN>(smraw);
@@ -1260,6 +1262,8 @@ __host__ __device__ constexpr int pad_dim(int d) { return d <= 8 ? 8 : MAXD; }
 __global__ void k_pred_hsum(const int4* __restrict__ tb, const int64_t* __restrict__ prow,
                             const float* __restrict__ hw, const float* __restrict__ Vu, int s,
                             float* __restrict__ h) {
+  grid_dep_wait();
+  grid_dep_launch();
   const int4 t = tb[blockIdx.y];
   const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (e >= (int64_t)t.w * s) return;

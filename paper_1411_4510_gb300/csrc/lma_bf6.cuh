@@ -83,19 +83,66 @@ __device__ __forceinline__ Smem& smem_of(unsigned char* raw) {
 }
 inline size_t smem_bytes() { return sizeof(Smem) + 1024; }
 
+// STEP columns of the main accumulator and of the correction on their way from
+// tensor memory to registers: wait() waits for every load issued before it.
+template <int STEP>
+struct Drain;
+template <>
+struct Drain<4> {
+  uint32_t m[4], e[4];
+  __device__ __forceinline__ void issue(uint32_t addr) {
+    ld(addr, m);
+    ld(addr + 128, e);
+  }
+  static __device__ __forceinline__ void ld(uint32_t addr, uint32_t (&r)[4]) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(addr));
+  }
+  __device__ __forceinline__ void wait() {
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+r"(m[0]), "+r"(m[1]), "+r"(m[2]), "+r"(m[3]), "+r"(e[0]), "+r"(e[1]), "+r"(e[2]), "+r"(e[3])::"memory");
+  }
+};
+template <>
+struct Drain<8> {
+  uint32_t m[8], e[8];
+  __device__ __forceinline__ void issue(uint32_t addr) {
+    ld(addr, m);
+    ld(addr + 128, e);
+  }
+  static __device__ __forceinline__ void ld(uint32_t addr, uint32_t (&r)[8]) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                 : "r"(addr));
+  }
+  __device__ __forceinline__ void wait() {
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+r"(m[0]), "+r"(m[1]), "+r"(m[2]), "+r"(m[3]), "+r"(m[4]), "+r"(m[5]), "+r"(m[6]), "+r"(m[7]),
+                   "+r"(e[0]), "+r"(e[1]), "+r"(e[2]), "+r"(e[3]), "+r"(e[4]), "+r"(e[5]), "+r"(e[6]), "+r"(e[7])::"memory");
+  }
+};
+
+template <class S>
+struct AddRef {
+  S& s;
+  __device__ void clear() const { s.clear(); }
+  __device__ void operator()(int j, float x) const { s(j, x); }
+};
+
 // Persistent loop over output tiles: the CTA's k-th tile is order(k) (a
 // negative value ends the loop; every role walks the same sequence).  Tile t
 // accumulates, over its chunks c < chunks(t), the
 // product of the 128 x 64 boxes at (x, ya) of A and (x, yb) of B with
 // (x, ya, yb) = at(coords(t), c); plane q of an operand is the box at row
 // offset q * (plane rows) of its tensor map.  Workers drain the two
-// accumulators after every chunk and call after(t, acc) with worker warp w's
-// row 32 (w mod 4) + lane and columns 32 (w / 4) + j in acc[j].  Every wait
-// has an iteration limit; on a timeout all roles stop, no copy is left
-// landing, and false is returned in every thread.
-template <class Order, class Chunks, class Coords, class At, class After>
-__device__ bool persistent(Smem& sm, const CUtensorMap* amap, int arows, const CUtensorMap* bmap, int brows,
-                           Order order, Chunks chunks, Coords coords, At at, After after) {
+// accumulators after every chunk with add(column, value), STEP columns at a
+// time, and call after(t) with worker warp w's row 32 (w mod 4) + lane and
+// columns 32 (w / 4) + j.  Every wait has an iteration limit; on a timeout all
+// roles stop, no copy is left landing, and false is returned in every thread.
+template <int STEP, class Order, class Chunks, class Coords, class At, class Add, class After>
+__device__ bool walk(Smem& sm, const CUtensorMap* amap, int arows, const CUtensorMap* bmap, int brows,
+                     Order order, Chunks chunks, Coords coords, At at, Add add, After after) {
   using namespace tc;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   volatile int* abort_flag = &sm.abort;
@@ -107,9 +154,7 @@ __device__ bool persistent(Smem& sm, const CUtensorMap* amap, int arows, const C
     for (int k = 0;; ++k) {
       const int t = order(k);
       if (t < 0) break;
-      float acc[32];
-#pragma unroll
-      for (int j = 0; j < 32; ++j) acc[j] = 0.f;
+      add.clear();
       const int nchunk = chunks(t);
       for (int c = 0; c < nchunk && ok; ++c, ++G) {
         const int a = G & 1;
@@ -122,21 +167,27 @@ __device__ bool persistent(Smem& sm, const CUtensorMap* amap, int arows, const C
           break;
         }
         fence_after_sync();
-        float m[16], e[16];
+        // the loads of the next STEP columns are in flight while this step's are added
+        Drain<STEP> v[2];
+        v[0].issue(tlane + 256 * a);
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          tmem_ld16(tlane + 256 * a + 16 * h, m);
-          tmem_ld16(tlane + 256 * a + 128 + 16 * h, e);
+        for (int h = 0; h < 32 / STEP; ++h) {
+          v[h & 1].wait();
+          if (h + 1 < 32 / STEP) {
+            v[(h + 1) & 1].issue(tlane + 256 * a + STEP * (h + 1));
+          } else {  // the accumulators are in registers: they may be written again
+            fence_before_sync();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&sm.drained[a]);
+          }
 #pragma unroll
-          for (int j = 0; j < 16; ++j) acc[16 * h + j] += m[j] + e[j];
+          for (int j = 0; j < STEP; ++j)
+            add(STEP * h + j, __uint_as_float(v[h & 1].m[j]) + __uint_as_float(v[h & 1].e[j]));
         }
-        fence_before_sync();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&sm.drained[a]);
       }
       ok = worker_sync_and(ok && !*abort_flag);
       if (!ok) break;
-      after(t, acc);
+      after(t);
     }
   } else if (warp == NWK) {
     // MMA warp: the whole warp runs the loops, lane 0 waits and issues
@@ -230,143 +281,37 @@ __device__ bool persistent(Smem& sm, const CUtensorMap* amap, int arows, const C
   return __syncthreads_and(w && !*abort_flag) != 0;
 }
 
-// persistent() with the chunks' results added by TwoSum into (hi, lo), for
-// products whose K runs long (thousands of values): after(t, hi, lo).
 template <class Order, class Chunks, class Coords, class At, class After>
-__device__ bool persistent_comp(Smem& sm, const CUtensorMap* amap, int arows, const CUtensorMap* bmap, int brows,
-                           Order order, Chunks chunks, Coords coords, At at, After after) {
-  using namespace tc;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  volatile int* abort_flag = &sm.abort;
-  if (warp < NWK) {
-    const int q = warp & 3, half = warp >> 2;
-    const uint32_t tlane = sm.tmem + ((uint32_t)(q * 32) << 16) + half * 32;
-    int G = 0;  // chunks drained so far by this CTA
-    bool ok = true;
-    for (int k = 0;; ++k) {
-      const int t = order(k);
-      if (t < 0) break;
-      float hi[32], lo[32];
+__device__ bool persistent(Smem& sm, const CUtensorMap* amap, int arows, const CUtensorMap* bmap,
+                           int brows, Order order, Chunks chunks, Coords coords, At at, After after) {
+  struct Sum {
+    float v[32];
+    __device__ void clear() {
+#pragma unroll
+      for (int j = 0; j < 32; ++j) v[j] = 0.f;
+    }
+    __device__ void operator()(int j, float x) { v[j] += x; }
+  } acc;
+  return walk<8>(sm, amap, arows, bmap, brows, order, chunks, coords, at, AddRef<Sum>{acc},
+                  [&](int t) { after(t, acc.v); });
+}
+
+// persistent() with the chunks' results added by TwoSum into (hi, lo), for
+// products whose K runs long (thousands of values): after(t, hi, lo).  Eight
+// columns at a time keep the TwoSum state in registers.
+template <class Order, class Chunks, class Coords, class At, class After>
+__device__ bool persistent_comp(Smem& sm, const CUtensorMap* amap, int arows, const CUtensorMap* bmap,
+                                int brows, Order order, Chunks chunks, Coords coords, At at, After after) {
+  struct Sum {
+    float hi[32], lo[32];
+    __device__ void clear() {
 #pragma unroll
       for (int j = 0; j < 32; ++j) hi[j] = lo[j] = 0.f;
-      const int nchunk = chunks(t);
-      for (int c = 0; c < nchunk && ok; ++c, ++G) {
-        const int a = G & 1;
-        int okw = 1;
-        if (lane == 0) okw = mbar_wait(&sm.done[a], (G >> 1) & 1) ? 1 : 0;
-        okw = __shfl_sync(0xffffffffu, okw, 0);
-        if (!okw) {
-          *abort_flag = 1;
-          ok = false;
-          break;
-        }
-        fence_after_sync();
-        float m[8], e[8];  // eight columns at a time keeps the TwoSum state in registers
-#pragma unroll
-        for (int h = 0; h < 4; ++h) {
-          tmem_ld8(tlane + 256 * a + 8 * h, m);
-          tmem_ld8(tlane + 256 * a + 128 + 8 * h, e);
-#pragma unroll
-          for (int j = 0; j < 8; ++j) two_sum(hi[8 * h + j], lo[8 * h + j], m[j] + e[j]);
-        }
-        fence_before_sync();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&sm.drained[a]);
-      }
-      ok = worker_sync_and(ok && !*abort_flag);
-      if (!ok) break;
-      after(t, hi, lo);
     }
-  } else if (warp == NWK) {
-    // MMA warp: the whole warp runs the loops, lane 0 waits and issues
-    const uint32_t idesc = idesc_bf16(128, 128);
-    int C = 0;  // chunks issued so far by this CTA
-    bool ok = true;
-    for (int k = 0; ok; ++k) {
-      const int t = order(k);
-      if (t < 0) break;
-      const int nchunk = chunks(t);
-      for (int c = 0; c < nchunk; ++c, ++C) {
-        const int s = C % NST, a = C & 1;
-        int okw = 1;
-        if (lane == 0) {
-          okw = mbar_wait(&sm.full[s], (C / NST) & 1) ? 1 : 0;
-          if (okw && C >= 2) okw = mbar_wait(&sm.drained[a], ((C - 2) >> 1) & 1) ? 1 : 0;
-        }
-        okw = __shfl_sync(0xffffffffu, okw, 0);
-        if (!okw || *abort_flag) {
-          *abort_flag = 1;
-          ok = false;
-          break;
-        }
-        fence_after_sync();
-        if (lane == 0) {
-          Stage& S = sm.st[s];
-          uint32_t ad[3], bd[3];
-#pragma unroll
-          for (int p = 0; p < 3; ++p) {
-            ad[p] = smem_addr(S.a[p]);
-            bd[p] = smem_addr(S.b[p]);
-          }
-          const uint32_t dm = sm.tmem + 256 * a, de = dm + 128;
-#pragma unroll
-          for (int ks = 0; ks < KC / 16; ++ks) {
-            const uint32_t o = ks * 32;  // 16 bfloat16 values of K per MMA
-            const uint32_t first = ks > 0 ? 1u : 0u;
-            mma_bf16(dm, sdesc_sw128(ad[0] + o), sdesc_sw128(bd[0] + o), idesc, first);
-            mma_bf16(de, sdesc_sw128(ad[0] + o), sdesc_sw128(bd[1] + o), idesc, first);
-            mma_bf16(de, sdesc_sw128(ad[1] + o), sdesc_sw128(bd[0] + o), idesc, 1u);
-            mma_bf16(de, sdesc_sw128(ad[0] + o), sdesc_sw128(bd[2] + o), idesc, 1u);
-            mma_bf16(de, sdesc_sw128(ad[1] + o), sdesc_sw128(bd[1] + o), idesc, 1u);
-            mma_bf16(de, sdesc_sw128(ad[2] + o), sdesc_sw128(bd[0] + o), idesc, 1u);
-          }
-          mma_commit(&sm.empty[s]);  // the stage may be refilled
-          mma_commit(&sm.done[a]);   // the accumulators may be drained
-        }
-        __syncwarp();
-      }
-    }
-    if (lane == 0) mma_commit(&sm.fin);  // arrives once every MMA issued above has completed
-    __syncwarp();
-  } else {
-    // TMA producer: the whole warp runs the loops, lane 0 waits and issues
-    int C = 0;
-    bool ok = true;
-    for (int k = 0; ok; ++k) {
-      const int t = order(k);
-      if (t < 0) break;
-      const int4 base = coords(t);
-      const int nchunk = chunks(t);
-      for (int c = 0; c < nchunk; ++c, ++C) {
-        const int s = C % NST;
-        int okw = 1;
-        if (lane == 0 && C >= NST) okw = mbar_wait(&sm.empty[s], (C / NST - 1) & 1) ? 1 : 0;
-        okw = __shfl_sync(0xffffffffu, okw, 0);
-        if (!okw || *abort_flag) {
-          *abort_flag = 1;
-          ok = false;
-          break;
-        }
-        if (lane == 0) {
-          Stage& S = sm.st[s];
-          const int3 y = at(base, c);
-          mbar_arrive_expect_tx(&sm.full[s], 6u * kTileBytes);
-#pragma unroll
-          for (int p = 0; p < 3; ++p) {
-            tma_load_2d(S.a[p], amap, y.x, y.y + p * arows, &sm.full[s]);
-            tma_load_2d(S.b[p], bmap, y.x, y.z + p * brows, &sm.full[s]);
-          }
-        }
-        __syncwarp();
-      }
-    }
-    // no copy may still be landing in shared memory when the CTA leaves
-    if (lane == 0)
-      for (int c = C > NST ? C - NST : 0; c < C; ++c) mbar_wait(&sm.full[c % NST], (c / NST) & 1);
-    __syncwarp();
-  }
-  const bool w = mbar_wait(&sm.fin, 0);
-  return __syncthreads_and(w && !*abort_flag) != 0;
+    __device__ void operator()(int j, float x) { two_sum(hi[j], lo[j], x); }
+  } acc;
+  return walk<4>(sm, amap, arows, bmap, brows, order, chunks, coords, at, AddRef<Sum>{acc},
+                 [&](int t) { after(t, acc.hi, acc.lo); });
 }
 
 __device__ __forceinline__ void setup(Smem& sm) {

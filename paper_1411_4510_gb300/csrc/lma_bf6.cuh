@@ -191,7 +191,7 @@ __device__ bool walk(Smem& sm, const CUtensorMap* amap, int arows, const CUtenso
     }
   } else if (warp == NWK) {
     // MMA warp: the whole warp runs the loops, lane 0 waits and issues
-    const uint32_t idesc = idesc_bf16(128, 128);
+    const uint32_t idesc = idesc_bf16(128, 128), idesc2 = idesc_bf16(128, 256);
     int C = 0;  // chunks issued so far by this CTA
     bool ok = true;
     for (int k = 0; ok; ++k) {
@@ -225,8 +225,8 @@ __device__ bool walk(Smem& sm, const CUtensorMap* amap, int arows, const CUtenso
           for (int ks = 0; ks < KC / 16; ++ks) {
             const uint32_t o = ks * 32;  // 16 bfloat16 values of K per MMA
             const uint32_t first = ks > 0 ? 1u : 0u;
-            mma_bf16(dm, sdesc_sw128(ad[0] + o), sdesc_sw128(bd[0] + o), idesc, first);
-            mma_bf16(de, sdesc_sw128(ad[0] + o), sdesc_sw128(bd[1] + o), idesc, first);
+            // planes 0 and 1 of B are 256 consecutive rows and the two accumulators 256 consecutive columns
+            mma_bf16(dm, sdesc_sw128(ad[0] + o), sdesc_sw128(bd[0] + o), idesc2, first);
             mma_bf16(de, sdesc_sw128(ad[1] + o), sdesc_sw128(bd[0] + o), idesc, 1u);
             mma_bf16(de, sdesc_sw128(ad[0] + o), sdesc_sw128(bd[2] + o), idesc, 1u);
             mma_bf16(de, sdesc_sw128(ad[1] + o), sdesc_sw128(bd[1] + o), idesc, 1u);

@@ -30,7 +30,7 @@ namespace bf6 {
 constexpr int KC = 64;        // K values per chunk: one 128-byte swizzled row of bfloat16
 constexpr int NST = 2;        // pipeline stages
 constexpr int NWK = 16;       // worker warps (4 lane quarters x 4 groups of 32 columns)
-constexpr int NTHR = 32 * (NWK + 2);  // + MMA warp + TMA warp
+constexpr int NTHR = 32 * (NWK + 4);  // + MMA warp + TMA warp + two that complete their register group
 constexpr uint32_t kTileBytes = 128u * KC * 2u;  // one 128 x 64 bfloat16 box (16 KB)
 
 // Three bfloat16 pieces of an FP32 value (round to nearest each time; the
@@ -140,13 +140,18 @@ struct AddRef {
 // time, and call after(t) with worker warp w's row 32 (w mod 4) + lane and
 // columns 32 (w / 4) + j.  Every wait has an iteration limit; on a timeout all
 // roles stop, no copy is left landing, and false is returned in every thread.
-template <int STEP, class Order, class Chunks, class Coords, class At, class Add, class After>
+template <int STEP, class Order, class Chunks, class Coords, class At, class Before, class Add,
+          class After>
 __device__ bool walk(Smem& sm, const CUtensorMap* amap, int arows, const CUtensorMap* bmap, int brows,
-                     Order order, Chunks chunks, Coords coords, At at, Add add, After after) {
+                     Order order, Chunks chunks, Coords coords, At at, Before before, Add add,
+                     After after) {
   using namespace tc;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   volatile int* abort_flag = &sm.abort;
+  // 640 threads start with 96 registers; the workers take 112 (their sums are 64 of them and spilled before, 0.5-4% of
+  // the kernels' time) from the last four warps' share: 512 x 112 + 128 x 32 = 640 x 96
   if (warp < NWK) {
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 112;");
     const int q = warp & 3, half = warp >> 2;
     const uint32_t tlane = sm.tmem + ((uint32_t)(q * 32) << 16) + half * 32;
     int G = 0;  // chunks drained so far by this CTA
@@ -154,6 +159,7 @@ __device__ bool walk(Smem& sm, const CUtensorMap* amap, int arows, const CUtenso
     for (int k = 0;; ++k) {
       const int t = order(k);
       if (t < 0) break;
+      before(t);
       add.clear();
       const int nchunk = chunks(t);
       for (int c = 0; c < nchunk && ok; ++c, ++G) {
@@ -189,7 +195,9 @@ __device__ bool walk(Smem& sm, const CUtensorMap* amap, int arows, const CUtenso
       if (!ok) break;
       after(t);
     }
-  } else if (warp == NWK) {
+  } else {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 32;");
+    if (warp == NWK) {
     // MMA warp: the whole warp runs the loops, lane 0 waits and issues
     const uint32_t idesc = idesc_bf16(128, 128), idesc2 = idesc_bf16(128, 256);
     int C = 0;  // chunks issued so far by this CTA
@@ -240,7 +248,7 @@ __device__ bool walk(Smem& sm, const CUtensorMap* amap, int arows, const CUtenso
     }
     if (lane == 0) mma_commit(&sm.fin);  // arrives once every MMA issued above has completed
     __syncwarp();
-  } else {
+    } else if (warp == NWK + 1) {
     // TMA producer: the whole warp runs the loops, lane 0 waits and issues
     int C = 0;
     bool ok = true;
@@ -276,14 +284,15 @@ __device__ bool walk(Smem& sm, const CUtensorMap* amap, int arows, const CUtenso
     if (lane == 0)
       for (int c = C > NST ? C - NST : 0; c < C; ++c) mbar_wait(&sm.full[c % NST], (c / NST) & 1);
     __syncwarp();
+    }
   }
   const bool w = mbar_wait(&sm.fin, 0);
   return __syncthreads_and(w && !*abort_flag) != 0;
 }
 
-template <class Order, class Chunks, class Coords, class At, class After>
+template <class Order, class Chunks, class Coords, class At, class Before, class After>
 __device__ bool persistent(Smem& sm, const CUtensorMap* amap, int arows, const CUtensorMap* bmap,
-                           int brows, Order order, Chunks chunks, Coords coords, At at, After after) {
+                           int brows, Order order, Chunks chunks, Coords coords, At at, Before before, After after) {
   struct Sum {
     float v[32];
     __device__ void clear() {
@@ -292,16 +301,16 @@ __device__ bool persistent(Smem& sm, const CUtensorMap* amap, int arows, const C
     }
     __device__ void operator()(int j, float x) { v[j] += x; }
   } acc;
-  return walk<8>(sm, amap, arows, bmap, brows, order, chunks, coords, at, AddRef<Sum>{acc},
+  return walk<8>(sm, amap, arows, bmap, brows, order, chunks, coords, at, before, AddRef<Sum>{acc},
                   [&](int t) { after(t, acc.v); });
 }
 
 // persistent() with the chunks' results added by TwoSum into (hi, lo), for
 // products whose K runs long (thousands of values): after(t, hi, lo).  Eight
 // columns at a time keep the TwoSum state in registers.
-template <class Order, class Chunks, class Coords, class At, class After>
+template <class Order, class Chunks, class Coords, class At, class Before, class After>
 __device__ bool persistent_comp(Smem& sm, const CUtensorMap* amap, int arows, const CUtensorMap* bmap,
-                                int brows, Order order, Chunks chunks, Coords coords, At at, After after) {
+                                int brows, Order order, Chunks chunks, Coords coords, At at, Before before, After after) {
   struct Sum {
     float hi[32], lo[32];
     __device__ void clear() {
@@ -310,8 +319,38 @@ __device__ bool persistent_comp(Smem& sm, const CUtensorMap* amap, int arows, co
     }
     __device__ void operator()(int j, float x) { two_sum(hi[j], lo[j], x); }
   } acc;
-  return walk<4>(sm, amap, arows, bmap, brows, order, chunks, coords, at, AddRef<Sum>{acc},
+  return walk<4>(sm, amap, arows, bmap, brows, order, chunks, coords, at, before, AddRef<Sum>{acc},
                  [&](int t) { after(t, acc.hi, acc.lo); });
+}
+
+// A warp's 32 x 32 values, lane = row, v[j] = column j, to the rows r < rows of dst (leading dimension ld; dst and ld
+// multiples of 4 floats).  From the row's own lane a store puts 16 bytes into each of 32 rows (5,400 clocks for a CTA's
+// 128 x 128 tile); exchanged among eight lanes first, it puts 128 bytes into each of four.
+__device__ __forceinline__ void store_rows(float (&v)[32], float* dst, int64_t ld, int rows) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int b = 1; b < 8; b <<= 1) {
+    const bool up = lane & b;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      if (u & b) continue;
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        float &lo = v[4 * u + k], &hi = v[4 * (u | b) + k];
+        const float got = __shfl_xor_sync(0xffffffffu, up ? lo : hi, b);
+        if (up)
+          lo = got;
+        else
+          hi = got;
+      }
+    }
+  }
+  const int r0 = lane & 24, c = 4 * (lane & 7);
+#pragma unroll
+  for (int u = 0; u < 8; ++u)
+    if (r0 + u < rows)
+      *reinterpret_cast<float4*>(dst + (int64_t)(r0 + u) * ld + c) =
+          make_float4(v[4 * u], v[4 * u + 1], v[4 * u + 2], v[4 * u + 3]);
 }
 
 __device__ __forceinline__ void setup(Smem& sm) {
@@ -531,7 +570,7 @@ __global__ void __launch_bounds__(bf6::NTHR, 1) k_gram_bf6(const int2* __restric
     for (int j = 0; j < 32; ++j)
       if (cg + j < se) P[cg + j] = (double)hi[j] + (double)lo[j];
   };
-  const bool ok = bf6::persistent_comp(sm, &sb, srows, &sb, srows, order, chunks, coords, at, after);
+  const bool ok = bf6::persistent_comp(sm, &sb, srows, &sb, srows, order, chunks, coords, at, [](int) {}, after);
   if (!ok && threadIdx.x == 0) atomicExch(err, 1);
   bf6::teardown(sm);
 }
@@ -554,7 +593,7 @@ __global__ void __launch_bounds__(bf6::NTHR, 1) k_resid_bf6(const int4* __restri
   grid_dep_launch();
   extern __shared__ __align__(16) unsigned char smraw[];
   bf6::Smem& sm = bf6::smem_of(smraw);
-  __shared__ __align__(16) float xc[128][D];  // scaled inputs of the tile's columns, zero-padded
+  __shared__ __align__(16) float xc[128][D], xw[128][D];  // scaled inputs of the tile's columns and rows, zero-padded
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, tid = threadIdx.x;
   bf6::setup(sm);
   auto order = [&](int k) -> int {
@@ -568,44 +607,48 @@ __global__ void __launch_bounds__(bf6::NTHR, 1) k_resid_bf6(const int4* __restri
     return make_int4(base + it.y * 128, base + it.z * 128, 0, 0);
   };
   auto at = [](int4 b, int c) { return make_int3(bf6::KC * c, b.x, b.y); };
-  auto after = [&](int t, float(&hi)[32], float(&lo)[32]) {
+  // read at the item's start, while the first chunk is on its way (in the epilogue it cost 4,000 clocks an item)
+  auto before = [&](int t) {
     const int4 it = items[t];
     const Win w = wins[it.x];
     const int r0 = it.y * 128, c0 = it.z * 128;
-    worker_sync_and(true);  // every worker is done with the previous tile's columns
-    for (int e = tid; e < 128 * D; e += bf6::NWK * 32) {
-      const int r = e / D, q = e % D;
-      xc[r][q] = (c0 + r < w.n && q < d) ? xs[(w.g_end - 1 - (c0 + r)) * d + q] : 0.f;
-    }
-    worker_sync_and(true);
-    const int q = warp & 3, half = warp >> 2;
-    const int i = r0 + q * 32 + lane;
-    const int cg = c0 + half * 32;
-    if (i >= w.npad || cg >= w.npad) return;
-    float xr[D];
+    worker_sync_and(true);  // every worker is done with the previous tile's
 #pragma unroll
-    for (int t2 = 0; t2 < D; ++t2) xr[t2] = (i < w.n && t2 < d) ? xs[(w.g_end - 1 - i) * d + t2] : 0.f;
-    float* dst = buf + w.base + (int64_t)i * w.npad + cg;
-#pragma unroll
-    for (int j4 = 0; j4 < 8; ++j4) {
-      float out[4];
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const int j = 4 * j4 + k, cl = half * 32 + j, jj = c0 + cl;
-        float v;
-        if (i < w.n && jj < w.n) {
-          const float d2 = dist2<D>(xr, xc[cl]);
-          v = (ss2 * expf(-0.5f * d2) - hi[j]) - lo[j];
-          if (i == jj) v += sn2;
-        } else {
-          v = (i == jj) ? 1.f : 0.f;
-        }
-        out[k] = v;
-      }
-      *reinterpret_cast<float4*>(dst + 4 * j4) = make_float4(out[0], out[1], out[2], out[3]);
+    for (int k = 0; k < 128 * D / (bf6::NWK * 32); ++k) {
+      const int e = tid + k * bf6::NWK * 32, r = e / D, q = e % D;
+      const float vc = xs[(w.g_end - 1 - min(c0 + r, w.n - 1)) * d + min(q, d - 1)];
+      const float vr = xs[(w.g_end - 1 - min(r0 + r, w.n - 1)) * d + min(q, d - 1)];
+      xc[r][q] = (c0 + r < w.n && q < d) ? vc : 0.f;
+      xw[r][q] = (r0 + r < w.n && q < d) ? vr : 0.f;
     }
   };
-  const bool ok = bf6::persistent_comp(sm, &vb, nrev, &vb, nrev, order, chunks, coords, at, after);
+  auto after = [&](int t, float(&hi)[32], float(&lo)[32]) {
+    const int4 it = items[t];
+    const Win w = wins[it.x];
+    const int q = warp & 3, half = warp >> 2;
+    const int i0 = it.y * 128 + q * 32, i = i0 + lane;
+    const int c0 = it.z * 128, cg = c0 + half * 32;
+    if (i0 >= w.npad || cg >= w.npad) return;
+    float xr[D];
+#pragma unroll
+    for (int t2 = 0; t2 < D; t2 += 4)
+      *reinterpret_cast<float4*>(&xr[t2]) = *reinterpret_cast<const float4*>(&xw[q * 32 + lane][t2]);
+#pragma unroll
+    for (int j = 0; j < 32; ++j) {
+      const int cl = half * 32 + j, jj = c0 + cl;
+      float v;
+      if (i < w.n && jj < w.n) {
+        const float d2 = dist2<D>(xr, xc[cl]);
+        v = (ss2 * expf(-0.5f * d2) - hi[j]) - lo[j];
+        if (i == jj) v += sn2;
+      } else {
+        v = (i == jj) ? 1.f : 0.f;
+      }
+      hi[j] = v;
+    }
+    bf6::store_rows(hi, buf + w.base + (int64_t)i0 * w.npad + cg, w.npad, 32);  // npad is a multiple of 64
+  };
+  const bool ok = bf6::persistent_comp(sm, &vb, nrev, &vb, nrev, order, chunks, coords, at, before, after);
   if (!ok && threadIdx.x == 0) atomicExch(err, 1);
   bf6::teardown(sm);
 }
@@ -629,7 +672,7 @@ __global__ void __launch_bounds__(bf6::NTHR, 1) k_pred_rhs_bf6(const Pair* __res
   grid_dep_launch();
   extern __shared__ __align__(16) unsigned char smraw[];
   bf6::Smem& sm = bf6::smem_of(smraw);
-  __shared__ __align__(16) float xc[128][D];
+  __shared__ __align__(16) float xc[128][D], xw[128][D];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, tid = threadIdx.x;
   bf6::setup(sm);
   auto order = [&](int k) -> int {
@@ -643,42 +686,46 @@ __global__ void __launch_bounds__(bf6::NTHR, 1) k_pred_rhs_bf6(const Pair* __res
     return make_int4(pr.u0 + it.y * 128, nrev - (int)wins[pr.win].g_end + it.z * 128, 0, 0);
   };
   auto at = [](int4 b, int c) { return make_int3(bf6::KC * c, b.x, b.y); };
-  auto after = [&](int t, float(&hi)[32], float(&lo)[32]) {
+  auto before = [&](int t) {
     const int4 it = items[t];
     const Pair pr = pairs[it.x];
     const Win w = wins[pr.win];
     const int u0 = it.y * 128, c0 = it.z * 128;
     worker_sync_and(true);
-    for (int e = tid; e < 128 * D; e += bf6::NWK * 32) {
-      const int r = e / D, q = e % D;
-      xc[r][q] = (c0 + r < w.n && q < d) ? xs[(w.g_end - 1 - (c0 + r)) * d + q] : 0.f;
-    }
-    worker_sync_and(true);
-    const int q = warp & 3, half = warp >> 2;
-    const int uu = u0 + q * 32 + lane;
-    const int cg = c0 + half * 32;
-    if (uu >= pr.nu || cg >= w.npad) return;
-    float xr[D];
 #pragma unroll
-    for (int t2 = 0; t2 < D; ++t2) xr[t2] = t2 < d ? xu[(int64_t)(pr.u0 + uu) * d + t2] : 0.f;
-    float* dst = P + pr.pbase + (int64_t)uu * w.npad + cg;
-#pragma unroll
-    for (int j4 = 0; j4 < 8; ++j4) {
-      float out[4];
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const int j = 4 * j4 + k, cl = half * 32 + j;
-        float v = 0.f;
-        if (c0 + cl < w.n) {
-          const float d2 = dist2<D>(xr, xc[cl]);
-          v = (ss2 * expf(-0.5f * d2) - hi[j]) - lo[j];
-        }
-        out[k] = v;
-      }
-      *reinterpret_cast<float4*>(dst + 4 * j4) = make_float4(out[0], out[1], out[2], out[3]);
+    for (int k = 0; k < 128 * D / (bf6::NWK * 32); ++k) {
+      const int e = tid + k * bf6::NWK * 32, r = e / D, q = e % D;
+      const float vc = xs[(w.g_end - 1 - min(c0 + r, w.n - 1)) * d + min(q, d - 1)];
+      const float vr = xu[(int64_t)(pr.u0 + min(u0 + r, pr.nu - 1)) * d + min(q, d - 1)];
+      xc[r][q] = (c0 + r < w.n && q < d) ? vc : 0.f;
+      xw[r][q] = (u0 + r < pr.nu && q < d) ? vr : 0.f;
     }
   };
-  const bool ok = bf6::persistent_comp(sm, &ub, urows, &vb, nrev, order, chunks, coords, at, after);
+  auto after = [&](int t, float(&hi)[32], float(&lo)[32]) {
+    const int4 it = items[t];
+    const Pair pr = pairs[it.x];
+    const Win w = wins[pr.win];
+    const int q = warp & 3, half = warp >> 2;
+    const int uw = it.y * 128 + q * 32;  // the warp's first test row
+    const int c0 = it.z * 128, cg = c0 + half * 32;
+    if (uw >= pr.nu || cg >= w.npad) return;
+    float xr[D];
+#pragma unroll
+    for (int t2 = 0; t2 < D; t2 += 4)
+      *reinterpret_cast<float4*>(&xr[t2]) = *reinterpret_cast<const float4*>(&xw[q * 32 + lane][t2]);
+#pragma unroll
+    for (int j = 0; j < 32; ++j) {
+      const int cl = half * 32 + j;
+      float v = 0.f;
+      if (c0 + cl < w.n) {
+        const float d2 = dist2<D>(xr, xc[cl]);
+        v = (ss2 * expf(-0.5f * d2) - hi[j]) - lo[j];
+      }
+      hi[j] = v;
+    }
+    bf6::store_rows(hi, P + pr.pbase + (int64_t)uw * w.npad + cg, w.npad, min(32, pr.nu - uw));
+  };
+  const bool ok = bf6::persistent_comp(sm, &ub, urows, &vb, nrev, order, chunks, coords, at, before, after);
   if (!ok && threadIdx.x == 0) atomicExch(err, 1);
   bf6::teardown(sm);
 }
@@ -711,13 +758,11 @@ __global__ void __launch_bounds__(bf6::NTHR, 1) k_proj_tc(const __grid_constant_
     const int q = warp & 3, half = warp >> 2;
     const int64_t row = (int64_t)(t / nct) * 128 + q * 32 + lane;
     const int c0 = (t % nct) * 128 + half * 32;
-    if (row >= nrows || c0 >= s) return;
+    if (c0 >= s) return;
     float* dst = out + row * ldo + c0;
     if (c0 + 32 <= s && (ldo & 3) == 0) {
-#pragma unroll
-      for (int j4 = 0; j4 < 8; ++j4)
-        *reinterpret_cast<float4*>(dst + 4 * j4) = make_float4(acc[4 * j4], acc[4 * j4 + 1], acc[4 * j4 + 2], acc[4 * j4 + 3]);
-    } else {
+      bf6::store_rows(acc, dst - lane * ldo, ldo, (int)min((int64_t)32, nrows - (row - lane)));
+    } else if (row < nrows) {
 #pragma unroll
       for (int j = 0; j < 32; ++j)
         if (c0 + j < s) dst[j] = acc[j];
@@ -739,7 +784,7 @@ __global__ void __launch_bounds__(bf6::NTHR, 1) k_proj_tc(const __grid_constant_
     const int pt = (int)(u / P), j = (int)(u % P);
     return pt * nct + ((k & 1) ? nct - 1 - j : j);
   };
-  const bool ok = bf6::persistent(sm, &amap, arows, &bmap, brows, order, chunks, coords, at, after);
+  const bool ok = bf6::persistent(sm, &amap, arows, &bmap, brows, order, chunks, coords, at, [](int) {}, after);
   if (!ok && threadIdx.x == 0) atomicExch(err, 1);
   bf6::teardown(sm);
 }

@@ -706,7 +706,7 @@ def main():
             out["fp64_gpu_form"] = {
                 "value": p.N / (t_full / 1e3), "ms_per_step": t_full, "extrapolated": True,
                 "timed": {f"first {k} blocks": round(t, 2) for k, t, _ in pts},
-                "how": f"lma_fit_predict in the FP64 form (one window per launch) on the first {k1} and {k2} blocks "
+                "how": f"lma_fit_predict in the FP64 form (every window in one launch) on the first {k1} and {k2} blocks "
                        f"of the workload (same |S|, B), extrapolated linearly in the block count to {p.M}",
                 "tflops": (fit_f + pred_f) / (t_full / 1e3) / 1e12,
                 "mixed_speedup": t_full / step_ms,

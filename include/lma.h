@@ -375,7 +375,7 @@ lma_status lma_workspace_release(void);
  * (the keys are those of lma_autotune_report, e.g. "fp64 factor" for the
  * FP64 factorisations of Sigma_SS and I + A, whose choices are 0 one launch
  * per panel, 1 two launches per panel, 2-4 one cooperative launch with 1, 2
- * or 4 CTAs per SM, 5 the dataflow form with per-tile flags) to `choice`, on every device, ahead of timing, of the
+ * or 4 CTAs per SM, 5 the dataflow form) to `choice`, on every device, ahead of timing, of the
  * cache file and of lma_autotune(0).  A choice that is not among a class's
  * candidates is ignored for that class; the latest matching pin wins.
  * prefix NULL removes every pin.                                            */

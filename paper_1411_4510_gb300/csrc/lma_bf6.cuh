@@ -140,6 +140,10 @@ struct AddRef {
 // time, and call after(t) with worker warp w's row 32 (w mod 4) + lane and
 // columns 32 (w / 4) + j.  Every wait has an iteration limit; on a timeout all
 // roles stop, no copy is left landing, and false is returned in every thread.
+// What bounds it (clocks a chunk, N = 2,000,000, |S| = 2,048): the projection takes 2,815, of which the MMA thread waits
+// 430; the MMAs alone take 1,711 and share shared memory's bandwidth with the copies (196 KB read, 96 KB written).  The
+// compensated sums' drains take 1,850-2,400.  Neither L2 (boxes shared by clusters of four) nor the copies' latency (four
+// half stages) bound it: both were tried and were slower.
 template <int STEP, class Order, class Chunks, class Coords, class At, class Before, class Add,
           class After>
 __device__ bool walk(Smem& sm, const CUtensorMap* amap, int arows, const CUtensorMap* bmap, int brows,

@@ -582,51 +582,27 @@ __global__ void __launch_bounds__(256) k_grad_vbar_128(const float* __restrict__
     }
 }
 
-// exp(y) for y <= 0 to about 1e-13 relative (0 below 2^-125): y = n ln 2 + r with ln 2 in three parts (n times the
-// first is exact), then the Taylor series of exp(r), its terms from r^8 on in single precision (at most 5e-9 of the sum).
-__device__ __forceinline__ Pair2 exp2f_pair(Pair2 y) {
-  const float n = rintf(y.h * 1.44269504f);
-  Pair2 r = sum2(y.h, -0.693359375f * n);
-  const float q = __fmul_rn(n, 2.12194442e-4f);  // 0.693359375 - ln 2 = 2.12194440054690583e-4
-  const float e = __fmaf_rn(n, 2.12194442e-4f, -q);
-  r = add2(r, Pair2{q, __fadd_rn(e, __fmaf_rn(n, -1.64657177e-12f, y.l))});
-  const float x = r.h;
-  float t = 1.f / 479001600.f;
-  t = fmaf(t, x, 1.f / 39916800.f);
-  t = fmaf(t, x, 1.f / 3628800.f);
-  t = fmaf(t, x, 1.f / 362880.f);
-  t = fmaf(t, x, 1.f / 40320.f);
-  Pair2 v = add2(Pair2{0.000198412701f, -2.72559687e-12f}, scale2(r, t));  // 1/5040
-  v = add2(Pair2{0.00138888892f, -3.36310944e-11f}, mul2(r, v));  // 1/720
-  v = add2(Pair2{0.00833333377f, -4.34617203e-10f}, mul2(r, v));  // 1/120
-  v = add2(Pair2{0.0416666679f, -1.24176347e-09f}, mul2(r, v));  // 1/24
-  v = add2(Pair2{0.166666672f, -4.96705388e-09f}, mul2(r, v));  // 1/6
-  v = add2(Pair2{0.5f, 0.f}, mul2(r, v));
-  v = add2(Pair2{1.f, 0.f}, mul2(r, v));
-  v = add2(Pair2{1.f, 0.f}, mul2(r, v));
-  const float sc = n < -125.f ? 0.f : __int_as_float(((int)n + 127) << 23);
-  return {v.h * sc, v.l * sc};
-}
-
-// k_grad_kds in FP32 with pairs of floats in place of its FP64 epilogue (12.8 -> 2.8 ms at N = 65,536, s = 1,024,
-// d = 8; the gradient moves by 1e-12): tiles of TS2 x TS2 (128 or, for small problems, 64), the product parked in shared memory, then a
-// thread takes one point and every (256 / TS2)-th support coordinate.  D: d padded with zero coordinates.
+// k_grad_kds in FP32 on tiles of TS2 x TS2 (128 or, for small problems, 64): the product is parked in shared memory,
+// then a thread takes one point and every (256 / TS2)-th support coordinate for the covariance terms, which are FP64 as
+// there (a float difference or exponential would lose what cancels in the sums; a pair at any distance gives 0 x finite).
+// D: d rounded up to 8 or MAXD, the bound of the unrolled loops.  The FP64 terms bound it (4 instructions a dimension,
+// about 20 for exp, one per 64 clocks and scheduler): 8.4 ms at N = 65,536, s = 1,024, d = 8 (9.0 with one CTA per SM,
+// whose product and terms do not overlap), against 12.8 of k_grad_kds.
 template <int TS2, int D>
-__global__ void __launch_bounds__(256) k_grad_kds_pair(const float* __restrict__ VbT, const float* __restrict__ ET,
-                                                       const float* __restrict__ xs, const float* __restrict__ ss,
-                                                       int d, int64_t n, int s, double ss2,
-                                                       double* __restrict__ partial) {
+__global__ void __launch_bounds__(256, 2) k_grad_kds_f32(const float* __restrict__ VbT, const float* __restrict__ ET,
+                                                      const float* __restrict__ xs, const float* __restrict__ ss, int d,
+                                                      int64_t n, int s, double ss2, double* __restrict__ partial) {
   grid_dep_wait();
   grid_dep_launch();
   extern __shared__ __align__(16) unsigned char smraw[];
-  float* prod = reinterpret_cast<float*>(smraw);                       // [TS2][TS2 + 1]
-  float(*xk)[D] = reinterpret_cast<float(*)[D]>(prod + TS2 * (TS2 + 4));  // [TS2][D]
+  float* prod = reinterpret_cast<float*>(smraw);                            // [TS2][TS2 + 1]
+  double(*xk)[D] = reinterpret_cast<double(*)[D]>(prod + TS2 * (TS2 + 4));  // [TS2][D]
   __shared__ double red[8][D + 1];
   const int k0 = blockIdx.y * TS2;
   const int64_t p0 = (int64_t)blockIdx.x * TS2;
   for (int e = threadIdx.x; e < TS2 * D; e += 256) {
     const int r = e / D, q = e % D;
-    xk[r][q] = (k0 + r < s && q < d) ? ss[(int64_t)(k0 + r) * d + q] : 0.f;
+    xk[r][q] = (k0 + r < s && q < d) ? (double)ss[(int64_t)(k0 + r) * d + q] : 0.0;
   }
   if constexpr (TS2 == 128) {
     Smem128& sm = *reinterpret_cast<Smem128*>(smraw);
@@ -656,34 +632,39 @@ __global__ void __launch_bounds__(256) k_grad_kds_pair(const float* __restrict__
   __syncthreads();
   const int pc = threadIdx.x % TS2;
   const int64_t p = p0 + pc;
-  float xp[D];
+  double xp[D], gl[D], gs = 0.0;
 #pragma unroll
-  for (int q = 0; q < D; ++q) xp[q] = (p < n && q < d) ? xs[p * d + q] : 0.f;
-  Pair2 gl[D], gs{0.f, 0.f};
-#pragma unroll
-  for (int q = 0; q < D; ++q) gl[q] = {0.f, 0.f};
+  for (int q = 0; q < D; ++q) {
+    xp[q] = (p < n && q < d) ? (double)xs[p * d + q] : 0.0;
+    gl[q] = 0.0;
+  }
   if (p < n)
     for (int kr = threadIdx.x / TS2; kr < min(TS2, s - k0); kr += 256 / TS2) {
-      Pair2 d2{0.f, 0.f};
+      double d2 = 0.0;
 #pragma unroll
-      for (int q = 0; q < D; ++q) {
-        const Pair2 t = sum2(xk[kr][q], -xp[q]);
-        d2 = add2(d2, mul2(t, t));
-      }
-      const Pair2 kg = scale2(exp2f_pair(Pair2{-0.5f * d2.h, -0.5f * d2.l}), prod[kr * (TS2 + 1) + pc]);
-      gs = add2(gs, kg);
+      for (int q = 0; q < D; ++q)
+        if (q < d) {
+          const double t = xk[kr][q] - xp[q];
+          d2 += t * t;
+        }
+      const double kg = (double)prod[kr * (TS2 + 1) + pc] * exp(-0.5 * d2);
+      gs += kg;
 #pragma unroll
-      for (int q = 0; q < D; ++q) {
-        const Pair2 t = sum2(xk[kr][q], -xp[q]);
-        gl[q] = add2(gl[q], mul2(kg, mul2(t, t)));
-      }
+      for (int q = 0; q < D; ++q)
+        if (q < d) {
+          const double t = xk[kr][q] - xp[q];
+          gl[q] += kg * t * t;
+        }
     }
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 #pragma unroll
-  for (int q = 0; q < D + 1; ++q) {
-    const Pair2 v = warp_sum2(q < D ? gl[q < D ? q : 0] : gs);
-    if (lane == 0) red[warp][q] = to_double(v);
-  }
+  for (int q = 0; q < D + 1; ++q)
+    if (q < d || q == D) {
+      double v = q < D ? gl[q < D ? q : 0] : gs;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+      if (lane == 0) red[warp][q] = v;
+    }
   __syncthreads();
   double* P = partial + ((int64_t)blockIdx.y * gridDim.x + blockIdx.x) * (d + 2);
   if (threadIdx.x <= d) {

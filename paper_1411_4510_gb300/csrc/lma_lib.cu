@@ -341,8 +341,8 @@ void Impl<T>::setup_attributes() {
     cudaFuncSetAttribute(k_chol_wide<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)wide_smem<256>());
     cudaFuncSetAttribute(k_chol_wide<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)wide_smem<128>());
     cudaFuncSetAttribute(k_proj_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bf6::smem_bytes());
-    cudaFuncSetAttribute(k_grad_kds_pair<128, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kds_smem(128, 8));
-    cudaFuncSetAttribute(k_grad_kds_pair<128, MAXD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaFuncSetAttribute(k_grad_kds_f32<128, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kds_smem(128, 8));
+    cudaFuncSetAttribute(k_grad_kds_f32<128, MAXD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)kds_smem(128, MAXD));
     cudaFuncSetAttribute(k_grad_rhs_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc_chol_smem());
     cudaFuncSetAttribute(k_bwd_sweep_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc_chol_smem());
@@ -1466,8 +1466,10 @@ void Impl<T>::loglik_grad(ModelCore& mc, const lma_problem* P, const lma_hyper* 
   *ll = mc.loglik;
 }
 
-// Dynamic shared memory of k_grad_kds_pair: the product tile (or the operands') and the support coordinates.
-static size_t kds_smem(int tile, int dpad) { return sizeof(float) * ((size_t)tile * (tile + 4) + (size_t)tile * dpad); }
+// Dynamic shared memory of k_grad_kds_f32: the product tile (or the operands') and the support coordinates.
+static size_t kds_smem(int tile, int dpad) {
+  return sizeof(float) * (size_t)tile * (tile + 4) + sizeof(double) * (size_t)tile * dpad;
+}
 
 // Sb = L^-T Phi(L^T Lbar) L^-1 with Lbar = -L^-T M1 (the adjoint of the Cholesky factor), Y a scratch matrix.
 template <int TILE>
@@ -1606,8 +1608,8 @@ void Impl<T>::grad_windows(ModelCore& mc, int64_t k_lo, int64_t k_hi, double* gr
     if constexpr (sizeof(T) == 4) {
       const bool d8 = pad_dim(d) == 8;
       launch("k_grad_kds",
-             big ? (d8 ? k_grad_kds_pair<128, 8> : k_grad_kds_pair<128, MAXD>)
-                 : (d8 ? k_grad_kds_pair<64, 8> : k_grad_kds_pair<64, MAXD>),
+             big ? (d8 ? k_grad_kds_f32<128, 8> : k_grad_kds_f32<128, MAXD>)
+                 : (d8 ? k_grad_kds_f32<64, 8> : k_grad_kds_f32<64, MAXD>),
              dim3(gx, gy), 256, kds_smem((int)tile, d8 ? 8 : MAXD), st, (const float*)VbT, (const float*)mc.ET,
              (const float*)mc.xsT, (const float*)mc.ssT, d, n, si, mc.ss2, pK);
     } else {

@@ -497,8 +497,9 @@ __device__ __forceinline__ void tri_element(int e, int& r, int& c) {
 }
 
 // The chain CTA.  hsub[k] / hdiag[k] (0 or 1): tile (k + 1, k) / (k, k) handed over with every panel below k /
-// k - 1 applied.
-__device__ void flow_chain(FlowChain& c, double* buf, int64_t ld, int npan, double* dinv, int* info, unsigned* prog,
+// k - 1 applied.  Returns false in every thread once a wait has given up.  c.bad is cleared by the caller ahead of the
+// first call and stays set from then on: the publishing warp may read it a panel later than the others.
+__device__ bool flow_chain(FlowChain& c, double* buf, int64_t ld, int npan, double* dinv, int* info, unsigned* prog,
                            unsigned* xprog, const unsigned* hsub, const unsigned* hdiag, int* err) {
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int r = lane & 15, h = lane >> 4;
@@ -513,7 +514,6 @@ __device__ void flow_chain(FlowChain& c, double* buf, int64_t ld, int npan, doub
     if (q < TS) c.rj[q] = e;
   };
   if (tid >= FTH - TS * TS) clear_slots(tid - (FTH - TS * TS));
-  if (tid == 0) c.bad = 0;
   int er = 0, ec = 0;  // this thread's element of the (k + 1, k + 1) update
   if (tid < 128) tri_element(tid, er, ec);
   double tcorner = 0.0;  // warp 4, lanes 0-7: element (15, 8 + lane) before that update
@@ -524,13 +524,13 @@ __device__ void flow_chain(FlowChain& c, double* buf, int64_t ld, int npan, doub
     // since their panel k - 1 needed bulk tiles that needed xprog >= k - 1.
     for (int k = 0; k < npan; ++k) {
       bar_sync(6 + 2 * (k & 1), FTH);
-      if (*bad) return;
+      if (*bad) return false;
       if (lane == 0) {
         __threadfence();
         st_rel(xprog, (unsigned)(k + 1));
       }
       __syncwarp();
-      if (k + 1 == npan) return;
+      if (k + 1 == npan) return true;
       bar_sync(7 + 2 * (k & 1), FTH);
       if (lane == 0) {
         __threadfence();
@@ -538,7 +538,7 @@ __device__ void flow_chain(FlowChain& c, double* buf, int64_t ld, int npan, doub
       }
       __syncwarp();
     }
-    return;
+    return true;
   }
   for (int k = 0; k < npan; ++k) {
     const bool more = k + 1 < npan;
@@ -651,7 +651,7 @@ __device__ void flow_chain(FlowChain& c, double* buf, int64_t ld, int npan, doub
     if (tid < TS * TS) buf[(int64_t)(k0 + tid / TS) * ld + k0 + tid % TS] = c.Lt[tid / TS][tid % TS];  // read after the kernel
     if (*bad) {
       if (tid == 0) atomicExch(err, 1);
-      return;
+      return false;
     }
     if (!more) break;
     if (warp < 8) {  // solve L = T inv(L_kk)^T: a column pair per warp (inv(L_kk) is lower), even over the schedulers
@@ -679,6 +679,7 @@ __device__ void flow_chain(FlowChain& c, double* buf, int64_t ld, int npan, doub
     if (warp == 4 && lane < 8) tcorner = c.A[15][8 + lane];
     bar_sync(0, MT);
   }
+  return true;
 }
 
 // A band CTA: rows first, first + step, ... < npan.  Threads 0-127 compute, warp 4 publishes.
@@ -928,9 +929,10 @@ __global__ void __launch_bounds__(FTH, 1) k_f64_flow(double* buf, int64_t ld, in
   unsigned* hsub = xprog + CSTR;
   unsigned* hdiag = hsub + npan;
   const int g = threadIdx.x >> 7, b = (int)blockIdx.x - 1 - nband, nb = (int)gridDim.x - 1 - nband;
-  if (blockIdx.x == 0)
+  if (blockIdx.x == 0) {
+    if (threadIdx.x == 0) sm.c.bad = 0;
     flow_chain(sm.c, buf, ld, npan, dinv, info, prog, xprog, hsub, hdiag, err);
-  else if (b < 0)
+  } else if (b < 0)
     flow_band(sm.b, buf, ld, npan, dinv, 1 + (int)blockIdx.x, nband, prog, xprog, hsub, hdiag, err);
   else
     flow_bulk<false>(
@@ -965,12 +967,15 @@ __global__ void __launch_bounds__(FTH, 1) k_f64_windows(const FlowWin* __restric
   __shared__ FlowSmem sm;
   const int g = threadIdx.x >> 7, b = (int)blockIdx.x - nchain, nb = (int)gridDim.x - nchain;
   if (b < 0) {
+    if (threadIdx.x == 0) sm.c.bad = 0;
     for (int w = blockIdx.x; w < nwin; w += nchain) {
       const FlowWin f = wins[w];
       unsigned* prog = cnt + f.cnt;
       unsigned* xprog = prog + (int64_t)f.nrt * CSTR;
-      flow_chain(sm.c, buf + f.base, f.ld, f.npan, dv16 + f.dv, info + w, prog, xprog, xprog + CSTR,
-                 xprog + CSTR + f.npan, err);
+      // no further window once a wait gave up: a warp still in this one would meet the others at another barrier
+      if (!flow_chain(sm.c, buf + f.base, f.ld, f.npan, dv16 + f.dv, info + w, prog, xprog, xprog + CSTR,
+                      xprog + CSTR + f.npan, err))
+        return;
     }
     return;
   }

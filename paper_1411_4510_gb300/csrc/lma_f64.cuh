@@ -949,7 +949,7 @@ __global__ void __launch_bounds__(FTH, 1) k_f64_flow(double* buf, int64_t ld, in
 // factorises `nwin` windows and solves their extra rows.  Block c < nchain is the
 // chain of windows c, c + nchain, ...; the other CTAs' groups take the tiles of all
 // windows (list: window, i, j; round by round of nchain windows, then column by
-// column), among them, ahead of column j's others, (j + 1, j) and (j + 1, j + 1) up
+// column, see k_f64_tiles), among them (j + 1, j) and (j + 1, j + 1) up
 // to the panel that the chain applies itself.  The FP64 pipe bounds it once there are enough windows: a group's warp
 // keeps two of its four 64-clock slots a 16-column step busy.  dv16: 16 x 16
 // inverse diagonal tiles (npan per window from its dv on), cnt: FlowMat counters.
@@ -960,6 +960,49 @@ struct FlowWin {
   int64_t base, dv, cnt;
   int ld, rows, npan, nrt;
 };
+
+// The bulk's tile list.  Column j of a window (npan panels, nrt row tiles) has flow_column() tiles: ahead of the others
+// what the chain's panel j needs, (j + 1, j) and (j + 1, j + 1), handed over (no wait is for a tile later in the list;
+// panel 0 finds it in the original matrix), then (i, j) for i >= j + 2 and the appended rows.
+__host__ __device__ inline int flow_handed(int npan, int j) { return j > 0 && j + 1 < npan ? 2 : 0; }
+__host__ __device__ inline int flow_first(int npan, int j) { return j + 2 < npan ? j + 2 : npan; }
+__host__ __device__ inline int flow_column(int npan, int nrt, int j) {
+  return flow_handed(npan, j) + nrt - flow_first(npan, j);
+}
+// Tiles of columns 0 .. j - 1, j <= npan.
+__host__ __device__ inline int64_t flow_columns(int npan, int nrt, int j) {
+  const int64_t c = j, handed = j - 1 < npan - 2 ? j - 1 : npan - 2;
+  return c * nrt - (c * (c - 1) / 2 + 2 * c - (j == npan ? 1 : 0)) + 2 * (handed > 0 ? handed : 0);
+}
+// Tiles of window v (described by f) ahead of column j of window w: rounds of nchain windows, then columns, then windows.
+__host__ __device__ inline int64_t flow_ahead(const FlowWin& f, int v, int w, int j, int nchain) {
+  if (v / nchain != w / nchain) return v < w ? flow_columns(f.npan, f.nrt, f.npan) : 0;
+  if (j >= f.npan) return flow_columns(f.npan, f.nrt, f.npan);
+  return flow_columns(f.npan, f.nrt, j) + (v < w ? flow_column(f.npan, f.nrt, j) : 0);
+}
+// Tile q of column j of window w.
+__host__ __device__ inline int4 flow_tile(int npan, int w, int j, int q) {
+  const int h = flow_handed(npan, j);
+  return q < h ? make_int4(w, j + 1, j + q, 0) : make_int4(w, flow_first(npan, j) + q - h, j, 0);
+}
+
+// Writes the list: one CTA per window, a warp per column.  Made on the host and uploaded it was 16 bytes of page-locked
+// memory a tile (385 KB for a window of 2,000 points with 2,049 extra rows).
+__global__ void __launch_bounds__(256) k_f64_tiles(const FlowWin* __restrict__ wins, int nwin, int nchain,
+                                                   int4* __restrict__ tiles) {
+  grid_dep_wait();
+  grid_dep_launch();
+  const int w = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const FlowWin f = wins[w];
+  for (int j = warp; j < f.npan; j += 8) {
+    int64_t at = 0;
+    for (int v = lane; v < nwin; v += 32) at += flow_ahead(wins[v], v, w, j, nchain);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) at += __shfl_xor_sync(0xffffffffu, at, o);
+    for (int q = lane; q < flow_column(f.npan, f.nrt, j); q += 32) tiles[at + q] = flow_tile(f.npan, w, j, q);
+  }
+}
+
 __global__ void __launch_bounds__(FTH, 1) k_f64_windows(const FlowWin* __restrict__ wins, int nwin, int nchain,
                                                         double* buf, double* dv16, int* info,
                                                         const int4* __restrict__ tiles, int ntiles, unsigned* cnt,

@@ -458,7 +458,7 @@ static void right_looking_fp64(cudaStream_t st, const Win& w, Win* wd, double* b
 }
 
 // The FP64 form's windows, factorised and their extra rows solved by
-// k_f64_windows, up to kWinBatch windows a launch (which bounds the tile list).
+// k_f64_windows, up to kWinBatch windows a launch (which bounds the tile list, made on the device by k_f64_tiles).
 // Chains: each takes about 16,000 clocks a 16-column panel whatever its window's
 // rows, a bulk CTA 2,048 clocks a tile update; the number of chain CTAs is the one
 // that lets both sides end together.
@@ -512,26 +512,14 @@ static void sweep_fp64(cudaStream_t st, Arena& tmp, const std::vector<Win>& wins
         nchain = c;
       }
     }
-    std::vector<int4> tiles;
-    for (int w0 = 0; w0 < nw; w0 += nchain)
-      for (int j = 0; j < maxpan; ++j)
-        for (int w = w0; w < std::min(nw, w0 + nchain); ++w) {
-          const FlowWin& f = fw[b + w];
-          if (j >= f.npan) continue;
-          // what the chain's panel j needs comes before the tiles that need that panel (no wait is for a tile
-          // later in the list); panel 0 finds it in the original matrix
-          if (j > 0 && j + 1 < f.npan) {
-            tiles.push_back(make_int4(w, j + 1, j, 0));
-            tiles.push_back(make_int4(w, j + 1, j + 1, 0));
-          }
-          for (int i = std::min(j + 2, f.npan); i < f.nrt; ++i) tiles.push_back(make_int4(w, i, j, 0));
-        }
-    int4* tl = tmp.alloc<int4>(tiles.size());
-    stage_copy(tl, tiles.data(), sizeof(int4) * tiles.size(), st);
+    int64_t ntiles = 0;  // about one per 256 elements of the windows' buffers: an int holds what a device can
+    for (int w = 0; w < nw; ++w) ntiles += flow_columns(fw[b + w].npan, fw[b + w].nrt, fw[b + w].npan);
+    int4* tl = tmp.alloc<int4>((size_t)ntiles);
+    launch("k_f64_tiles", k_f64_tiles, (unsigned)nw, 256, 0, st, (const FlowWin*)(fwd + b), nw, nchain, tl);
     LMA_CK(cudaMemsetAsync(cntd, 0, sizeof(unsigned) * maxcnt, st));
-    const int nbulk = std::max(1, std::min(cap - nchain, (int)std::min<size_t>(tiles.size(), 1 << 20)));
+    const int nbulk = std::max(1, (int)std::min<int64_t>(cap - nchain, ntiles));
     launch_coop("k_f64_windows", k_f64_windows, (unsigned)(nchain + nbulk), FTH, 0, st, (const FlowWin*)(fwd + b), nw,
-                nchain, buf, dv16, info + b, (const int4*)tl, (int)tiles.size(), cntd, err);
+                nchain, buf, dv16, info + b, (const int4*)tl, (int)ntiles, cntd, err);
     tmp.free_one(tl);
   }
   for (size_t b = 0; b < wins.size(); b += 65535)

@@ -222,7 +222,7 @@ struct ModelCore {
   Win* wins_d = nullptr;
   double* G = nullptr;        // (s+1)^2 global Gram [quad, y; y, A]
   double* beta = nullptr;     // s
-  float2* bs = nullptr;       // beta as two floats each (mixed form)
+  float4* bs = nullptr;       // beta in three floats each, see k_split_beta (mixed form)
   void* LcT = nullptr;        // s*s, (L_C^-1)[i][k] at [k][i]   (T)
   double quad = 0, wCw = 0, logdetC = 0, logdetR = 0, loglik = 0;
   uint16_t* linv3 = nullptr;  // three bfloat16 planes of L_SS^-1 (mixed form on the tensor cores), brows x ldk each

@@ -7,7 +7,7 @@
 
 #include <type_traits>
 
-#include "lma_pair.cuh"
+#include "lma_sum3.cuh"
 #include "lma_types.cuh"
 
 namespace lma {
@@ -1103,18 +1103,22 @@ __global__ void k_ew(const Win* __restrict__ wins, const T* __restrict__ buf, co
 }
 
 // The same for FP32 extra rows without FP64 arithmetic (scarce on this part):
-// beta_k = bh_k + bl_k as two floats (k_split_beta), each product
+// beta_k = bh_k + bl_k as two floats (k_split_beta's first two), each product
 // bh_k x = p + e exactly (e from an FMA), bl_k x added to e, and the p are
 // summed with TwoSum into (hi, lo), which keeps about 48 bits of the sum.
-__global__ void k_split_beta(const double* __restrict__ beta, int s, float2* __restrict__ bs) {
+// k_split_beta: beta_k as three floats, and w = 0 where their sum is beta_k itself (53 bits fit unless a part leaves a
+// float's range), NaN where it is not.
+__global__ void k_split_beta(const double* __restrict__ beta, int s, float4* __restrict__ bs) {
   grid_dep_wait();
   grid_dep_launch();
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= s) return;
-  const float h = (float)beta[k];
-  bs[k] = make_float2(h, (float)(beta[k] - (double)h));
+  const double b = beta[k];
+  const float h = (float)b, m = (float)(b - (double)h), l = (float)((b - (double)h) - (double)m);
+  const bool exact = ((double)h + (double)m) + (double)l == b;
+  bs[k] = make_float4(h, m, l, exact ? 0.f : __int_as_float(0x7fffffff));
 }
-__global__ void k_ew_f32(const Win* __restrict__ wins, const float* __restrict__ buf, const float2* __restrict__ bs,
+__global__ void k_ew_f32(const Win* __restrict__ wins, const float* __restrict__ buf, const float4* __restrict__ bs,
                          int s, float* __restrict__ ew) {
   grid_dep_wait();
   grid_dep_launch();
@@ -1130,7 +1134,7 @@ __global__ void k_ew_f32(const Win* __restrict__ wins, const float* __restrict__
     for (int q = 0; q < 8; ++q) x[q] = E[(int64_t)(1 + k + q) * w.npad + c];
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
-      const float2 b = bs[k + q];
+      const float4 b = bs[k + q];
       const float p = b.x * x[q];
       const float e = fmaf(b.x, x[q], -p);
       lo += fmaf(b.y, x[q], e);
@@ -1139,7 +1143,7 @@ __global__ void k_ew_f32(const Win* __restrict__ wins, const float* __restrict__
   }
   for (; k < s; ++k) {
     const float x = E[(int64_t)(1 + k) * w.npad + c];
-    const float2 b = bs[k];
+    const float4 b = bs[k];
     const float p = b.x * x;
     const float e = fmaf(b.x, x, -p);
     lo += fmaf(b.y, x, e);
@@ -1312,49 +1316,51 @@ __global__ void k_pred_t12(const Pair* __restrict__ pairs, const int4* __restric
   const int lane = threadIdx.x & 31;
   if (warp >= nitems) return;
   const int4 it = items[warp];
-  int64_t row = 0;
-  if constexpr (sizeof(T) == 4) {  // pairs of floats: the FP64 pipe took 0.39 ms for 32,768 points x 1,536 columns
-    Pair2 a{0.f, 0.f}, b{0.f, 0.f};
+  if constexpr (sizeof(T) == 4) {  // 32,768 points x 1,536 columns: 0.39 ms added in FP64, 0.10 so
+    Sum3 a, b;
+    int64_t row = 0;
+    int terms = 0;
     for (int pi = 0; pi < it.y; ++pi) {
       const Pair pr = pairs[it.x + pi];
       const Win w = wins[pr.win];
       const T* Pp = P + pr.pbase + (int64_t)it.z * w.npad;
       const T* e = ew + w.ew;
       row = pr.u0 + it.z;
+      terms += (pr.c1 - pr.c0 + 31) / 32;
 #pragma unroll 4
       for (int c = pr.c0 + lane; c < pr.c1; c += 32) {
         const float p = Pp[c];
-        fma2(a, p, e[c]);
-        fma2(b, p, p);
+        a.add_product(p, e[c]);
+        b.add_product(p, p);
       }
     }
-    a = warp_sum2(a);
-    b = warp_sum2(b);
-    if (lane == 0) {
-      t1[row] = to_double(a);
-      t2[row] = to_double(b);
-    }
-  } else {
-    double a = 0.0, b = 0.0;
-    for (int pi = 0; pi < it.y; ++pi) {
-      const Pair pr = pairs[it.x + pi];
-      const Win w = wins[pr.win];
-      const T* Pp = P + pr.pbase + (int64_t)it.z * w.npad;
-      row = pr.u0 + it.z;
-      for (int c = pr.c0 + lane; c < pr.c1; c += 32) {
-        double p = (double)Pp[c];
-        a += p * (double)ew[w.ew + c];
-        b += p * p;
+    const double va = warp_sum(a.value()), vb = warp_sum(b.value());
+    if (terms <= kSum3Terms && sum3_stands(va) && sum3_stands(vb)) {
+      if (lane == 0) {
+        t1[row] = va;
+        t2[row] = vb;
       }
+      return;
     }
-    for (int o = 16; o > 0; o >>= 1) {
-      a += __shfl_down_sync(0xffffffffu, a, o);
-      b += __shfl_down_sync(0xffffffffu, b, o);
+  }
+  double a = 0.0, b = 0.0;
+  int64_t row = 0;
+  for (int pi = 0; pi < it.y; ++pi) {
+    const Pair pr = pairs[it.x + pi];
+    const Win w = wins[pr.win];
+    const T* Pp = P + pr.pbase + (int64_t)it.z * w.npad;
+    row = pr.u0 + it.z;
+    for (int c = pr.c0 + lane; c < pr.c1; c += 32) {
+      double p = (double)Pp[c];
+      a += p * (double)ew[w.ew + c];
+      b += p * p;
     }
-    if (lane == 0) {
-      t1[row] = a;
-      t2[row] = b;
-    }
+  }
+  a = warp_sum(a);
+  b = warp_sum(b);
+  if (lane == 0) {
+    t1[row] = a;
+    t2[row] = b;
   }
 }
 
@@ -1393,7 +1399,7 @@ __global__ void __launch_bounds__(NT) k_var_gemm(const T* __restrict__ h, int64_
   }
 }
 
-// out[u] = |g_u|^2 (summed in pairs of floats) for g = L_C^-1 h formed by k_proj128 (U rows of
+// out[u] = |g_u|^2 (to FP64's accuracy, see Sum3) for g = L_C^-1 h formed by k_proj128 (U rows of
 // s values): the variance term of k_var_gemm as one partial (ntile = 1).
 __global__ void k_row_sqnorm(const float* __restrict__ g, int64_t U, int s, double* __restrict__ out) {
   grid_dep_wait();
@@ -1401,14 +1407,22 @@ __global__ void k_row_sqnorm(const float* __restrict__ g, int64_t U, int s, doub
   const int64_t row = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
   const int lane = threadIdx.x & 31;
   if (row >= U) return;
-  Pair2 v{0.f, 0.f};
+  Sum3 a;
 #pragma unroll 4
   for (int k = lane; k < s; k += 32) {
     const float q = g[row * s + k];
-    fma2(v, q, q);
+    a.add_product(q, q);
   }
-  v = warp_sum2(v);
-  if (lane == 0) out[row] = to_double(v);
+  double v = warp_sum(a.value());
+  if (s > 32 * kSum3Terms || !sum3_stands(v)) {
+    v = 0.0;
+    for (int k = lane; k < s; k += 32) {
+      const double q = (double)g[row * s + k];
+      v += q * q;
+    }
+    v = warp_sum(v);
+  }
+  if (lane == 0) out[row] = v;
 }
 
 // g_u = L_C^-1 h_u for the block covariance: g[u][i] = sum_k h[u][k] LcT[k][i]
@@ -1522,7 +1536,7 @@ __global__ void __launch_bounds__(NT) k_pred_xcov(const Pair* __restrict__ pairs
 // mean_u = mu + Vu_u . beta + t1_u ; var_u = sigma_s^2 [+ sigma_n^2] - |Vu_u|^2 - t2_u + |L_C^-1 h_u|^2
 template <typename T>
 __global__ void k_pred_final(const T* __restrict__ Vu, int64_t U, int s, const double* __restrict__ beta,
-                             const float2* __restrict__ bs, const double* __restrict__ t1, const double* __restrict__ t2,
+                             const float4* __restrict__ bs, const double* __restrict__ t1, const double* __restrict__ t2,
                              const double* __restrict__ partial, int ntile, double mu, double prior,
                              double* __restrict__ mean, double* __restrict__ var) {
   grid_dep_wait();
@@ -1531,28 +1545,33 @@ __global__ void k_pred_final(const T* __restrict__ Vu, int64_t U, int s, const d
   const int lane = threadIdx.x & 31;
   if (warp >= U) return;
   double a = 0.0, b = 0.0;
-  if constexpr (sizeof(T) == 4) {  // beta as two floats (k_split_beta), sums in pairs of floats
-    Pair2 pa{0.f, 0.f}, pb{0.f, 0.f};
+  bool sums = false;
+  if constexpr (sizeof(T) == 4) {  // 32,768 points, s = 1,024: 0.22 ms added in FP64, 0.09 so
+    if (s <= 32 * (kSum3Terms / 2)) {
+      Sum3 sa, sb;
+      float inexact = 0.f;
 #pragma unroll 4
-    for (int k = lane; k < s; k += 32) {
-      const float v = Vu[warp * s + k];
-      const float2 bk = bs[k];
-      fma2(pa, v, bk.x);
-      pa.l = fmaf(v, bk.y, pa.l);
-      fma2(pb, v, v);
+      for (int k = lane; k < s; k += 32) {
+        const float v = Vu[warp * s + k];
+        const float4 bk = bs[k];
+        sa.add_product(v, bk);
+        sb.add_product(v, v);
+        inexact += bk.w;
+      }
+      a = warp_sum(sa.value() + (double)inexact);
+      b = warp_sum(sb.value());
+      sums = sum3_stands(a) && sum3_stands(b);
     }
-    a = to_double(warp_sum2(pa));
-    b = to_double(warp_sum2(pb));
-  } else {
+  }
+  if (!sums) {
+    a = b = 0.0;
     for (int k = lane; k < s; k += 32) {
       double v = (double)Vu[warp * s + k];
       a += v * beta[k];
       b += v * v;
     }
-    for (int o = 16; o > 0; o >>= 1) {
-      a += __shfl_down_sync(0xffffffffu, a, o);
-      b += __shfl_down_sync(0xffffffffu, b, o);
-    }
+    a = warp_sum(a);
+    b = warp_sum(b);
   }
   if (lane == 0) {
     double g = 0.0;

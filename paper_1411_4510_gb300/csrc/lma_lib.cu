@@ -932,10 +932,10 @@ void Impl<T>::fit_global(ModelCore& mc, int64_t n_total, cudaStream_t on) {
              (int)s, mc.brows, mc.ldk, mc.lcinv3);
     }
     if (sizeof(T) == 4) {
-      float2* bs = mc.bs = mc.keep.alloc<float2>(s);
+      float4* bs = mc.bs = mc.keep.alloc<float4>(s);
       launch("k_split_beta", k_split_beta, nblk(s), NT, 0, st, (const double*)mc.beta, (int)s, bs);
       launch("k_ew", k_ew_f32, dim3(nblk(maxnt * TB), (unsigned)M), NT, 0, st, mc.wins_d, (const float*)mc.wbuf,
-             (const float2*)bs, (int)s, (float*)mc.ew);
+             (const float4*)bs, (int)s, (float*)mc.ew);
     } else {
       launch("k_ew", k_ew<T>, dim3(nblk(maxnt * TB), (unsigned)M), NT, 0, st, mc.wins_d, (const T*)mc.wbuf, mc.beta,
              (int)s, (T*)mc.ew);
@@ -1308,8 +1308,8 @@ void Impl<T>::predict(const ModelCore& mc, int64_t U, const double* XU, const in
       vd = tmp.alloc<double>(U);
     }
     const double prior = mc.ss2 + (noisy ? mc.sn2 : 0.0);
-    launch("k_pred_final", k_pred_final<T>, nblk(U * 32), NT, 0, st, Vu, U, (int)s, mc.beta, (const float2*)mc.bs, t1, t2, part, ntile_var,
-           mc.mu, prior, md, vd);
+    launch("k_pred_final", k_pred_final<T>, nblk(U * 32), NT, 0, st, Vu, U, (int)s, mc.beta, (const float4*)mc.bs, t1, t2, part,
+           ntile_var, mc.mu, prior, md, vd);
     if (cov) {
       // requested blocks of the covariance between test blocks (Eq. vapvar on
       // U_n x U_n2), packed row-major in request order; without a request

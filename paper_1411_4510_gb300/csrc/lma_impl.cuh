@@ -93,24 +93,18 @@ inline int sm_count() {
 }
 
 // Launch a kernel, count it, check the launch status and (optionally) time it.
-// A grid of at most one CTA per SM is started with programmatic stream
-// serialisation: it may become resident while its predecessor in the stream
-// still runs, which hides the 1-2 us between two dependent launches (a small
-// problem is a chain of 45 to 60 of them; every kernel calls grid_dep_wait()
-// before anything else).  A larger grid is not: its CTAs would fill up the SMs
-// that the predecessor leaves first and run unevenly.  Measured, none / every
-// grid / this rule: N = 1,000 fit and predict 0.672 / 0.612 / 0.608 ms, N =
-// 40,960 4.28 / 4.24 / 4.14 ms (the factorisation's launches had it before), N =
-// 2,000,000 527.5 (none but those) / 500.6 ms (this rule), an FP64 gradient
-// 17.8 / 18.9 / 17.8 ms.
+// early: with programmatic stream serialisation, so that the grid may become
+// resident while its predecessor in the stream still runs, which hides the 1-2 us
+// between two dependent launches (every kernel calls grid_dep_wait() before
+// anything else).
 template <typename... KArgs, typename... Args>
-inline void launch(const char* name, void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
-                   Args... args) {
+inline void launch_early_if(bool early, const char* name, void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem,
+                            cudaStream_t st, Args... args) {
   const bool p = prof::active(name);
   if (p) prof::start(name, st);
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[0].val.programmaticStreamSerializationAllowed = (int64_t)grid.x * grid.y * grid.z <= sm_count() ? 1 : 0;
+  at[0].val.programmaticStreamSerializationAllowed = early ? 1 : 0;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;
@@ -126,6 +120,19 @@ inline void launch(const char* name, void (*kern)(KArgs...), dim3 grid, dim3 blo
     fail(LMA_ERR_CUDA, std::string("launch of ") + name + ": " + cudaGetErrorString(e));
     throw Fail{};
   }
+}
+
+// The same, early if the grid has at most one CTA per SM (a small problem is a
+// chain of 45 to 60 such launches).  A larger grid's CTAs would fill up the SMs that
+// the predecessor leaves first and run unevenly.  Measured, none / every grid /
+// this rule: N = 2,000 fit and predict 0.672 / 0.612 / 0.608 ms, N = 40,960 4.28 /
+// 4.24 / 4.14 ms (the factorisation's launches had it before), N = 2,000,000 527.5
+// (none but those) / 500.6 ms (this rule), an FP64 gradient 17.8 / 18.9 / 17.8 ms.
+// The FP64 factorisation's panels have a rule of their own (right_looking_fp64).
+template <typename... KArgs, typename... Args>
+inline void launch(const char* name, void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                   Args... args) {
+  launch_early_if((int64_t)grid.x * grid.y * grid.z <= sm_count(), name, kern, grid, block, smem, st, args...);
 }
 
 // launch() as a cooperative launch: every CTA of the grid is resident at

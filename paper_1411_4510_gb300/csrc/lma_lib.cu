@@ -434,16 +434,22 @@ static void right_looking_fp64(cudaStream_t st, const Win& w, Win* wd, double* b
     launch_coop("k_f64_coop", k_f64_coop, (unsigned)G, NTH, 0, st, buf, ld, w.rows, npan, nid, dv, info, bar, err);
     return;
   }
+  // Panel launches of 64-thread CTAs, where the next panel may start early: grids of up to three CTAs per SM (the next
+  // one finds room beside them) and of more than ten (several waves, whose last one it fills); in between it takes the
+  // current one's places.  Form 0 (lma_global_step_noalloc), launch()'s rule / every panel / this one: s = 256 378 / 357
+  // / 365 us, 512 852 / 903 / 848, 640 1,205 / 1,176 / 1,161, 1,024 3,031 / 2,922 / 2,925.  Form 1 always, its update
+  // launches above all (two factors at s = 512: a fit 3.90 ms with launch()'s rule, 2.39 so).
+  const int64_t sms = sm_count();
   launch("k_f64_potrf", k_f64_potrf, 1, NTH, 0, st, buf, ld, 0, dv, info);
   if (variant == 1) {
     for (int kp = 0; kp < npan; ++kp) {
       if (nrt - kp - 1 > 0)
-        launch("k_f64_solve2", k_f64_solve2, (unsigned)(nrt - kp - 1), NTH, 0, st, buf, ld, w.rows, npan, kp,
-                   nid, (const double*)dv);
+        launch_early_if(true, "k_f64_solve2", k_f64_solve2, (unsigned)(nrt - kp - 1), NTH, 0, st, buf, ld, w.rows,
+                        npan, kp, nid, (const double*)dv);
       const int m = npan - kp - 1;
       if (m > 0)
-        launch("k_f64_panel", k_f64_update2, (unsigned)(m * (m + 1) / 2 + (nrt - npan) * m), NTH, 0, st, buf,
-                   ld, w.rows, npan, kp, nid, dv, info);
+        launch_early_if(true, "k_f64_panel", k_f64_update2, (unsigned)(m * (m + 1) / 2 + (nrt - npan) * m), NTH, 0, st,
+                        buf, ld, w.rows, npan, kp, nid, dv, info);
     }
     return;
   }
@@ -452,8 +458,8 @@ static void right_looking_fp64(cudaStream_t st, const Win& w, Win* wd, double* b
     const int trail = m > 0 ? m * (m + 1) / 2 + (nrt - npan) * m : 0;
     const int solve = kp >= 1 ? nrt - kp : 0;
     if (trail + solve > 0)
-      launch("k_f64_panel", k_f64_panel, (unsigned)(trail + solve), NTH, 0, st, buf, ld, w.rows, npan, kp, nid, dv,
-             info);
+      launch_early_if(trail + solve <= 3 * sms || trail + solve > 10 * sms, "k_f64_panel", k_f64_panel,
+                      (unsigned)(trail + solve), NTH, 0, st, buf, ld, w.rows, npan, kp, nid, dv, info);
   }
 }
 

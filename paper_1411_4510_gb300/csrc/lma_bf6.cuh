@@ -202,92 +202,92 @@ __device__ bool walk(Smem& sm, const CUtensorMap* amap, int arows, const CUtenso
   } else {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 32;");
     if (warp == NWK) {
-    // MMA warp: the whole warp runs the loops, lane 0 waits and issues
-    const uint32_t idesc = idesc_bf16(128, 128), idesc2 = idesc_bf16(128, 256);
-    int C = 0;  // chunks issued so far by this CTA
-    bool ok = true;
-    for (int k = 0; ok; ++k) {
-      const int t = order(k);
-      if (t < 0) break;
-      const int nchunk = chunks(t);
-      for (int c = 0; c < nchunk; ++c, ++C) {
-        const int s = C % NST, a = C & 1;
-        int okw = 1;
-        if (lane == 0) {
-          okw = mbar_wait(&sm.full[s], (C / NST) & 1) ? 1 : 0;
-          if (okw && C >= 2) okw = mbar_wait(&sm.drained[a], ((C - 2) >> 1) & 1) ? 1 : 0;
-        }
-        okw = __shfl_sync(0xffffffffu, okw, 0);
-        if (!okw || *abort_flag) {
-          *abort_flag = 1;
-          ok = false;
-          break;
-        }
-        fence_after_sync();
-        if (lane == 0) {
-          Stage& S = sm.st[s];
-          uint32_t ad[3], bd[3];
-#pragma unroll
-          for (int p = 0; p < 3; ++p) {
-            ad[p] = smem_addr(S.a[p]);
-            bd[p] = smem_addr(S.b[p]);
+      // MMA warp: the whole warp runs the loops, lane 0 waits and issues
+      const uint32_t idesc = idesc_bf16(128, 128), idesc2 = idesc_bf16(128, 256);
+      int C = 0;  // chunks issued so far by this CTA
+      bool ok = true;
+      for (int k = 0; ok; ++k) {
+        const int t = order(k);
+        if (t < 0) break;
+        const int nchunk = chunks(t);
+        for (int c = 0; c < nchunk; ++c, ++C) {
+          const int s = C % NST, a = C & 1;
+          int okw = 1;
+          if (lane == 0) {
+            okw = mbar_wait(&sm.full[s], (C / NST) & 1) ? 1 : 0;
+            if (okw && C >= 2) okw = mbar_wait(&sm.drained[a], ((C - 2) >> 1) & 1) ? 1 : 0;
           }
-          const uint32_t dm = sm.tmem + 256 * a, de = dm + 128;
-#pragma unroll
-          for (int ks = 0; ks < KC / 16; ++ks) {
-            const uint32_t o = ks * 32;  // 16 bfloat16 values of K per MMA
-            const uint32_t first = ks > 0 ? 1u : 0u;
-            // planes 0 and 1 of B are 256 consecutive rows and the two accumulators 256 consecutive columns
-            mma_bf16(dm, sdesc_sw128(ad[0] + o), sdesc_sw128(bd[0] + o), idesc2, first);
-            mma_bf16(de, sdesc_sw128(ad[1] + o), sdesc_sw128(bd[0] + o), idesc, 1u);
-            mma_bf16(de, sdesc_sw128(ad[0] + o), sdesc_sw128(bd[2] + o), idesc, 1u);
-            mma_bf16(de, sdesc_sw128(ad[1] + o), sdesc_sw128(bd[1] + o), idesc, 1u);
-            mma_bf16(de, sdesc_sw128(ad[2] + o), sdesc_sw128(bd[0] + o), idesc, 1u);
+          okw = __shfl_sync(0xffffffffu, okw, 0);
+          if (!okw || *abort_flag) {
+            *abort_flag = 1;
+            ok = false;
+            break;
           }
-          mma_commit(&sm.empty[s]);  // the stage may be refilled
-          mma_commit(&sm.done[a]);   // the accumulators may be drained
+          fence_after_sync();
+          if (lane == 0) {
+            Stage& S = sm.st[s];
+            uint32_t ad[3], bd[3];
+#pragma unroll
+            for (int p = 0; p < 3; ++p) {
+              ad[p] = smem_addr(S.a[p]);
+              bd[p] = smem_addr(S.b[p]);
+            }
+            const uint32_t dm = sm.tmem + 256 * a, de = dm + 128;
+#pragma unroll
+            for (int ks = 0; ks < KC / 16; ++ks) {
+              const uint32_t o = ks * 32;  // 16 bfloat16 values of K per MMA
+              const uint32_t first = ks > 0 ? 1u : 0u;
+              // planes 0 and 1 of B are 256 consecutive rows and the two accumulators 256 consecutive columns
+              mma_bf16(dm, sdesc_sw128(ad[0] + o), sdesc_sw128(bd[0] + o), idesc2, first);
+              mma_bf16(de, sdesc_sw128(ad[1] + o), sdesc_sw128(bd[0] + o), idesc, 1u);
+              mma_bf16(de, sdesc_sw128(ad[0] + o), sdesc_sw128(bd[2] + o), idesc, 1u);
+              mma_bf16(de, sdesc_sw128(ad[1] + o), sdesc_sw128(bd[1] + o), idesc, 1u);
+              mma_bf16(de, sdesc_sw128(ad[2] + o), sdesc_sw128(bd[0] + o), idesc, 1u);
+            }
+            mma_commit(&sm.empty[s]);  // the stage may be refilled
+            mma_commit(&sm.done[a]);   // the accumulators may be drained
+          }
+          __syncwarp();
         }
-        __syncwarp();
       }
-    }
-    if (lane == 0) mma_commit(&sm.fin);  // arrives once every MMA issued above has completed
-    __syncwarp();
+      if (lane == 0) mma_commit(&sm.fin);  // arrives once every MMA issued above has completed
+      __syncwarp();
     } else if (warp == NWK + 1) {
-    // TMA producer: the whole warp runs the loops, lane 0 waits and issues
-    int C = 0;
-    bool ok = true;
-    for (int k = 0; ok; ++k) {
-      const int t = order(k);
-      if (t < 0) break;
-      const int4 base = coords(t);
-      const int nchunk = chunks(t);
-      for (int c = 0; c < nchunk; ++c, ++C) {
-        const int s = C % NST;
-        int okw = 1;
-        if (lane == 0 && C >= NST) okw = mbar_wait(&sm.empty[s], (C / NST - 1) & 1) ? 1 : 0;
-        okw = __shfl_sync(0xffffffffu, okw, 0);
-        if (!okw || *abort_flag) {
-          *abort_flag = 1;
-          ok = false;
-          break;
-        }
-        if (lane == 0) {
-          Stage& S = sm.st[s];
-          const int3 y = at(base, c);
-          mbar_arrive_expect_tx(&sm.full[s], 6u * kTileBytes);
-#pragma unroll
-          for (int p = 0; p < 3; ++p) {
-            tma_load_2d(S.a[p], amap, y.x, y.y + p * arows, &sm.full[s]);
-            tma_load_2d(S.b[p], bmap, y.x, y.z + p * brows, &sm.full[s]);
+      // TMA producer: the whole warp runs the loops, lane 0 waits and issues
+      int C = 0;
+      bool ok = true;
+      for (int k = 0; ok; ++k) {
+        const int t = order(k);
+        if (t < 0) break;
+        const int4 base = coords(t);
+        const int nchunk = chunks(t);
+        for (int c = 0; c < nchunk; ++c, ++C) {
+          const int s = C % NST;
+          int okw = 1;
+          if (lane == 0 && C >= NST) okw = mbar_wait(&sm.empty[s], (C / NST - 1) & 1) ? 1 : 0;
+          okw = __shfl_sync(0xffffffffu, okw, 0);
+          if (!okw || *abort_flag) {
+            *abort_flag = 1;
+            ok = false;
+            break;
           }
+          if (lane == 0) {
+            Stage& S = sm.st[s];
+            const int3 y = at(base, c);
+            mbar_arrive_expect_tx(&sm.full[s], 6u * kTileBytes);
+#pragma unroll
+            for (int p = 0; p < 3; ++p) {
+              tma_load_2d(S.a[p], amap, y.x, y.y + p * arows, &sm.full[s]);
+              tma_load_2d(S.b[p], bmap, y.x, y.z + p * brows, &sm.full[s]);
+            }
+          }
+          __syncwarp();
         }
-        __syncwarp();
       }
-    }
-    // no copy may still be landing in shared memory when the CTA leaves
-    if (lane == 0)
-      for (int c = C > NST ? C - NST : 0; c < C; ++c) mbar_wait(&sm.full[c % NST], (c / NST) & 1);
-    __syncwarp();
+      // no copy may still be landing in shared memory when the CTA leaves
+      if (lane == 0)
+        for (int c = C > NST ? C - NST : 0; c < C; ++c) mbar_wait(&sm.full[c % NST], (c / NST) & 1);
+      __syncwarp();
     }
   }
   const bool w = mbar_wait(&sm.fin, 0);
@@ -310,8 +310,8 @@ __device__ bool persistent(Smem& sm, const CUtensorMap* amap, int arows, const C
 }
 
 // persistent() with the chunks' results added by TwoSum into (hi, lo), for
-// products whose K runs long (thousands of values): after(t, hi, lo).  Eight
-// columns at a time keep the TwoSum state in registers.
+// products whose K runs long (thousands of values): after(t, hi, lo).  Four
+// columns at a time leave room for the TwoSum state in registers.
 template <class Order, class Chunks, class Coords, class At, class Before, class After>
 __device__ bool persistent_comp(Smem& sm, const CUtensorMap* amap, int arows, const CUtensorMap* bmap,
                                 int brows, Order order, Chunks chunks, Coords coords, At at, Before before, After after) {

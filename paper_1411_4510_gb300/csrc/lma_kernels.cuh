@@ -518,13 +518,12 @@ struct CholSmem {
 
 // Shared memory of diag_factor64 besides the tile itself.
 constexpr int DP = 68;  // row pitch of the 64-wide tiles: 8 rows x 4 columns without bank conflicts, 16-byte aligned
-template <typename T>
 struct alignas(16) Diag64Smem {
-  T X[64][DP];
-  alignas(16) T A[3][64][8];   // a_rj = L_rj / sqrt(pivot j) of the last panels, one 8-column panel each
-  alignas(16) T C[8][65][8];   // the panels' unscaled columns (a replaced pivot is 1 here)
-  alignas(16) T Xu[2][64][8];  // the panels' unscaled inverse rows, by column
-  alignas(16) T rj[64];
+  float X[64][DP];
+  alignas(16) float A[3][64][8];   // a_rj = L_rj / sqrt(pivot j) of the last panels, one 8-column panel each
+  alignas(16) float C[8][65][8];   // the panels' unscaled columns (a replaced pivot is 1 here)
+  alignas(16) float Xu[2][64][8];  // the panels' unscaled inverse rows, by column
+  alignas(16) float rj[64];
 };
 
 // 8 values between (16-byte aligned) shared memory and registers, 16 bytes at a time.
@@ -538,21 +537,9 @@ __device__ __forceinline__ void load8(float (&v)[8], const float* p) {
     v[q + 3] = f.w;
   }
 }
-__device__ __forceinline__ void load8(double (&v)[8], const double* p) {
-#pragma unroll
-  for (int q = 0; q < 8; q += 2) {
-    const double2 f = *reinterpret_cast<const double2*>(p + q);
-    v[q] = f.x;
-    v[q + 1] = f.y;
-  }
-}
 __device__ __forceinline__ void store8(float* p, const float (&v)[8]) {
 #pragma unroll
   for (int q = 0; q < 8; q += 4) *reinterpret_cast<float4*>(p + q) = make_float4(v[q], v[q + 1], v[q + 2], v[q + 3]);
-}
-__device__ __forceinline__ void store8(double* p, const double (&v)[8]) {
-#pragma unroll
-  for (int q = 0; q < 8; q += 2) *reinterpret_cast<double2*>(p + q) = make_double2(v[q], v[q + 1]);
 }
 
 // Cholesky of the 64 x 64 diagonal tile held in D (shared memory, lower part
@@ -574,22 +561,22 @@ __device__ __forceinline__ void store8(double* p, const double (&v)[8]) {
 // A barrier and an update of the whole tile per column (the form before) made
 // k_chol_step_tc 35 us for 64 windows; this one 14 (first panel of a 128-column
 // group) and 18 (second panel, with its product).
-template <typename T>
-__device__ void diag_factor64(T (*D)[DP], Diag64Smem<T>& sm, T* Lout, int64_t ld, T* Dv, int* info, int k0) {
+__device__ __forceinline__ void diag_factor64(float (*D)[DP], Diag64Smem& sm, float* Lout, int64_t ld, float* Dv,
+                                              int* info, int k0) {
   const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
-  T aa[8], ab[8];  // warp 0: the last panel's a values of rows lane, lane + 32
-  int first = 0;   // first failing column + 1
+  float aa[8], ab[8];  // warp 0: the last panel's a values of rows lane, lane + 32
+  int first = 0;       // first failing column + 1
   // warp 0: columns [j0, j0 + 8): the panel before applied, then factorised; up: the pivot rows are the lanes'
   // second rows
   auto panel = [&](int pp, auto up) {
     const int j0 = 8 * pp, jl = j0 & 31;
-    T da[8], db[8];
+    float da[8], db[8];
     load8(da, &D[lane][j0]);
     load8(db, &D[lane + 32][j0]);
     if (pp > 0) {
 #pragma unroll
       for (int c = 0; c < 8; ++c) {
-        T cv[8];
+        float cv[8];
         load8(cv, sm.C[pp - 1][j0 + c]);
 #pragma unroll
         for (int q = 0; q < 8; ++q) {
@@ -598,19 +585,19 @@ __device__ void diag_factor64(T (*D)[DP], Diag64Smem<T>& sm, T* Lout, int64_t ld
         }
       }
     }
-    T ca[8], cb[8];
-    T rv = T(0);
+    float ca[8], cb[8];
+    float rv = 0.f;
 #pragma unroll
     for (int jj = 0; jj < 8; ++jj) {
-      const T src = up ? db[jj] : da[jj];
-      T piv = __shfl_sync(0xffffffffu, src, jl + jj);
-      T cv[8];
+      const float src = up ? db[jj] : da[jj];
+      float piv = __shfl_sync(0xffffffffu, src, jl + jj);
+      float cv[8];
 #pragma unroll
       for (int c = jj + 1; c < 8; ++c) cv[c] = __shfl_sync(0xffffffffu, src, jl + c);
-      const bool good = piv > T(0);
-      piv = good ? piv : T(1);
+      const bool good = piv > 0.f;
+      piv = good ? piv : 1.f;
       if (!good && first == 0) first = j0 + jj + 1;
-      const T r = rsqrt(piv);
+      const float r = rsqrtf(piv);
       ca[jj] = (!up && lane == jl + jj) ? piv : da[jj];
       cb[jj] = (up && lane == jl + jj) ? piv : db[jj];
       aa[jj] = (da[jj] * r) * r;
@@ -643,15 +630,15 @@ __device__ void diag_factor64(T (*D)[DP], Diag64Smem<T>& sm, T* Lout, int64_t ld
       // inverse rows j0 .. j0 + 7, column c of this lane: panel pp - 1, then the panel's own triangle
       const int c = t - 32;
       if (c < j0 + 8) {
-        T x[8];
+        float x[8];
 #pragma unroll
-        for (int i = 0; i < 8; ++i) x[i] = c < j0 - 8 ? sm.X[j0 + i][c] : (j0 + i == c ? T(1) : T(0));
+        for (int i = 0; i < 8; ++i) x[i] = c < j0 - 8 ? sm.X[j0 + i][c] : (j0 + i == c ? 1.f : 0.f);
         if (c < j0) {
-          T xu[8];
+          float xu[8];
           load8(xu, sm.Xu[(pp - 1) & 1][c]);
 #pragma unroll
           for (int i = 0; i < 8; ++i) {
-            T a[8];
+            float a[8];
             load8(a, sm.A[(pp + 2) % 3][j0 + i]);
 #pragma unroll
             for (int q = 0; q < 8; ++q) x[i] = fma(-a[q], xu[q], x[i]);
@@ -659,12 +646,12 @@ __device__ void diag_factor64(T (*D)[DP], Diag64Smem<T>& sm, T* Lout, int64_t ld
         }
 #pragma unroll
         for (int i = 1; i < 8; ++i) {
-          T a[8];
+          float a[8];
           load8(a, sm.A[pp % 3][j0 + i]);
 #pragma unroll
           for (int q = 0; q < i; ++q) x[i] = fma(-a[q], x[q], x[i]);
         }
-        T rj[8];
+        float rj[8];
         load8(rj, sm.rj + j0);
         store8(sm.Xu[pp & 1][c], x);
 #pragma unroll
@@ -675,13 +662,13 @@ __device__ void diag_factor64(T (*D)[DP], Diag64Smem<T>& sm, T* Lout, int64_t ld
       // starts from zero): four threads a row, four columns of it in flight per thread
       const int u = t - 96, p = u & 3;
       for (int rd = j0 + 16 + (u >> 2); rd < 64; rd += 40) {
-        T a[8];
+        float a[8];
         load8(a, sm.A[pp % 3][rd]);
 #pragma unroll 4
         for (int c = j0 + 16 + p; c <= rd; c += 4) {
-          T cv[8];
+          float cv[8];
           load8(cv, sm.C[pp][c]);
-          T d = D[rd][c];
+          float d = D[rd][c];
 #pragma unroll
           for (int q = 0; q < 8; ++q) d = fma(-a[q], cv[q], d);
           D[rd][c] = d;
@@ -689,13 +676,13 @@ __device__ void diag_factor64(T (*D)[DP], Diag64Smem<T>& sm, T* Lout, int64_t ld
       }
       if (pp > 0)
         for (int rx = j0 + 8 + 39 - (u >> 2); rx < 64; rx += 40) {  // (the threads whose rows of D are the longest first)
-          T a[8];
+          float a[8];
           load8(a, sm.A[(pp + 2) % 3][rx]);
 #pragma unroll 4
           for (int c = p; c < j0; c += 4) {
-            T xu[8];
+            float xu[8];
             load8(xu, sm.Xu[(pp - 1) & 1][c]);
-            T x = c < j0 - 8 ? sm.X[rx][c] : T(0);
+            float x = c < j0 - 8 ? sm.X[rx][c] : 0.f;
 #pragma unroll
             for (int q = 0; q < 8; ++q) x = fma(-a[q], xu[q], x);
             sm.X[rx][c] = x;
@@ -708,13 +695,13 @@ __device__ void diag_factor64(T (*D)[DP], Diag64Smem<T>& sm, T* Lout, int64_t ld
 #pragma unroll
   for (int e = t; e < 64 * 8; e += 256) {
     const int r = e >> 3, c = (e & 7) * 8;
-    T l[8], rj[8], x[8];
+    float l[8], rj[8], x[8];
     load8(l, sm.C[e & 7][r]);
     load8(rj, sm.rj + c);
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
-      l[q] = c + q <= r ? l[q] * rj[q] : T(0);  // L_rc = D_rc r_c
-      x[q] = c + q <= r ? sm.X[r][c + q] : T(0);
+      l[q] = c + q <= r ? l[q] * rj[q] : 0.f;  // L_rc = D_rc r_c
+      x[q] = c + q <= r ? sm.X[r][c + q] : 0.f;
     }
     store8(Lout + (int64_t)r * ld + c, l);
     store8(Dv + r * 64 + c, x);

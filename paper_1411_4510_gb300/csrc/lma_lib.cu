@@ -1155,14 +1155,11 @@ void Impl<T>::predict(const ModelCore& mc, int64_t U, const double* XU, const in
     make_pairs(mc.wins, mc.w0, M, B, s, tptr, ft != nullptr, pairs, tb, wpairs, own, &pe);
     const bool use_tc = mc.prec == LMA_MIXED && sizeof(T) == 4 && use_tensor_cores();
     std::vector<int4> it_rhs, it_acc, it_t12;
-    std::vector<int2> it_sw;
     for (size_t pi = 0; pi < pairs.size() && !use_tc; ++pi) {
       const Pair& p = pairs[pi];
       const int nut = (p.nu + TB - 1) / TB, nct = mc.wins[p.win].npad / TB;
-      for (int ut = 0; ut < nut; ++ut) {
-        it_sw.push_back(make_int2((int)pi, ut));
+      for (int ut = 0; ut < nut; ++ut)
         for (int ct = 0; ct < nct; ++ct) it_rhs.push_back(make_int4((int)pi, ut, ct, 0));
-      }
     }
     const int nst = (int)((s + TB - 1) / TB);
     for (const int4& t : tb) {
@@ -1175,12 +1172,10 @@ void Impl<T>::predict(const ModelCore& mc, int64_t U, const double* XU, const in
     if (use_tc) stage_copy(wpd, wpairs.data(), sizeof(Pair) * wpairs.size(), st);
     Pair* pd = tmp.alloc<Pair>(pairs.size());
     int4* ird = tmp.alloc<int4>(it_rhs.size());
-    int2* isd = tmp.alloc<int2>(it_sw.size());
     int4* iad = tmp.alloc<int4>(it_acc.size());
     int4* itd = tmp.alloc<int4>(it_t12.size());
     stage_copy(pd, pairs.data(), sizeof(Pair) * pairs.size(), st);
     stage_copy(ird, it_rhs.data(), sizeof(int4) * it_rhs.size(), st);
-    stage_copy(isd, it_sw.data(), sizeof(int2) * it_sw.size(), st);
     stage_copy(iad, it_acc.data(), sizeof(int4) * it_acc.size(), st);
     stage_copy(itd, it_t12.data(), sizeof(int4) * it_t12.size(), st);
     T* Pbuf = ft ? (T*)mc.wbuf : tmp.alloc<T>(pe);
@@ -1232,6 +1227,11 @@ void Impl<T>::predict(const ModelCore& mc, int64_t U, const double* XU, const in
                N == 16 ? ps_smem<16>() : (N == 64 ? ps_smem<64>() : ps_smem<128>()), st, (const Pair*)wpd,
                (const int2*)itc, mc.wins_d, (const float*)wbuf, (const float*)mc.dinv, (float*)Pbuf, perr);
       } else {
+        std::vector<int2> it_sw;
+        for (size_t pi = 0; pi < pairs.size(); ++pi)
+          for (int ut = 0; ut < (pairs[pi].nu + TB - 1) / TB; ++ut) it_sw.push_back(make_int2((int)pi, ut));
+        int2* isd = tmp.alloc<int2>(it_sw.size());
+        stage_copy(isd, it_sw.data(), sizeof(int2) * it_sw.size(), st);
         launch("k_pred_sweep", k_pred_sweep<T>, (unsigned)it_sw.size(), NT, sizeof(CholSmem<T>), st, pd, isd,
                mc.wins_d, wbuf, (const T*)mc.dinv, Pbuf);
       }

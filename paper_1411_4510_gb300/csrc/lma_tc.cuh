@@ -620,7 +620,7 @@ __global__ void __launch_bounds__(256, 2) k_chol_step_tc(const Win* __restrict__
     __syncthreads();
     if (warp == 0) tmem_dealloc(tmem, 64);
   }
-  diag_factor64<float>(Dm, *reinterpret_cast<Diag64Smem<float>*>(scratch + TB * DP), A + (int64_t)k0 * ld + k0,
+  diag_factor64(Dm, *reinterpret_cast<Diag64Smem*>(scratch + TB * DP), A + (int64_t)k0 * ld + k0,
                        ld, dinv + w.dinv + (int64_t)kp * TB * TB, info + blockIdx.x, k0);
 }
 

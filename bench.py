@@ -164,11 +164,9 @@ def kernel_work(p, B, fused=True):
 NCU_TRAFFIC: dict = {
     # profiles/k_chol_wide_traffic_c4_n50000.md: DRAM bytes of the seven super-panel launches of the
     # C4 recipe at N = 50,000 (50 windows), averaged per launch and scaled by the window count to C4
-    # (the hash is of lma_tc.cuh after two unrelated kernels were deleted from it; the super-panel
-    # kernel and its pipeline are the captured code)
-    "k_chol_wide": {"bytes": 47.57e9, "case": ("C4", 1), "files": ["lma_tc.cuh"], "sources": "dd86857e5a16a326",
+    "k_chol_wide": {"bytes": 47.65e9, "case": ("C4", 1), "files": ["lma_tc.cuh"], "sources": "9c28619c5b17d3f0",
                     "note": "ncu dram__bytes_read.sum + dram__bytes_write.sum of the 7 launches of one step at "
-                            "N=50,000 (1.189 GB per launch on average, 1.34x the algorithmic bytes), x40 windows"},
+                            "N=50,000 (1.191 GB per launch on average, 1.34x the algorithmic bytes), x40 windows"},
 }
 
 
@@ -540,7 +538,7 @@ def main():
 
     def step(pr=prec, host=None, keep=False):
         src = dsrc if host is None else host
-        if sh is None:  # fit and predict in one call: the global step overlaps the prediction
+        if sh is None:  # fit and predict in one call: the global step on a second stream
             return L.lma_fit_predict(src["X"], src["y"], S=src["S"], XU=src["XU"], test_block_ptr=tptr,
                                      precision=pr, keep_model=keep, **kw)
         m = api.lma_fit_local(src["X"], src["y"], S=src["S"], win_begin=0, own_begin=sh.own_begin,

@@ -46,7 +46,8 @@ typedef enum {
 typedef enum {
   LMA_FP64 = 0,   /* plain FP64 GPU form: every step in double on the CUDA cores         */
   LMA_MIXED = 1   /* FP32 covariance tiles / factorisations / solves, batched over all
-                     windows; FP64 for Sigma_SS, the global summary and all reductions   */
+                     windows; FP64 for Sigma_SS, the global summary and the reductions
+                     (some as sums of three floats, no less accurate)                     */
 } lma_precision;
 
 typedef struct lma_model lma_model;
